@@ -49,6 +49,9 @@ struct tpfa_ctx {
   int loop_key_precond;
   int loop_key_vy, loop_key_stages;
   int loop_key_zc, loop_key_mode, loop_key_chunk, loop_key_sweep, loop_key_tile;
+  unsigned long long* comm;  // exchange buffers of the resident CG (allocated on first use)
+  size_t comm_words;
+  int resident_off;  // the device refused a cooperative launch of this size
   TmaMaps* maps;     // tensor maps of the TMA-staged sweep (host copy, built with the loop)
   TmaPlan tplan;
   cudaStream_t cap_stream;
@@ -143,6 +146,15 @@ bool use_tma_apply(const tpfa_ctx* c, bool b16) {
 }
 bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
+// Grids that fit on the chip run their inner solves in the resident kernel
+// (in either loop mode) unless a sweep is asked for.  An explicit z-run asks
+// for the tiling of a batch (so that results are bit-identical to it): the
+// bricks a batched instance gets.
+bool use_resident(const tpfa_ctx* c, ResPlan* p) {
+  return c->sweep_sel == 0 && c->vy == 4 && !c->resident_off &&
+         plan_resident(c->g, c->num_sms, c->zc > 0, p);
+}
+
 // The CG vectors of a solve: the separate arrays, or with the TMA-staged
 // sweep the interleaved records.
 CgVecs loop_vecs(const tpfa_ctx* c, bool b16) {
@@ -183,6 +195,29 @@ int ensure_partials(tpfa_ctx* c, size_t need) {
   return TPFA_OK;
 }
 
+int ensure_r64(tpfa_ctx* c) {
+  if (c->r64 == nullptr && cudaMalloc(&c->r64, (size_t)c->g.n * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    c->r64 = nullptr;
+    return TPFA_ENOMEM;
+  }
+  return TPFA_OK;
+}
+
+int ensure_comm(tpfa_ctx* c, size_t words) {
+  if (words <= c->comm_words) return TPFA_OK;
+  unsigned long long* m = nullptr;
+  if (cudaMalloc(&m, words * 8) != cudaSuccess) {
+    cudaGetLastError();
+    return TPFA_ENOMEM;
+  }
+  if (c->comm) cudaFree(c->comm);
+  c->comm = m;
+  c->comm_words = words;
+  CK(cudaMemset(m, 0, words * 8));
+  return TPFA_OK;
+}
+
 int ensure_vectors(tpfa_ctx* c) {
   if (c->vec != nullptr) return TPFA_OK;
   const size_t n = (size_t)c->g.n;
@@ -191,13 +226,6 @@ int ensure_vectors(tpfa_ctx* c) {
   if (cudaMalloc(&c->vec, 7 * pad * sizeof(float)) != cudaSuccess) {
     cudaGetLastError();
     c->vec = nullptr;
-    return TPFA_ENOMEM;
-  }
-  if (cudaMalloc(&c->r64, n * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(c->vec);
-    c->vec = nullptr;
-    c->r64 = nullptr;
     return TPFA_ENOMEM;
   }
   float* b = c->vec;
@@ -329,6 +357,11 @@ int read_state(tpfa_ctx* c, cudaStream_t s) {
 }  // namespace
 
 namespace tpfa {
+std::mutex& resident_mutex(int device) {
+  static std::mutex m[64];
+  return m[(unsigned)device % 64u];
+}
+
 int64_t ctx_cells(const tpfa_ctx* c) { return c ? c->g.n : 0; }
 void ctx_dims(const tpfa_ctx* c, int64_t* d3) {
   d3[0] = c->g.nx;
@@ -450,6 +483,7 @@ int tpfa_destroy(tpfa_ctx* c) {
   if (c->vec) cudaFree(c->vec);
   if (c->r64) cudaFree(c->r64);
   if (c->dinv) cudaFree(c->dinv);
+  if (c->comm) cudaFree(c->comm);
   if (c->vec4) cudaFree(c->vec4);
   delete c->maps;
   if (c->partials) cudaFree(c->partials);
@@ -703,7 +737,10 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
     return TPFA_EINVAL;
   if ((const void*)b == (const void*)x) return TPFA_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = ensure_vectors(c);
+  ResPlan rp;
+  const bool resident = use_resident(c, &rp);
+  rc = ensure_r64(c);
+  if (!rc) rc = resident ? ensure_comm(c, rp.words) : ensure_vectors(c);
   if (rc) return rc;
   if (b16 && c->precond && c->dinv == nullptr) {
     if (cudaMalloc(&c->dinv, n * sizeof(float)) != cudaSuccess) {
@@ -712,9 +749,11 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
       return TPFA_ENOMEM;
     }
   }
-  rc = ensure_loop(c, coef, b16);
-  if (rc) return rc;
-  const CgVecs vecs = loop_vecs(c, b16);
+  if (!resident) {
+    rc = ensure_loop(c, coef, b16);
+    if (rc) return rc;
+  }
+  const CgVecs vecs = resident ? CgVecs{} : loop_vecs(c, b16);
   CK(cudaMemsetAsync(c->counter, 0, 64, s));
   CK(cudaEventRecord(c->ev[0], s));
   if (b16 && c->precond) {
@@ -755,14 +794,42 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
       const double floor_rtol = b16 ? c->inner_rtol_bf16 : c->inner_rtol;
       if (rtol < floor_rtol) rtol = floor_rtol;
       if (rtol > 0.5) rtol = 0.5;
-      CK(launch_prepare(c->g, c->r64, vecs, c->st, rtol, (long long)(maxit - total_iters), s));
-      launches += 1;
       int inner_status = kRunning;
+      if (resident) {
+        // the stream is idle here (the state was just read), so nothing the
+        // launch waits for can need the lock
+        std::lock_guard<std::mutex> lock(resident_mutex(c->device));
+        CK(cudaEventRecord(c->ev[2], s));
+        const cudaError_t e =
+            launch_resident(make_res_prob(c->g, rp, coef, b16, c->dinv, c->r64, x, c->st, rtol,
+                                          (long long)(maxit - total_iters), c->comm),
+                            c->precond == 1, s);
+        if (e == cudaErrorCooperativeLaunchTooLarge && outer == 0) {
+          // fewer SMs than the device reports: this context keeps the sweeps
+          cudaGetLastError();
+          c->resident_off = 1;
+        } else {
+          CK(e);
+          CK(cudaEventRecord(c->ev[3], s));
+          rc = read_state(c, s);
+          if (rc) return rc;
+          float ms = 0.f;
+          CK(cudaEventElapsedTime(&ms, c->ev[2], c->ev[3]));
+          inner_ms += ms;
+          inner_status = hs->done;
+          if (inner_status == kGuard) CK(cudaMemsetAsync(c->comm, 0, c->comm_words * 8, s));
+        }
+      } else {
+        CK(launch_prepare(c->g, c->r64, vecs, c->st, rtol, (long long)(maxit - total_iters), s));
+        launches += 1;
+      }
+      if (resident && c->resident_off)
+        return solve_impl(c, coef, b16, coef64, b, x, tol, maxit, info, stream);
       // host-side bound on relaunches (the device guard normally ends the
       // loop first): chunks of sweeps in mode 1, finalize restarts in mode 0
       const long long max_relaunch = (maxit - total_iters) / (c->loop_mode == 1 ? c->chunk : 1) + 64;
       long long relaunch = 0;
-      for (;;) {
+      while (!resident) {
         if (++relaunch > max_relaunch) { inner_status = kGuard; break; }
         CK(cudaEventRecord(c->ev[2], s));
         CK(cudaGraphLaunch(c->loop_exec, s));
@@ -797,10 +864,13 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
       if (inner_status == kNonFinite) { status = TPFA_ENONFINITE; break; }
       if (inner_status == kBreakdown && hs->iter == 0) { status = TPFA_EBREAKDOWN; break; }
       // x += e / scale;  r64 = b - A x
-      CK(launch_correct(c->g, vecs, x, c->st, s));
+      if (!resident) {  // the resident kernel has added its correction
+        CK(launch_correct(c->g, vecs, x, c->st, s));
+        launches += 1;
+      }
       CK(launch_residual64(c->g, coef64, b, x, c->r64, nullptr, c->st, c->partials, c->counter,
                            c->elem_nblocks, s));
-      launches += 2;
+      launches += 1;
       ++outer;
       rc = read_state(c, s);
       if (rc) return rc;

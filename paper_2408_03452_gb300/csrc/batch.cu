@@ -10,6 +10,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -47,6 +48,49 @@ bool batch_tma(const tpfa_batch* b) {
   for (const Grid& g : b->g)
     if (!tma_sweep_ok(g, false, b->precond == 1)) return false;
   return true;
+}
+
+// The inner solves run in the resident kernel when every instance fits on the
+// chip, unless a sweep, a tile or z-runs are asked for.
+bool batch_resident(const tpfa_batch* b) {
+  if (b->sweep_sel != 0 || b->tma_tile != 0 || b->resident_off || b->ninst > kResMaxProb)
+    return false;
+  ResPlan p;
+  for (int i = 0; i < b->ninst; ++i)
+    if (b->zc_req[i] > 0 || !plan_resident(b->g[i], b->num_sms, true, &p)) return false;
+  return true;
+}
+
+// Plans and buffers of the resident solves, on first use.
+int setup_batch_resident(tpfa_batch* b) {
+  if (b->sched != nullptr) return TPFA_OK;
+  const int N = b->ninst;
+  b->rplan.resize(N);
+  b->comm_off.resize(N);
+  size_t words = 0, blocks = 0;
+  for (int i = 0; i < N; ++i) {
+    if (!plan_resident(b->g[i], b->num_sms, true, &b->rplan[i])) return TPFA_EINVAL;
+    b->comm_off[i] = words;
+    words += (b->rplan[i].words + 31) / 32 * 32;
+    blocks += (size_t)b->rplan[i].nblk;
+  }
+  b->comm_words = words;
+  if (cudaMalloc(&b->comm, words * 8) != cudaSuccess ||
+      cudaMalloc(&b->team, blocks * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&b->prob_dev, sizeof(ResProb) * N) != cudaSuccess ||
+      cudaMalloc(&b->sched, resident_batch_words(N, b->num_sms) * 8) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(b->comm);
+    cudaFree(b->team);
+    cudaFree(b->prob_dev);
+    b->comm = nullptr;
+    b->team = nullptr;
+    b->prob_dev = nullptr;
+    b->sched = nullptr;
+    return TPFA_ENOMEM;
+  }
+  BK(cudaMemset(b->comm, 0, words * 8));
+  return TPFA_OK;
 }
 
 // Automatic z-runs of the TMA-staged batched sweep: one common run length,
@@ -336,6 +380,10 @@ int tpfa_batch_destroy(tpfa_batch* b) {
   cudaFree(b->vec4);
   cudaFree(b->maps_dev);
   cudaFree(b->tinst_dev);
+  cudaFree(b->comm);
+  cudaFree(b->team);
+  cudaFree(b->prob_dev);
+  cudaFree(b->sched);
   cudaFree(b->r64);
   cudaFree(b->partials);
   cudaFree(b->counters);
@@ -457,10 +505,12 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       !dev_ok(rhs, n * 8, 8, b->device) || !dev_ok(x, n * 8, 8, b->device))
     return TPFA_EINVAL;
   if ((const void*)rhs == (const void*)x) return TPFA_EINVAL;
-  rc = ensure_batch_loop(b, coef);
+  const bool resident = batch_resident(b);
+  rc = resident ? setup_batch_resident(b) : ensure_batch_loop(b, coef);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const int N = b->ninst;
+  std::vector<ResProb> probs;
   const float4* cf = reinterpret_cast<const float4*>(coef);
   unsigned int* ecounter = b->counters + N;  // shared by the per-instance helper kernels
   CgState* hs = b->host_st;
@@ -513,11 +563,66 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       }
     }
     if (nact == 0) break;
+    if (resident) {
+      probs.clear();
+      std::vector<int> order;
+      for (int i = 0; i < N; ++i)
+        if (active[i]) order.push_back(i);
+      // largest teams first, among equals the longest solve of the last step
+      std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
+        const int np = b->rplan[p].nblk, nq = b->rplan[q].nblk;
+        return np != nq ? np > nq : iters[p] > iters[q];
+      });
+      std::vector<size_t> team0(N, 0);
+      for (int i = 1; i < N; ++i) team0[i] = team0[i - 1] + (size_t)b->rplan[i - 1].nblk;
+      for (int i : order) {
+        double rtol = 0.5 * tol / rel[i];
+        if (rtol < b->inner_rtol) rtol = b->inner_rtol;
+        if (rtol > 0.5) rtol = 0.5;
+        const int64_t o = b->off[i];
+        probs.push_back(make_res_prob(b->g[i], b->rplan[i], cf + o, false, nullptr, b->r64 + o,
+                                      x + o, b->st + i, rtol, (long long)(maxit - iters[i]),
+                                      b->comm + b->comm_off[i]));
+        probs.back().abort = reinterpret_cast<uint32_t*>(b->sched + 2);
+        probs.back().team = b->team + team0[i];
+      }
+      BK(cudaMemcpyAsync(b->prob_dev, probs.data(), sizeof(ResProb) * probs.size(),
+                         cudaMemcpyHostToDevice, s));
+      BK(cudaStreamSynchronize(s));
+      // the stream is idle: nothing the launch waits for can need the lock
+      std::lock_guard<std::mutex> lock(resident_mutex(b->device));
+      for (int i : order) hs[i].done = kGuard;  // what a team that never ran would leave
+      BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
+      BK(cudaEventRecord(b->ev[2], s));
+      const cudaError_t e = launch_resident_batch(b->prob_dev, (int)probs.size(), b->num_sms,
+                                                  b->precond == 1, b->sched, s);
+      if (e == cudaErrorCooperativeLaunchTooLarge && step == 0) {
+        // fewer SMs than the device reports: this batch keeps the sweeps
+        cudaGetLastError();
+        b->resident_off = 1;
+      } else {
+        BK(e);
+        BK(cudaEventRecord(b->ev[3], s));
+        ++launches;
+        rc = read_states();
+        if (rc) return rc;
+        float ms = 0.f;
+        BK(cudaEventElapsedTime(&ms, b->ev[2], b->ev[3]));
+        inner_ms += ms;
+        bool gave_up = false;
+        for (int i : order) gave_up = gave_up || hs[i].done == kGuard;
+        if (gave_up) BK(cudaMemsetAsync(b->comm, 0, b->comm_words * 8, s));
+      }
+    }
+    if (resident && b->resident_off)
+      return cg_solve_batch(b, coef, coef64, rhs, x, tol, maxit, infos, total, stream);
     // inactive instances: mark done so their sweep blocks return at once
-    for (int i = 0; i < N; ++i)
-      if (!active[i]) hs[i].done = kConvTrue;
-    BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
-    for (int i = 0; i < N; ++i) {
+    if (!resident) {
+      for (int i = 0; i < N; ++i)
+        if (!active[i]) hs[i].done = kConvTrue;
+      BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
+    }
+    for (int i = 0; i < N && !resident; ++i) {
       if (!active[i]) continue;
       double rtol = 0.5 * tol / rel[i];
       if (rtol < b->inner_rtol) rtol = b->inner_rtol;
@@ -527,7 +632,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       ++launches;
     }
     // while any instance runs: batched sweep + condition (guarded)
-    for (int relaunch = 0;; ++relaunch) {
+    for (int relaunch = 0; !resident; ++relaunch) {
       // the captured condition kernel stops the loop once the sweep counter
       // passes 0: start it at minus the guard limit
       const long long start = -(2 * mx + 64);
@@ -552,7 +657,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
         if (active[i] && hs[i].done == kRunning) ++again;
       if (again == 0 || relaunch > 64) break;
     }
-    {
+    if (!resident) {
       // every batched sweep launch (and the condition kernel after it) is
       // counted once in each instance's state: the most any instance saw
       long long sweeps = 0;
@@ -572,9 +677,12 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
     for (int i = 0; i < N; ++i) {
       if (!active[i]) continue;
       const int64_t o = b->off[i];
-      BK(launch_correct(b->g[i], vecs_at(b->v, o), x + o, b->st + i, s));
+      if (!resident) {  // the resident kernel has added its correction
+        BK(launch_correct(b->g[i], vecs_at(b->v, o), x + o, b->st + i, s));
+        ++launches;
+      }
       BK(residual(i));
-      launches += 2;
+      ++launches;
       ++outer[i];
     }
     rc = read_states();

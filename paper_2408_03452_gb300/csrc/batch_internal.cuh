@@ -41,6 +41,16 @@ struct tpfa_batch {
   CUtensorMap* maps_dev;
   int64_t tma_blocks;
   size_t partials_cap;  // doubles
+  // resident inner solves (instances that all fit on the chip): plans, exchange
+  // buffers of every instance (comm_off: first word), teams, table, scheduler
+  std::vector<tpfa::ResPlan> rplan;
+  std::vector<size_t> comm_off;
+  unsigned long long* comm;
+  size_t comm_words;
+  int* team;
+  tpfa::ResProb* prob_dev;
+  unsigned long long* sched;
+  int resident_off;  // the device refused the cooperative launch
   cudaGraphExec_t loop_exec;
   const void* loop_key_coef;
   int loop_key_precond;

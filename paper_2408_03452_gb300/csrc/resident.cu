@@ -1,0 +1,888 @@
+// Resident conjugate gradient: the whole inner solve of a grid that fits on
+// the chip, in one cooperative launch.
+//
+// A sweep of a small grid is bound by latency, not by memory: on 32^3 and 64^3
+// grids the sweep loop (one graph-node launch and a march through ten planes
+// per iteration) takes 20 us per iteration while the data of an iteration
+// would move in well under 1 us.  Here every block owns a brick of 32 x 16 x
+// CZ cells for the whole solve: the face transmissibilities, the diagonal and
+// the search direction live in shared memory, r, q = A p and x in registers,
+// and nothing but the brick faces and four partial sums crosses the chip per
+// iteration.  Capacity: num_sms bricks of 8,192 cells (1.2 M cells on GB300).
+//
+// One grid-wide exchange per iteration.  With the q of a neighbour's face cell
+// a block can form r and p of its halo cells itself (r_h -= alpha q_h, p_h =
+// z_h + beta p_h), so the neighbours' q and the four dot products are the only
+// things an iteration needs from other blocks, and both are complete at the
+// same point.  They travel as words that carry their own sequence number
+// ({value, epoch}, 8 bytes, single-copy atomic): a reader polls the data
+// itself, so an iteration costs one store-to-load round trip through L2 and
+// no fence, no counter and no second read.  Two buffers alternate: a block
+// overwrites a buffer only after it has seen every block's sums of the
+// iteration in between, which each block sends after it has read that buffer.
+//
+// Scalars.  FP64 runs at 1/64 of the FP32 rate on this chip, so beyond the
+// thread sums (compensated FP32, as in the sweeps) the dot products are added
+// as unevaluated pairs of floats (48 bits; Dekker 1971, Knuth TAOCP 4.2.2:
+// TwoSum, and products by FMA), in a fixed order, and every block forms the
+// same alpha and beta from them.  The operator is scaled by a power of two at
+// load time (largest D in [1, 2)), which changes no mantissa and keeps the
+// pairs inside the FP32 range; the solution is scaled back at the end.
+//
+// Measured (GB300, plain CG): see the rule in plan_resident.
+#include <math.h>
+
+#include "sweep_common.cuh"
+
+namespace tpfa {
+namespace {
+
+constexpr int kRW = 16;                 // warps per block = brick rows
+constexpr int kRT = kRW * 32;           // threads
+constexpr uint32_t kPollLimit = 1u << 23;  // polls of one wait before giving up
+
+// ---- unevaluated sums of two floats ----------------------------------------
+struct Dfl {
+  float h, l;
+};
+__device__ __forceinline__ Dfl df_fast(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Dfl df_add(Dfl a, Dfl b) {
+  const float s = __fadd_rn(a.h, b.h);
+  const float v = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
+  return df_fast(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ bool df_le(Dfl a, Dfl b) {
+  return a.h < b.h || (a.h == b.h && a.l <= b.l);
+}
+// the same without the final normalisation: for trees of a few levels, where
+// the correction stays small; only one addition is on the critical path
+__device__ __forceinline__ Dfl df_acc(Dfl a, Dfl b) {
+  const float s = __fadd_rn(a.h, b.h);
+  const float v = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
+  return {s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ Dfl df_mulf(Dfl a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return df_fast(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+// a / b to an ulp: a quotient from the approximate reciprocal and one residual
+// correction
+__device__ __forceinline__ float quot(float a, float b) {
+  const float y = __fdividef(1.f, b);
+  const float q = __fmul_rn(a, y);
+  return __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
+}
+__device__ __forceinline__ Dfl df_xor(Dfl a, int m) {
+  return {__shfl_xor_sync(kFull, a.h, m), __shfl_xor_sync(kFull, a.l, m)};
+}
+
+// ---- sequence-numbered words -------------------------------------------------
+__device__ __forceinline__ uint2 ll_load(const uint2* p) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return make_uint2((uint32_t)w, (uint32_t)(w >> 32));
+}
+__device__ __forceinline__ void ll_store(uint2* p, float v, uint32_t epoch) {
+  const unsigned long long w = (unsigned long long)__float_as_uint(v) | ((unsigned long long)epoch << 32);
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+
+// ---- layout ------------------------------------------------------------------
+template <int CZ>
+struct ResLayout {
+  static constexpr int kTx = 0;                                   // [CZ][W][33], column 0: x - 1
+  static constexpr int kTy = kTx + CZ * kRW * 33;                 // [CZ][W + 1][32], row 0: y - 1
+  static constexpr int kTz = kTy + CZ * (kRW + 1) * 32;           // [CZ][W][32]
+  static constexpr int kD = kTz + CZ * kRW * 32;
+  static constexpr int kP = kD + CZ * kRW * 32;                   // [CZ][W + 2][34]
+  static constexpr int kM = kP + CZ * (kRW + 2) * 34;             // Jacobi: M^-1 [CZ][W][32]
+  static constexpr int floats(bool jac) { return kM + (jac ? CZ * kRW * 32 : 0); }
+  // face words of a block: x lo, x hi [W][CZ], y lo, y hi [CZ][32], z lo, z hi [W][32]
+  static constexpr int kFx = CZ * kRW, kFy = CZ * 32, kFz = kRW * 32;
+  static constexpr int kFaces = 2 * (kFx + kFy + kFz);
+};
+
+// what every thread needs from the scalars of an iteration
+struct ResNext {
+  float alpha, beta;
+  int done;
+};
+
+struct ResShared {
+  float2 a[kRW][4], b[kRW][4];  // sums per warp: of the block, of all blocks
+  float mx[kRW];
+  ResNext next;
+};
+
+// the block's sums of four values, sent to every block and added up in a fixed
+// order; the neighbours' face words arrive in the same wait
+template <int CZ>
+struct ResComm {
+  uint2* part;
+  const uint2* face;
+  uint32_t* abort;
+  int nblk, blk;
+  int hoff[5];  // face words this thread reads (index in one buffer), -1: none
+  size_t face_buf;
+
+  // warp-wide transposing sum of four pairs: lane l ends with value (l >> 3)
+  __device__ __forceinline__ static Dfl warp4(const Dfl (&v)[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool u = lane & 16;
+    Dfl a = u ? v[2] : v[0], b = u ? v[3] : v[1];
+    const Dfl sa = df_xor(u ? v[0] : v[2], 16), sb = df_xor(u ? v[1] : v[3], 16);
+    a = df_acc(a, sa);
+    b = df_acc(b, sb);
+    const bool w = lane & 8;
+    Dfl c = w ? b : a;
+    c = df_acc(c, df_xor(w ? a : b, 8));
+    c = df_acc(c, df_xor(c, 4));
+    c = df_acc(c, df_xor(c, 2));
+    return df_acc(c, df_xor(c, 1));
+  }
+  // sum over the block's warps: s[warp][value]; every lane gets value (lane & 3)
+  __device__ __forceinline__ static Dfl warps16(const float2 (*s)[4]) {
+    const int lane = threadIdx.x & 31, v = lane & 3, w = lane >> 2;
+    const float2 a = s[w][v], b = s[w + 8][v];
+    Dfl t = df_acc({a.x, a.y}, {b.x, b.y});
+    t = df_acc(t, df_xor(t, 4));
+    t = df_acc(t, df_xor(t, 8));
+    t = df_acc(t, df_xor(t, 16));
+    return df_fast(t.h, t.l);
+  }
+
+  // Sends this block's sums and waits for every block's and for the
+  // neighbours' face words.  The totals are there in warp 0 only.  Returns
+  // false when the wait ran out (or another block gave up).
+  __device__ __forceinline__ bool exchange(const Dfl (&mine)[4], uint32_t epoch, Dfl (&tot)[4],
+                                           float (&qh)[5], ResShared& sh) {
+    auto& sA = sh.a;
+    auto& sB = sh.b;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Dfl w = warp4(mine);
+    if ((lane & 7) == 0) sA[warp][lane >> 3] = make_float2(w.h, w.l);
+    __syncthreads();
+    const uint32_t par = epoch & 1u;
+    uint2* pb = part + (size_t)par * nblk * 8;
+    const uint2* fb = face + par * face_buf;
+    // a first look at the neighbours' words: they were sent before the
+    // reduction, so they are there as a rule.  With short bricks it is in flight
+    // while warp 0 sends the sums (64^3: 2.89 -> 2.66 us per iteration); with
+    // tall ones the loads would only hold up those (128x128x64: 5.3 against 5.9)
+    unsigned need = 0u;
+    uint2 f[5];
+    auto look = [&]() {
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        if (hoff[j] >= 0) {
+          need |= 1u << j;
+          f[j] = ll_load(fb + hoff[j]);
+        }
+    };
+    if (CZ <= 8) look();
+    if (warp == 0) {
+      const Dfl t = warps16(sA);
+      if (lane < 4) {
+        ll_store(pb + ((size_t)blk * 4 + lane) * 2, t.h, epoch);
+        ll_store(pb + ((size_t)blk * 4 + lane) * 2 + 1, t.l, epoch);
+      }
+    }
+    if (CZ > 8) look();
+    bool ok = true;
+    uint32_t polls = 0;
+    auto give_up = [&]() -> bool {
+      if ((++polls & 1023u) != 0u) return false;
+      return polls >= kPollLimit || *(volatile uint32_t*)abort != 0u;
+    };
+    while (need != 0u) {
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        if (((need >> j) & 1u) && f[j].y == epoch) {
+          qh[j] = __uint_as_float(f[j].x);
+          need &= ~(1u << j);
+        }
+      if (need != 0u && give_up()) {
+        ok = false;
+        break;
+      }
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        if ((need >> j) & 1u) f[j] = ll_load(fb + hoff[j]);
+    }
+    // the sums of every block: item = 4 block + value, in order
+    Dfl sum = {0.f, 0.f};
+    for (int item = tid; ok && item < 4 * nblk;) {
+      const uint2 a = ll_load(pb + (size_t)item * 2), b = ll_load(pb + (size_t)item * 2 + 1);
+      if (a.y == epoch && b.y == epoch) {
+        sum = df_acc(sum, {__uint_as_float(a.x), __uint_as_float(b.x)});
+        item += kRT;
+      } else if (give_up()) {
+        ok = false;
+      }
+    }
+    sum = df_acc(sum, df_xor(sum, 4));
+    sum = df_acc(sum, df_xor(sum, 8));
+    sum = df_acc(sum, df_xor(sum, 16));
+    if (lane < 4) sB[warp][lane] = make_float2(sum.h, sum.l);
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) *(volatile uint32_t*)abort = 1u;
+      return false;
+    }
+    if (warp == 0) {
+      const Dfl t = warps16(sB);
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        tot[v] = {__shfl_sync(kFull, t.h, v), __shfl_sync(kFull, t.l, v)};
+    }
+    return true;
+  }
+};
+
+// One inner solve, run by the blocks blk = 0 .. a.nblk - 1 of its brick grid.
+template <int CZ, bool JAC>
+__device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float* sm,
+                                               ResShared& sh) {
+  using LY = ResLayout<CZ>;
+  float* sTx = sm + LY::kTx;
+  float* sTy = sm + LY::kTy;
+  float* sTz = sm + LY::kTz;
+  float* sD = sm + LY::kD;
+  float* sP = sm + LY::kP;
+  float* sM = sm + LY::kM;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int bx = blk % a.nbx, by = (blk / a.nbx) % a.nby, bz = blk / (a.nbx * a.nby);
+  const Grid g = a.g;
+  const int64_t gx = 32 * bx + lane, gy = kRW * by + warp, Z0 = (int64_t)CZ * bz;
+  const bool inxy = gx < g.nx && gy < g.ny;
+  const int64_t c0 = gx + g.nx * gy;  // in-plane cell
+  CgState* st = a.st;
+  const double scale = st->rr64 > 0.0 ? 1.0 / sqrt(st->rr64) : 1.0;
+
+  // record of cell (x, y, z) as (Tx, Ty, Tz, D); zeros outside the grid
+  const float4* c32 = static_cast<const float4*>(a.coef);
+  const uint2* c16 = static_cast<const uint2*>(a.coef);
+  auto rec = [&](int64_t x, int64_t y, int64_t z) -> float4 {
+    if (x < 0 || y < 0 || z < 0 || x >= g.nx || y >= g.ny || z >= g.nz)
+      return make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t c = x + g.nx * y + g.plane * z;
+    if (!a.b16) return __ldg(c32 + c);
+    const uint2 u = __ldg(c16 + c);
+    return make_float4(bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y));
+  };
+
+  // ---- load the brick -------------------------------------------------------
+  float dmax = 0.f;
+  float tzlo = 0.f;  // Tz of the plane below the brick
+  if (inxy) tzlo = rec(gx, gy, Z0 - 1).z;
+  float tzm = tzlo;
+#pragma unroll
+  for (int k = 0; k < CZ; ++k) {
+    const int64_t z = Z0 + k;
+    float4 cf = rec(gx, gy, z);
+    const float txl = lane == 0 ? rec(gx - 1, gy, z).x : 0.f;
+    const float tyl = warp == 0 ? rec(gx, gy - 1, z).y : 0.f;
+    if (a.b16) {
+      const float txm = rec(gx - 1, gy, z).x, tym = rec(gx, gy - 1, z).y;
+      if (inxy && z < g.nz) cf.w = (((((txm + cf.x) + tym) + cf.y) + tzm) + cf.z) + cf.w;
+    }
+    tzm = cf.z;
+    sTx[(k * kRW + warp) * 33 + lane + 1] = cf.x;
+    if (lane == 0) sTx[(k * kRW + warp) * 33] = txl;
+    sTy[(k * (kRW + 1) + warp + 1) * 32 + lane] = cf.y;
+    if (warp == 0) sTy[k * (kRW + 1) * 32 + lane] = tyl;
+    sTz[(k * kRW + warp) * 32 + lane] = cf.z;
+    sD[(k * kRW + warp) * 32 + lane] = cf.w;
+    if (JAC)
+      sM[(k * kRW + warp) * 32 + lane] =
+          (inxy && z < g.nz) ? (a.b16 ? a.dinv[c0 + g.plane * z] : jac_inv(cf.w)) : 0.f;
+    dmax = fmaxf(dmax, cf.w);
+  }
+  for (int i = tid; i < CZ * (kRW + 2) * 34; i += kRT) sP[i] = 0.f;
+
+  ResComm<CZ> cm;
+  cm.part = a.part;
+  cm.face = a.face;
+  cm.abort = a.abort;
+  cm.nblk = a.nblk;
+  cm.blk = blk;
+  cm.face_buf = (size_t)a.nblk * LY::kFaces;
+  // halo cells of this thread: below, above, y - 1 and y + 16 of plane `warp`,
+  // and one x-halo cell; their r, M^-1 and (z) p
+  float rh[5], mh[5], pz[2] = {0.f, 0.f}, qh[5];
+  const int xs = tid / LY::kFx, xi = tid % LY::kFx;  // x-halo: side, index w CZ + k
+  int pslot[3];                                      // sP index of halo cells 2, 3, 4
+  {
+    const int nb[5] = {bz > 0 ? blk - a.nbx * a.nby : -1, bz + 1 < a.nbz ? blk + a.nbx * a.nby : -1,
+                       (warp < CZ && by > 0) ? blk - a.nbx : -1,
+                       (warp < CZ && by + 1 < a.nby) ? blk + a.nbx : -1,
+                       xs == 0 ? (bx > 0 ? blk - 1 : -1)
+                               : (xs == 1 && bx + 1 < a.nbx ? blk + 1 : -1)};
+    const int w[5] = {2 * (LY::kFx + LY::kFy) + LY::kFz + tid, 2 * (LY::kFx + LY::kFy) + tid,
+                      2 * LY::kFx + LY::kFy + tid, 2 * LY::kFx + tid,
+                      xs == 0 ? LY::kFx + xi : xi};
+    const int xk = xi % CZ, xw = xi / CZ;
+    pslot[0] = warp * (kRW + 2) * 34 + lane + 1;
+    pslot[1] = (warp * (kRW + 2) + kRW + 1) * 34 + lane + 1;
+    pslot[2] = (xk * (kRW + 2) + xw + 1) * 34 + (xs == 0 ? 0 : 33);
+    const int64_t hx[5] = {gx, gx, gx, gx, 32 * (int64_t)bx + (xs == 0 ? -1 : 32)};
+    const int64_t hy[5] = {gy, gy, kRW * (int64_t)by - 1, kRW * (int64_t)by + kRW,
+                           kRW * (int64_t)by + xw};
+    const int64_t hz[5] = {Z0 - 1, Z0 + CZ, Z0 + warp, Z0 + warp, Z0 + xk};
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      cm.hoff[j] = nb[j] < 0 ? -1 : nb[j] * LY::kFaces + w[j];
+      rh[j] = 0.f;
+      mh[j] = 0.f;
+      qh[j] = 0.f;
+      if (nb[j] >= 0 && hx[j] < g.nx && hy[j] < g.ny && hz[j] < g.nz) {
+        const int64_t c = hx[j] + g.nx * hy[j] + g.plane * hz[j];
+        rh[j] = (float)(scale * a.r64[c]);
+        if (JAC) mh[j] = a.b16 ? a.dinv[c] : jac_inv(__ldg(c32 + c).w);
+      }
+    }
+  }
+
+  float r[CZ], q[CZ], x[CZ];
+#pragma unroll
+  for (int k = 0; k < CZ; ++k) {
+    r[k] = (inxy && Z0 + k < g.nz) ? (float)(scale * a.r64[c0 + g.plane * (Z0 + k)]) : 0.f;
+    q[k] = 0.f;
+    x[k] = 0.f;
+  }
+
+  // ---- power-of-two scale of the operator: the largest D of the grid ----------
+  uint32_t epoch = *(volatile uint32_t*)a.ctl;
+  bool fault = false;
+  float tscale = 1.f;
+  {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, o));
+    auto& sMax = sh.mx;
+    if (lane == 0) sMax[warp] = dmax;
+    __syncthreads();
+    for (int w = 0; w < kRW; ++w) dmax = fmaxf(dmax, sMax[w]);
+    ++epoch;
+    uint2* pb = a.part + (size_t)(epoch & 1u) * a.nblk * 8;
+    if (tid == 0) ll_store(pb + (size_t)blk * 8, dmax, epoch);
+    uint32_t polls = 0;
+    for (int i = tid; i < a.nblk && !fault; i += kRT) {
+      for (;;) {
+        const uint2 v = ll_load(pb + (size_t)i * 8);
+        if (v.y == epoch) {
+          dmax = fmaxf(dmax, __uint_as_float(v.x));
+          break;
+        }
+        if ((++polls & 1023u) == 0u &&
+            (polls >= kPollLimit || *(volatile uint32_t*)a.abort != 0u)) {
+          fault = true;
+          break;
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, o));
+    if (lane == 0) sMax[warp] = dmax;
+    fault = __syncthreads_or(fault);
+    for (int w = 0; w < kRW; ++w) dmax = fmaxf(dmax, sMax[w]);
+    if (dmax > 0.f && isfinite(dmax)) {
+      int e = ilogbf(dmax);
+      e = e > 120 ? 120 : (e < -120 ? -120 : e);
+      tscale = exp2f((float)-e);
+    }
+  }
+  const float mscale = 1.f / tscale;  // exact: a power of two
+  tzlo *= tscale;
+#pragma unroll
+  for (int k = 0; k < CZ; ++k) {
+    sTx[(k * kRW + warp) * 33 + lane + 1] *= tscale;
+    if (lane == 0) sTx[(k * kRW + warp) * 33] *= tscale;
+    sTy[(k * (kRW + 1) + warp + 1) * 32 + lane] *= tscale;
+    if (warp == 0) sTy[k * (kRW + 1) * 32 + lane] *= tscale;
+    sTz[(k * kRW + warp) * 32 + lane] *= tscale;
+    sD[(k * kRW + warp) * 32 + lane] *= tscale;
+    if (JAC) sM[(k * kRW + warp) * 32 + lane] *= mscale;
+  }
+  if (JAC)
+#pragma unroll
+    for (int j = 0; j < 5; ++j) mh[j] *= mscale;
+
+  // ---- iterations -------------------------------------------------------------
+  const float rtol2h = (float)a.rtol2, rtol2l = (float)(a.rtol2 - (double)rtol2h);
+  float alpha = 0.f, beta = 0.f;
+  Dfl rho = {0.f, 0.f}, rho0 = {0.f, 0.f}, thresh = {0.f, 0.f};
+  long long iter = 0, sweeps = 0;  // (warp 0)
+  const long long maxit = a.maxit, guard = 2 * maxit + 64;
+  int done = kRunning;
+  ResNext& sNext = sh.next;
+  uint2* fmine = a.face + (size_t)blk * LY::kFaces;
+  const bool fy0 = warp == 0 && by > 0, fy1 = warp == kRW - 1 && by + 1 < a.nby;
+
+  // r -= alpha q, x += alpha p, p = z + beta p (with `dir`), on the own and the
+  // halo cells; returns the sums of r'z
+  auto step = [&](bool dir, Acc& s0) {
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      if (cm.hoff[j] < 0) continue;
+      rh[j] = fmaf(-alpha, qh[j], rh[j]);
+      if (!dir) continue;
+      const float z = JAC ? rh[j] * mh[j] : rh[j];
+      if (j < 2) {
+        pz[j] = fmaf(beta, pz[j], z);
+      } else {
+        float* ps = sP + pslot[j - 2];
+        *ps = fmaf(beta, *ps, z);
+      }
+    }
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < CZ; ++k) {
+      float* ps = sP + (k * (kRW + 2) + warp + 1) * 34 + lane + 1;
+      const float p0 = *ps;
+      x[k] = fmaf(alpha, p0, x[k]);
+      r[k] = fmaf(-alpha, q[k], r[k]);
+      const float z = JAC ? r[k] * sM[(k * kRW + warp) * 32 + lane] : r[k];
+      if (dir) *ps = fmaf(beta, p0, z);
+      s = fmaf(r[k], z, s);
+      if ((k & 3) == 3 || k == CZ - 1) {
+        kadd(s0, s);
+        s = 0.f;
+      }
+    }
+  };
+
+  while (!fault) {
+    Acc acc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    step(true, acc[0]);
+    __syncthreads();
+    ++epoch;
+    uint2* fo = fmine + (epoch & 1u) * cm.face_buf;
+    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    float tz0 = tzlo, pm = pz[0];
+    float pc = sP[(warp + 1) * 34 + lane + 1];
+#pragma unroll
+    for (int k = 0; k < CZ; ++k) {
+      const float* ps = sP + (k * (kRW + 2) + warp + 1) * 34 + lane + 1;
+      const float pp = k + 1 < CZ ? ps[(kRW + 2) * 34] : pz[1];
+      const float* tx = sTx + (k * kRW + warp) * 33 + lane;
+      const float* ty = sTy + (k * (kRW + 1) + warp) * 32 + lane;
+      const int i = (k * kRW + warp) * 32 + lane;
+      const float4 cf = make_float4(tx[1], ty[32], sTz[i], sD[i]);
+      const float v = stencil7(cf, tx[0], ty[0], tz0, pc, ps[1], ps[-1], ps[34], ps[-34], pp, pm);
+      q[k] = v;
+      float z = r[k], mq = v;
+      if (JAC) {
+        const float m = sM[i];
+        z *= m;
+        mq *= m;
+      }
+      s1 = fmaf(pc, v, s1);
+      s2 = fmaf(z, v, s2);
+      s3 = fmaf(v, mq, s3);
+      if ((k & 3) == 3 || k == CZ - 1) {
+        kadd(acc[1], s1);
+        kadd(acc[2], s2);
+        kadd(acc[3], s3);
+        s1 = s2 = s3 = 0.f;
+      }
+      tz0 = cf.z;
+      pm = pc;
+      pc = pp;
+    }
+    // the neighbours' words, once all of q is there: a store between the planes
+    // would keep the loads of the next plane behind it (320 instead of 100
+    // cycles per plane)
+    if (bz > 0) ll_store(fo + 2 * (LY::kFx + LY::kFy) + tid, q[0], epoch);
+    if (bz + 1 < a.nbz) ll_store(fo + 2 * (LY::kFx + LY::kFy) + LY::kFz + tid, q[CZ - 1], epoch);
+    if (fy0 || fy1) {
+      uint2* f = fo + 2 * LY::kFx + (fy0 ? 0 : LY::kFy) + lane;
+#pragma unroll
+      for (int k = 0; k < CZ; ++k) ll_store(f + k * 32, q[k], epoch);
+    }
+    if (bx > 0 || bx + 1 < a.nbx) {
+      // lanes 0..15 take q[lane] of lane 0, lanes 16..31 q[lane - 16] of lane
+      // 31: one store per warp instead of one per plane
+      float v = 0.f;
+#pragma unroll
+      for (int k = 0; k < CZ; ++k) {
+        const float t = __shfl_sync(kFull, q[k], lane < 16 ? 0 : 31);
+        if ((lane & 15) == k) v = t;
+      }
+      if ((lane & 15) < CZ && (lane < 16 ? bx > 0 : bx + 1 < a.nbx))
+        ll_store(fo + (lane < 16 ? 0 : LY::kFx) + warp * CZ + (lane & 15), v, epoch);
+    }
+    Dfl mine[4], tot[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) mine[v] = df_fast(acc[v].s, -acc[v].c);
+    if (!cm.exchange(mine, epoch, tot, qh, sh)) {
+      fault = true;
+      break;
+    }
+    // alpha, beta and the stop test (as cg_finish), formed by warp 0 alone: in
+    // all 16 warps the same chain takes twice as long
+    if (warp == 0) {
+      rho = tot[0];
+      if (iter == 0) {
+        rho0 = rho;
+        thresh = df_add(df_mulf(rho0, rtol2h), df_mulf(rho0, rtol2l));
+      }
+      // alpha is the FP32 step the vectors take, so that rho - 2 alpha r'q +
+      // alpha^2 q'q is the norm of the residual it leaves
+      const float al = quot(rho.h, tot[1].h);
+      const Dfl u = df_mulf(tot[3], al);
+      const Dfl v = df_mulf(df_add({2.f * tot[2].h, 2.f * tot[2].l}, {-u.h, -u.l}), al);
+      Dfl rn = df_add(rho, {-v.h, -v.l});
+      if (rn.h < 0.f) rn = {0.f, 0.f};
+      alpha = al;
+      beta = quot(rn.h, rho.h);
+      // 0 unless one of the sums is infinite or NaN
+      const float bad = fmaf(tot[0].h, 0.f, fmaf(tot[1].h, 0.f, fmaf(tot[2].h, 0.f, tot[3].h * 0.f)));
+      const bool stay = bad == 0.f && tot[1].h > 0.f && !df_le(rho, thresh);
+      ++iter;
+      if (!stay || df_le(rn, thresh) || iter >= maxit || ++sweeps > guard) {
+        done = stay ? (df_le(rn, thresh) ? kConvEst : iter >= maxit ? kMaxit : kGuard)
+                    : (bad != 0.f ? kNonFinite : df_le(rho, thresh) ? kConvTrue : kBreakdown);
+        if (!stay) {
+          alpha = 0.f;
+          --iter;
+        }
+      }
+      if (lane == 0) sNext = {alpha, beta, done};
+    }
+    __syncthreads();
+    alpha = sNext.alpha;
+    beta = sNext.beta;
+    done = sNext.done;
+    if (done == kRunning) continue;
+    if (done != kConvEst && done != kMaxit) break;
+    // the last step, and the true r'r (r' M^-1 r) of the residual it leaves
+    Acc s0 = {0.f, 0.f};
+    step(false, s0);
+    ++epoch;
+    // the face words of this exchange are not sent: nothing reads them
+    int keep[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      keep[j] = cm.hoff[j];
+      cm.hoff[j] = -1;
+      mine[j < 4 ? j : 0] = {0.f, 0.f};
+    }
+    mine[0] = df_fast(s0.s, -s0.c);
+    const bool ok = cm.exchange(mine, epoch, tot, qh, sh);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) cm.hoff[j] = keep[j];
+    if (!ok) {
+      fault = true;
+      break;
+    }
+    if (warp == 0) {
+      const Dfl prev = rho;
+      rho = tot[0];
+      if (done == kConvEst && !df_le(rho, thresh) && iter < a.maxit && isfinite(rho.h) &&
+          prev.h > 0.f) {
+        // the estimate was too optimistic: go on with the exact continuation
+        beta = quot(rho.h, prev.h);
+        done = kRunning;
+      }
+      if (lane == 0) sNext = {0.f, beta, done};
+    }
+    __syncthreads();
+    alpha = sNext.alpha;
+    beta = sNext.beta;
+    done = sNext.done;
+    if (done != kRunning) break;
+  }
+
+  if (fault) done = kGuard;
+  // x64 += correction (the scaled operator's solution times the scale)
+  if (done != kNonFinite && done != kGuard && inxy) {
+    const double inv = (double)tscale / scale;
+#pragma unroll
+    for (int k = 0; k < CZ; ++k)
+      if (Z0 + k < g.nz) {
+        const int64_t c = c0 + g.plane * (Z0 + k);
+        a.x64[c] = fma((double)x[k], inv, a.x64[c]);
+      }
+  }
+  if (blk == 0 && tid == 0) {
+    st->rho = (double)rho.h + (double)rho.l;
+    st->rho0 = (double)rho0.h + (double)rho0.l;
+    st->scale = scale;
+    st->iter = iter;
+    st->launches = 1;
+    st->done = done;
+    st->fault = fault ? 1 : 0;
+    *(volatile uint32_t*)a.ctl = epoch;
+  }
+}
+
+template <int CZ, bool JAC>
+__global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant__ ResProb a) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ ResShared sh;
+  resident_solve<CZ, JAC>(a, blockIdx.x, sm, sh);
+}
+
+// ---- many instances in one launch --------------------------------------------
+// One block per SM; the instances' inner solves run on teams of blocks.  A team
+// needs all its blocks at once, so teams are formed by a scheduler in device
+// memory, run under a lock by the first warp of a block whose team has finished
+// (at the start: of block 0): it returns the team's blocks to the free list,
+// then starts the largest waiting instance that fits the free blocks, and so on
+// down the list.  Free blocks wait for a word in their mailbox.  A started team
+// always has all its blocks, so every wait ends.
+struct ResSched {
+  int lock, nfree, left;   // left: instances not yet started
+  int pad;
+};
+constexpr uint32_t kMailLimit = 1u << 28;  // looks at an empty mailbox before giving up
+constexpr uint32_t kExit = 0xffffffffu;
+
+struct ResBatchArgs {
+  const ResProb* prob;  // sorted by blocks, largest first
+  int nprob, nblocks;
+  ResSched* sched;      // zeroed before the launch, like the arrays that follow
+  int* started;         // [nprob]
+  int* freel;           // [nblocks] free block ids
+  uint32_t* sent;       // [nblocks] words sent to a block so far
+  unsigned long long* mail;  // [nblocks] {message, sequence number}
+  uint32_t* abort;      // the instances' abort flag, shared
+};
+
+// Returns `n` blocks (members, or all blocks when null) to the free list and starts what
+// fits.  One whole warp.
+__device__ void sched_release(const ResBatchArgs& a, const int* members, int n) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    uint32_t polls = 0;
+    while (atomicCAS(&a.sched->lock, 0, 1) != 0) {
+      if (++polls >= kPollLimit) {
+        *(volatile uint32_t*)a.abort = 1u;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncwarp();
+  if (*(volatile uint32_t*)a.abort != 0u) return;
+  volatile int* fl = a.freel;
+  volatile int* st = a.started;
+  int nfree = *(volatile int*)&a.sched->nfree, left = *(volatile int*)&a.sched->left;
+  for (int j = lane; j < n; j += 32) fl[nfree + j] = members != nullptr ? *(volatile const int*)(members + j) : j;
+  nfree += n;
+  __syncwarp();
+  auto send = [&](int id, uint32_t msg) {
+    volatile uint32_t* c = a.sent + id;
+    const uint32_t q = *c + 1u;
+    *c = q;
+    const unsigned long long w = (unsigned long long)msg | ((unsigned long long)q << 32);
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(a.mail + id), "l"(w) : "memory");
+  };
+  for (int i0 = 0; i0 < a.nprob && left > 0 && nfree > 0;) {
+    const int i = i0 + lane;
+    const bool fits = i < a.nprob && st[i] == 0 && a.prob[i].nblk <= nfree;
+    const unsigned m = __ballot_sync(kFull, fits);
+    if (m == 0u) {
+      i0 += 32;
+      continue;
+    }
+    const int p = i0 + __ffs(m) - 1;
+    const int need = a.prob[p].nblk;
+    int* mem = a.prob[p].team;
+    for (int j = lane; j < need; j += 32) *(volatile int*)(mem + j) = fl[nfree - 1 - j];
+    __threadfence();  // the team's list before its first block's message
+    __syncwarp();
+    for (int j = lane; j < need; j += 32)
+      send(fl[nfree - 1 - j], ((uint32_t)p << 12) | (uint32_t)j);
+    if (lane == 0) st[p] = 1;
+    nfree -= need;
+    --left;
+    __syncwarp();
+  }
+  if (left == 0) {  // nothing waits any more: the free blocks leave
+    for (int j = lane; j < nfree; j += 32) send(fl[j], kExit);
+    nfree = 0;
+  }
+  __syncwarp();
+  if (lane == 0) {
+    *(volatile int*)&a.sched->nfree = nfree;
+    *(volatile int*)&a.sched->left = left;
+    __threadfence();
+    atomicExch(&a.sched->lock, 0);
+  }
+  __syncwarp();
+}
+
+template <bool JAC>
+__global__ void __launch_bounds__(kRT, 1) resident_batch_kernel(const __grid_constant__ ResBatchArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ ResShared sh;
+  __shared__ ResProb prob;  // shared memory: no registers held for its fields
+  __shared__ uint32_t msg;
+  const int me = blockIdx.x, warp = threadIdx.x >> 5;
+  if (me == 0 && warp == 0) {
+    if (threadIdx.x == 0) *(volatile int*)&a.sched->left = a.nprob;
+    __syncwarp();
+    sched_release(a, nullptr, a.nblocks);
+  }
+  for (uint32_t seq = 1;; ++seq) {
+    if (threadIdx.x == 0) {
+      uint32_t got = kExit;
+      for (uint32_t polls = 0; polls < kMailLimit; ++polls) {
+        const uint2 w = ll_load(reinterpret_cast<const uint2*>(a.mail + me));
+        if (w.y == seq) {
+          got = w.x;
+          break;
+        }
+        if (*(volatile uint32_t*)a.abort != 0u) break;
+        __nanosleep(200);
+      }
+      msg = got;
+      if (got != kExit) prob = a.prob[got >> 12];
+    }
+    __syncthreads();
+    const uint32_t m = msg;
+    if (m == kExit) return;
+    const ResProb& p = prob;
+    const int rank = (int)(m & 4095u);
+    switch (p.cz) {
+      case 2: resident_solve<2, JAC>(p, rank, sm, sh); break;
+      case 4: resident_solve<4, JAC>(p, rank, sm, sh); break;
+      case 8: resident_solve<8, JAC>(p, rank, sm, sh); break;
+      case 12: resident_solve<12, JAC>(p, rank, sm, sh); break;
+      default: resident_solve<16, JAC>(p, rank, sm, sh); break;
+    }
+    __syncthreads();
+    // the blocks of a team end in the same iteration: its first block returns
+    // them together, so that a large instance waiting for that many blocks is
+    // not starved by small ones
+    if (rank == 0 && warp == 0) sched_release(a, p.team, p.nblk);
+  }
+}
+
+template <int CZ, bool JAC>
+cudaError_t launch_t(ResProb& a, cudaStream_t s) {
+  constexpr int smem = ResLayout<CZ>::floats(JAC) * 4;
+  auto fn = resident_kernel<CZ, JAC>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel((const void*)fn, dim3(a.nblk), dim3(kRT), args, smem, s);
+}
+
+template <int CZ>
+cudaError_t launch_cz(ResProb& a, bool jac, cudaStream_t s) {
+  return jac ? launch_t<CZ, true>(a, s) : launch_t<CZ, false>(a, s);
+}
+
+template <bool JAC>
+cudaError_t launch_batch_t(ResBatchArgs& a, cudaStream_t s) {
+  constexpr int smem = ResLayout<16>::floats(JAC) * 4;
+  auto fn = resident_batch_kernel<JAC>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel((const void*)fn, dim3(a.nblocks), dim3(kRT), args, smem, s);
+}
+
+size_t sched_words(int nprob, int nblocks) {  // 8-byte words after the sums and faces
+  return 4 + (size_t)nblocks + ((size_t)nprob + 2 * (size_t)nblocks + 1) / 2 + 2;
+}
+
+}  // namespace
+
+bool plan_resident(const Grid& g, int num_sms, bool dense, ResPlan* p) {
+  const int64_t bx = (g.nx + 31) / 32, by = (g.ny + kRW - 1) / kRW;
+  if (bx * by > num_sms) return false;
+  constexpr int fast[] = {1, 2, 4, 6, 8, 12, 16}, packed[] = {2, 4, 8, 12, 16};
+  const int* heights = dense ? packed : fast;
+  const int nh = dense ? 5 : 7;
+  double best = 0.0;
+  int cz = 0;
+  for (int h = 0; h < nh; ++h) {
+    const int64_t n = bx * by * ((g.nz + heights[h] - 1) / heights[h]);
+    if (n > num_sms) continue;
+    const double cost = dense ? (double)n * (1.9 + 0.21 * heights[h]) : (double)heights[h];
+    if (cz == 0 || cost < best) {
+      best = cost;
+      cz = heights[h];
+    }
+  }
+  if (cz == 0) return false;
+  p->cz = cz;
+  p->nbx = (int)bx;
+  p->nby = (int)by;
+  p->nbz = (int)((g.nz + cz - 1) / cz);
+  p->nblk = p->nbx * p->nby * p->nbz;
+  // control words, sums, faces (two buffers each)
+  p->words = 32 + (size_t)2 * p->nblk * 8 +
+             (size_t)2 * p->nblk * (2 * ((size_t)cz * kRW + (size_t)cz * 32 + kRW * 32));
+  return true;
+}
+
+ResProb make_res_prob(const Grid& g, const ResPlan& p, const void* coef, bool b16,
+                      const float* dinv, const double* r64, double* x64, CgState* st, double rtol,
+                      long long maxit, unsigned long long* comm) {
+  ResProb a;
+  a.g = g;
+  a.cz = p.cz;
+  a.nbx = p.nbx;
+  a.nby = p.nby;
+  a.nbz = p.nbz;
+  a.nblk = p.nblk;
+  a.coef = coef;
+  a.b16 = b16 ? 1 : 0;
+  a.dinv = dinv;
+  a.r64 = r64;
+  a.x64 = x64;
+  a.st = st;
+  a.rtol2 = rtol * rtol;
+  a.maxit = maxit;
+  a.ctl = reinterpret_cast<uint32_t*>(comm);
+  a.abort = a.ctl + 1;
+  a.part = reinterpret_cast<uint2*>(comm + 32);
+  a.face = a.part + (size_t)2 * p.nblk * 8;
+  a.team = nullptr;
+  return a;
+}
+
+cudaError_t launch_resident(const ResProb& prob, bool jac, cudaStream_t s) {
+  ResProb a = prob;
+  switch (a.cz) {
+    case 1: return launch_cz<1>(a, jac, s);
+    case 2: return launch_cz<2>(a, jac, s);
+    case 4: return launch_cz<4>(a, jac, s);
+    case 6: return launch_cz<6>(a, jac, s);
+    case 8: return launch_cz<8>(a, jac, s);
+    case 12: return launch_cz<12>(a, jac, s);
+    case 16: return launch_cz<16>(a, jac, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+size_t resident_batch_words(int nprob, int num_sms) { return sched_words(nprob, num_sms); }
+
+cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int num_sms, bool jac,
+                                  unsigned long long* sched, cudaStream_t s) {
+  const size_t words = sched_words(nprob, num_sms);
+  cudaError_t e = cudaMemsetAsync(sched, 0, words * 8, s);
+  if (e != cudaSuccess) return e;
+  ResBatchArgs a;
+  a.prob = prob_dev;
+  a.nprob = nprob;
+  a.nblocks = num_sms;
+  a.sched = reinterpret_cast<ResSched*>(sched);
+  a.abort = reinterpret_cast<uint32_t*>(sched + 2);
+  a.mail = sched + 4;
+  a.started = reinterpret_cast<int*>(sched + 4 + num_sms);
+  a.freel = a.started + nprob;
+  a.sent = reinterpret_cast<uint32_t*>(a.freel + num_sms);
+  return jac ? launch_batch_t<true>(a, s) : launch_batch_t<false>(a, s);
+}
+
+}  // namespace tpfa

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "sweep_plan.h"
 #include "tpfa.h"
 
@@ -216,6 +218,55 @@ cudaError_t launch_apply_batch(const BatchInst* inst, int ninst, int64_t nblocks
                                const float4* coef, const float* p, float* Ap, double* pAp,
                                const int* act, int need, double* partials,
                                unsigned int* counters, cudaStream_t s);
+
+// Resident CG (resident.cu): inner solves of grids that fit on the chip in one
+// cooperative launch.  An inner solve runs r32 = r64 / ||r64||, the CG iteration
+// to rtol or maxit and x64 += correction, and leaves the result in *st (whose
+// rr64 is read).
+struct ResPlan {
+  int cz, nbx, nby, nbz, nblk;  // brick height, bricks per axis, bricks
+  size_t words;                 // 8-byte words of exchange buffers
+};
+struct ResProb {
+  Grid g;
+  int cz, nbx, nby, nbz, nblk;
+  const void* coef;       // FP32 records, or BF16 records (b16)
+  int b16;
+  const float* dinv;      // Jacobi with BF16 records: M^-1 per cell
+  const double* r64;
+  double* x64;
+  CgState* st;
+  double rtol2;
+  long long maxit;
+  uint2* part;            // [2][nblk][4][2] words
+  uint2* face;            // [2][nblk][face words of a brick]
+  uint32_t* ctl;          // last epoch used
+  uint32_t* abort;        // set by a block whose wait ran out
+  int* team;              // batched: [nblk] blocks that run it
+};
+// Bricks for one grid; false when it does not fit at one brick per SM.
+// dense = false: the lowest bricks that fit (shortest iterations of a solve that
+// has the chip to itself).  dense = true: the bricks with the least block time
+// per iteration (nblk times the measured 1.9 + 0.21 cz us), for solves that
+// share the chip: 48x48x24 takes 12 blocks instead of 144.
+bool plan_resident(const Grid& g, int num_sms, bool dense, ResPlan* p);
+// comm: p.words words, zeroed once (and after a launch that ended with kGuard);
+// launches that share it are ordered.
+ResProb make_res_prob(const Grid& g, const ResPlan& p, const void* coef, bool b16,
+                      const float* dinv, const double* r64, double* x64, CgState* st, double rtol,
+                      long long maxit, unsigned long long* comm);
+cudaError_t launch_resident(const ResProb& prob, bool jac, cudaStream_t s);
+// Several FP32-record instances (dense plans, device table sorted by nblk, largest first;
+// at most kResMaxProb) in one launch; each has its own comm, team, and prob.abort ==
+// the word at sched + 2.
+constexpr int kResMaxProb = 1 << 19;
+size_t resident_batch_words(int nprob, int num_sms);
+cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int num_sms, bool jac,
+                                  unsigned long long* sched, cudaStream_t s);
+// Resident launches of one device are made one at a time (held from the launch
+// until the host has waited for it), so that the blocks of two of them never
+// compete for the same SMs.
+std::mutex& resident_mutex(int device);
 
 // Argument checks shared by the entry points: a device (or managed)
 // allocation on `device` that holds [p, p + bytes) and is `align`-aligned.
