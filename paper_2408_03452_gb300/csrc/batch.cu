@@ -568,9 +568,11 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       std::vector<int> order;
       for (int i = 0; i < N; ++i)
         if (active[i]) order.push_back(i);
-      // largest teams first, among equals the longest solve of the last step
+      // one launch per brick height; largest teams first, among equals the
+      // longest solve of the last step
       std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
         const int np = b->rplan[p].nblk, nq = b->rplan[q].nblk;
+        if (b->rplan[p].cz != b->rplan[q].cz) return b->rplan[p].cz > b->rplan[q].cz;
         return np != nq ? np > nq : iters[p] > iters[q];
       });
       std::vector<size_t> team0(N, 0);
@@ -594,8 +596,13 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       for (int i : order) hs[i].done = kGuard;  // what a team that never ran would leave
       BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
       BK(cudaEventRecord(b->ev[2], s));
-      const cudaError_t e = launch_resident_batch(b->prob_dev, (int)probs.size(), b->num_sms,
-                                                  b->precond == 1, b->sched, s);
+      cudaError_t e = cudaSuccess;
+      for (size_t p0 = 0, p1 = 0; p0 < probs.size() && e == cudaSuccess; p0 = p1) {
+        while (p1 < probs.size() && probs[p1].cz == probs[p0].cz) ++p1;
+        e = launch_resident_batch(b->prob_dev + p0, (int)(p1 - p0), probs[p0].cz, b->num_sms,
+                                  b->precond == 1, b->sched, s);
+        ++launches;
+      }
       if (e == cudaErrorCooperativeLaunchTooLarge && step == 0) {
         // fewer SMs than the device reports: this batch keeps the sweeps
         cudaGetLastError();
@@ -603,7 +610,6 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       } else {
         BK(e);
         BK(cudaEventRecord(b->ev[3], s));
-        ++launches;
         rc = read_states();
         if (rc) return rc;
         float ms = 0.f;

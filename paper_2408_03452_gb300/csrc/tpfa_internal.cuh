@@ -248,7 +248,7 @@ struct ResProb {
 // dense = false: the lowest bricks that fit (shortest iterations of a solve that
 // has the chip to itself).  dense = true: the bricks with the least block time
 // per iteration (nblk times the measured 1.9 + 0.21 cz us), for solves that
-// share the chip: 48x48x24 takes 12 blocks instead of 144.
+// share the chip (heights 4, 8, 16): 48x48x24 takes 12 blocks instead of 144.
 bool plan_resident(const Grid& g, int num_sms, bool dense, ResPlan* p);
 // comm: p.words words, zeroed once (and after a launch that ended with kGuard);
 // launches that share it are ordered.
@@ -256,13 +256,13 @@ ResProb make_res_prob(const Grid& g, const ResPlan& p, const void* coef, bool b1
                       const float* dinv, const double* r64, double* x64, CgState* st, double rtol,
                       long long maxit, unsigned long long* comm);
 cudaError_t launch_resident(const ResProb& prob, bool jac, cudaStream_t s);
-// Several FP32-record instances (dense plans, device table sorted by nblk, largest first;
-// at most kResMaxProb) in one launch; each has its own comm, team, and prob.abort ==
-// the word at sched + 2.
+// Several FP32-record instances with dense plans of one brick height cz (device
+// table sorted by nblk, largest first; at most kResMaxProb) in one launch; each has
+// its own comm, team, and prob.abort == the word at sched + 2.
 constexpr int kResMaxProb = 1 << 19;
 size_t resident_batch_words(int nprob, int num_sms);
-cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int num_sms, bool jac,
-                                  unsigned long long* sched, cudaStream_t s);
+cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int cz, int num_sms,
+                                  bool jac, unsigned long long* sched, cudaStream_t s);
 // Resident launches of one device are made one at a time (held from the launch
 // until the host has waited for it), so that the blocks of two of them never
 // compete for the same SMs.
