@@ -18,12 +18,7 @@
 // The input gradient of a convolution is the same operation with the taps
 // flipped and the weight matrices transposed.
 //
-// Weight gradient.  dw[t][co][ci] = sum_v dy[v][co] x[v + off_t][ci] is a
-// GEMM with rows (t, ci) -- 128/CIN taps per 128-row tile -- columns co and
-// the voxels as the reduction.  Chunks of 64 voxels of x (shifted per tap)
-// and of dy are transposed 8x8 at a time with movmatrix into K-major tiles;
-// CTAs split the voxel range, write FP32 partial tiles, and a second kernel
-// adds the partials in a fixed order.
+// Weight gradient: see conv_wgrad_kernel.
 #include <cuda_bf16.h>
 
 #include "net_internal.cuh"
@@ -53,12 +48,6 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 template <int N>
 __device__ __forceinline__ void cp_wait_groups() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
-  uint32_t d;
-  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
-  return d;
 }
 
 __device__ __forceinline__ bool bf16_positive(uint32_t h) {
@@ -909,129 +898,177 @@ conv_fwd_ws_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
   if (warp == 5) tc::tmem_dealloc(acc0, Cfg::kCols);
 }
 
+// ---- weight gradient ---------------------------------------------------------
+// dw[t][co][ci] = sum_u dy[u - dx][co] x[u + (dz, dy)][ci]: a GEMM whose reduction
+// runs over voxels.  Rows are (dx, co) -- three copies of dy, each shifted by a
+// voxel -- and columns (dz, dy, ci), so that one MMA covers every tap of a (dx)
+// row set.  Both operands are staged as they lie in memory, 16 bytes (8
+// channels) per voxel, in blocks [8 channels][kKV voxels]: that is the MN-major
+// core-matrix layout (8 voxels of 16 bytes per core matrix, next 8 voxels 128
+// bytes on, next 8 channels kKV * 16 bytes on), which the tensor core transposes
+// itself.  16 -> 32 on 16 samples of 32^3 (GB300): 88 us and 11 us for the sum of
+// the partials; 1,008 and 15 us when 8 x 8 blocks went through movmatrix, which
+// left the tensor core idle.  Bound by the staging copies (every x voxel is
+// fetched for nine rows, from L2).
+// CTAs split the voxel range, write FP32 partial tiles, and a second kernel adds
+// the partials in a fixed order.
 template <int CIN, int COUT>
 struct WgCfg {
-  static constexpr int kTaps = 128 / CIN;                    // taps per 128-row tile
-  static constexpr int kMTiles = (27 + kTaps - 1) / kTaps;
-  static constexpr int kKV = 64;                             // voxels per reduction chunk
-  static constexpr int kABytes = 128 * kKV * 2;
-  static constexpr int kBBytes = COUT * kKV * 2;
-  static constexpr int kStage = kABytes + kBBytes;
-  static constexpr int kSmem = 2 * kStage;
-  static constexpr uint32_t kCols = COUT < 32 ? 32 : COUT;
-  static_assert(128 % CIN == 0, "CIN must divide 128");
+  static constexpr int kKV = 64;                   // voxels per stage
+  static constexpr int kS = 4;                     // stages
+  static constexpr int kRg = CIN == 16 ? 9 : 3;    // (dz, dy) rows per CTA: all, or one dz
+  static constexpr int kParts = 9 / kRg;
+  static constexpr int kN = kRg * CIN;             // columns of the accumulator
+  static constexpr int kRows = 3 * COUT;           // rows that mean something
+  static constexpr int kMTiles = (kRows + 127) / 128;
+  static constexpr int kABlocks = kRows / 8, kBBlocks = kN / 8;
+  static constexpr int kBlock = kKV * 16;          // bytes of 8 channels of a stage
+  static constexpr int kABytes = kABlocks * kBlock;
+  static constexpr int kStage = (kABlocks + kBBlocks) * kBlock;
+  static constexpr int kSmem = kS * kStage;
+  static constexpr int kUse = kMTiles * kN;
+  static constexpr uint32_t kCols = kUse <= 64 ? 64 : kUse <= 128 ? 128 : 256;
+  static constexpr int kThreads = 256;
+  // the MMA reads 16 row blocks per tile, those past the last from what follows
+  // in the stage (their accumulator rows are never read)
+  static_assert(kMTiles * 16 * kBlock <= kStage, "row blocks past the end stay in the stage");
+  static_assert(kN % 16 == 0 && kN <= 256 && kUse <= 256 && kSmem <= 227 * 1024, "shape");
 };
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(256)
 conv_wgrad_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ dy,
                   float* __restrict__ ws, Vol g, int nchunks) {
   using Cfg = WgCfg<CIN, COUT>;
-  constexpr int kKV = Cfg::kKV;
-  constexpr int kAB = Cfg::kTaps * (CIN / 8) * (kKV / 8);  // 8x8 blocks of A per chunk
-  constexpr int kBB = (COUT / 8) * (kKV / 8);              // 8x8 blocks of B per chunk
+  constexpr int kKV = Cfg::kKV, S = Cfg::kS;
+  constexpr int ka = COUT / 8, kb = CIN / 8;
+  constexpr int kACopies = Cfg::kABlocks * kKV, kBCopies = Cfg::kBBlocks * kKV;
   extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ __align__(8) uint64_t bars[S];
   __shared__ uint32_t tbase;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int mt = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y;
+  const int part = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y;
   const int my = (nchunks - split + nsplit - 1) / nsplit;
+  const int u00 = g.g0 - 1;  // first voxel u: dy is not zero for u - dx in [g0, g1)
 
-  if (tid == 0) {
-    tc::mbar_init(&bars[0], 1);
-    tc::mbar_init(&bars[1], 1);
-  }
+  if (tid == 0)
+    for (int i = 0; i < S; ++i) tc::mbar_init(&bars[i], 1);
   if (warp == 0) tc::tmem_alloc(&tbase, Cfg::kCols);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t acc = tbase;
-  bool abort = false;
 
+  // copies of chunk i into stage i % S (one group per call, empty past the end)
+  auto load = [&](int i) {
+    if (i < my) {
+      const int u0 = u00 + (split + i * nsplit) * kKV;
+      unsigned char* sA = sm + (i % S) * Cfg::kStage;
+      unsigned char* sB = sA + Cfg::kABytes;
+      for (int c = tid; c < kACopies; c += 256) {
+        const int cb = c % ka, v = (c / ka) % kKV, d = c / (ka * kKV);
+        const int row = u0 + v - (d - 1);
+        const bool ok = row >= g.g0 && row < g.g1;
+        cp16z(sA + (d * ka + cb) * Cfg::kBlock + v * 16,
+              dy + (size_t)(ok ? row : 0) * COUT + cb * 8, ok);
+      }
+      for (int c = tid; c < kBCopies; c += 256) {
+        const int cb = c % kb, v = (c / kb) % kKV, q = c / (kb * kKV);
+        const int rg = part * Cfg::kRg + q;
+        const int row = u0 + v + (rg / 3 - 1) * g.pp + (rg % 3 - 1) * g.wp;
+        const bool ok = row >= 0 && row < g.vp;
+        cp16z(sB + (q * kb + cb) * Cfg::kBlock + v * 16,
+              x + (size_t)(ok ? row : 0) * CIN + cb * 8, ok);
+      }
+    }
+    cp_commit_group();
+  };
+
+  bool abort = false;
+  for (int i = 0; i < S - 1; ++i) load(i);
   for (int i = 0; i < my; ++i) {
-    const int buf = i & 1;
-    if (i >= 2) {
-      const bool ok = tc::mbar_wait(&bars[buf], ((i - 2) >> 1) & 1, kWaitLimit);
-      if (__syncthreads_or(!ok)) {
-        abort = true;
-        break;
-      }
-    }
-    const int v0 = g.g0 + (split + i * nsplit) * kKV;
-    unsigned char* sA = sm + buf * Cfg::kStage;
-    unsigned char* sB = sA + Cfg::kABytes;
-    for (int b = warp; b < kAB + kBB; b += 4) {
-      uint32_t val = 0;
-      if (b < kAB) {
-        const int vb = b % 8, cb = (b / 8) % (CIN / 8), tl = b / (8 * (CIN / 8));
-        const int t = mt * Cfg::kTaps + tl;
-        if (t < 27) {
-          const int off = (t / 9 - 1) * g.pp + ((t / 3) % 3 - 1) * g.wp + (t % 3 - 1);
-          const int v = v0 + vb * 8 + (lane >> 2) + off;
-          if (v >= 0 && v < g.vp)
-            val = *reinterpret_cast<const uint32_t*>(x + (size_t)v * CIN + cb * 8 + 2 * (lane & 3));
-        }
-        val = movmatrix_trans(val);
-        *reinterpret_cast<uint32_t*>(
-            sA + tc::kmajor_off(tl * CIN + cb * 8 + (lane >> 2), vb * 8 + 2 * (lane & 3), kKV)) = val;
-      } else {
-        const int bb = b - kAB, vb = bb % 8, cb = bb / 8;
-        const int v = v0 + vb * 8 + (lane >> 2);
-        if (v < g.g1)
-          val = *reinterpret_cast<const uint32_t*>(dy + (size_t)v * COUT + cb * 8 + 2 * (lane & 3));
-        val = movmatrix_trans(val);
-        *reinterpret_cast<uint32_t*>(
-            sB + tc::kmajor_off(cb * 8 + (lane >> 2), vb * 8 + 2 * (lane & 3), kKV)) = val;
-      }
-    }
+    const int buf = i % S;
+    cp_wait_groups<S - 2>();  // chunk i has landed
     tc::fence_proxy_async();
     __syncthreads();
     if (tid == 0) {
       tc::fence_after();
-      constexpr uint32_t idesc = tc::idesc_bf16_f32(128, COUT);
-      const uint32_t a0 = tc::smem_addr(sA), b0 = tc::smem_addr(sB);
+      // bits 15, 16: A and B MN-major
+      constexpr uint32_t idesc = tc::idesc_bf16_f32(128, Cfg::kN) | (1u << 15) | (1u << 16);
+      const uint32_t a0 = tc::smem_addr(sm + buf * Cfg::kStage), b0 = a0 + Cfg::kABytes;
 #pragma unroll
       for (int ks = 0; ks < kKV / 16; ++ks)
-        tc::mma_bf16(acc, tc::smem_desc(a0 + ks * 256, 128, (kKV / 8) * 128),
-                     tc::smem_desc(b0 + ks * 256, 128, (kKV / 8) * 128), idesc, (i | ks) != 0);
+#pragma unroll
+        for (int mt = 0; mt < Cfg::kMTiles; ++mt)
+          tc::mma_bf16(acc + mt * Cfg::kN,
+                       tc::smem_desc(a0 + mt * 16 * Cfg::kBlock + ks * 256, 128, Cfg::kBlock),
+                       tc::smem_desc(b0 + ks * 256, 128, Cfg::kBlock), idesc, (i | ks) != 0);
       tc::mma_commit(&bars[buf]);
     }
+    // chunk i + S - 1 reuses the stage of chunk i - 1
+    bool ok = true;
+    if (i >= 1) ok = tc::mbar_wait(&bars[(i - 1) % S], ((i - 1) / S) & 1, kWaitLimit);
+    if (__syncthreads_or(!ok)) {
+      abort = true;
+      break;
+    }
+    load(i + S - 1);
   }
+  cp_wait_all();
   if (!abort && my > 0) {
-    const bool ok = tc::mbar_wait(&bars[(my - 1) & 1], ((my - 1) >> 1) & 1, kWaitLimit);
+    const bool ok = tc::mbar_wait(&bars[(my - 1) % S], ((my - 1) / S) & 1, kWaitLimit);
     if (__syncthreads_or(!ok)) abort = true;
   }
   tc::fence_after();
-  float* out = ws + ((size_t)(split * gridDim.x + mt) * 128 + warp * 32 + lane) * COUT;
-  if (!abort && my > 0) {
+  if (warp < 4) {
 #pragma unroll
-    for (int c0 = 0; c0 < COUT; c0 += 8) {
-      float v[8];
-      tc::tmem_ld8(acc + ((uint32_t)(warp * 32) << 16) + c0, v);
-      *reinterpret_cast<float4*>(out + c0) = make_float4(v[0], v[1], v[2], v[3]);
-      *reinterpret_cast<float4*>(out + c0 + 4) = make_float4(v[4], v[5], v[6], v[7]);
+    for (int mt = 0; mt < Cfg::kMTiles; ++mt) {
+      const int row = mt * 128 + warp * 32 + lane;
+      float* out = ws + ((size_t)(split * Cfg::kParts + part) * Cfg::kRows + row) * Cfg::kN;
+#pragma unroll
+      for (int c0 = 0; c0 < Cfg::kN; c0 += 16) {
+        float v[16];
+        if (!abort && my > 0)
+          tc::tmem_ld16(acc + ((uint32_t)(warp * 32) << 16) + mt * Cfg::kN + c0, v);
+        else
+          for (int c = 0; c < 16; ++c) v[c] = 0.f;
+        if (row < Cfg::kRows)
+#pragma unroll
+          for (int c = 0; c < 16; c += 4)
+            *reinterpret_cast<float4*>(out + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+      }
     }
-  } else {
-    for (int c = 0; c < COUT; ++c) out[c] = 0.f;
-    if (abort && tid == 0) atomicOr(&g_tc_timeout, 1);
   }
+  if (abort && tid == 0) atomicOr(&g_tc_timeout, 1);
   tc::fence_before();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(acc, Cfg::kCols);
 }
 
+// dw from the partial tiles: 32 outputs per block (consecutive ci), the splits
+// dealt to its 8 warps and added in a fixed order in FP64.
 template <int CIN, int COUT>
-__global__ void wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ dw,
-                                    int nsplit, int accumulate) {
+__global__ void __launch_bounds__(256)
+wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ dw, int nsplit,
+                    int accumulate) {
   using Cfg = WgCfg<CIN, COUT>;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 27 * COUT * CIN) return;
+  __shared__ double part[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;  // 27 COUT CIN is a multiple of 32
   const int ci = i % CIN, co = (i / CIN) % COUT, t = i / (CIN * COUT);
-  const int mt = t / Cfg::kTaps, row = (t % Cfg::kTaps) * CIN + ci;
+  const int rg = t / 3, d = t % 3;
+  const float* src = ws + ((size_t)(rg / Cfg::kRg) * Cfg::kRows + d * COUT + co) * Cfg::kN +
+                     (rg % Cfg::kRg) * CIN + ci;
   double s = 0.0;
-  for (int sp = 0; sp < nsplit; ++sp)
-    s += ws[((size_t)(sp * Cfg::kMTiles + mt) * 128 + row) * COUT + co];
-  dw[i] = accumulate ? (float)(dw[i] + s) : (float)s;
+#pragma unroll 4
+  for (int sp = warp; sp < nsplit; sp += 8)
+    s += src[(size_t)sp * Cfg::kParts * Cfg::kRows * Cfg::kN];
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+    for (int w = 1; w < 8; ++w) s += part[w][lane];
+    dw[i] = accumulate ? (float)(dw[i] + s) : (float)s;
+  }
 }
 
 // CTAs per SM from the shared-memory and tensor-memory budgets (the occupancy
@@ -1141,32 +1178,35 @@ cudaError_t ws_launch(const uint16_t* x, const uint16_t* w, const float* bias,
   return cudaGetLastError();
 }
 
-int wgrad_splits(int mtiles, int nchunks) {
+// one CTA per SM over all parts
+int wgrad_splits(int parts, int nchunks) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  int ns = (2 * nsm + mtiles - 1) / mtiles;
+  int ns = nsm / parts;
   if (ns > nchunks) ns = nchunks;
   return ns < 1 ? 1 : ns;
 }
+
+// chunks of 64 voxels u over [g0 - 1, g1 + 1)
+int wgrad_chunks(const Vol& g) { return g.g1 > g.g0 ? (g.g1 - g.g0 + 2 + 63) / 64 : 0; }
 
 template <int CIN, int COUT>
 cudaError_t wgrad_launch(const uint16_t* x, const uint16_t* dy, float* dw, float* ws,
                          const Vol& g, int accumulate, cudaStream_t s) {
   using Cfg = WgCfg<CIN, COUT>;
-  const int nchunks = (g.g1 - g.g0 + Cfg::kKV - 1) / Cfg::kKV;
-  const int nsplit = wgrad_splits(Cfg::kMTiles, nchunks);
+  const int nchunks = wgrad_chunks(g);
+  const int nsplit = wgrad_splits(Cfg::kParts, nchunks);
   if (nchunks > 0) {
     cudaFuncSetAttribute(conv_wgrad_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          Cfg::kSmem);
     conv_wgrad_kernel<CIN, COUT>
-        <<<dim3(Cfg::kMTiles, nsplit), 128, Cfg::kSmem, s>>>(x, dy, ws, g, nchunks);
+        <<<dim3(Cfg::kParts, nsplit), Cfg::kThreads, Cfg::kSmem, s>>>(x, dy, ws, g, nchunks);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  const int n = 27 * COUT * CIN;
-  wgrad_reduce_kernel<CIN, COUT><<<(n + 255) / 256, 256, 0, s>>>(ws, dw, nchunks > 0 ? nsplit : 0,
-                                                                  accumulate);
+  wgrad_reduce_kernel<CIN, COUT><<<27 * COUT * CIN / 32, 256, 0, s>>>(
+      ws, dw, nchunks > 0 ? nsplit : 0, accumulate);
   return cudaGetLastError();
 }
 
@@ -1221,10 +1261,10 @@ cudaError_t conv_fwd(const uint16_t* x, const uint16_t* w, const float* bias, co
 }
 
 size_t conv_wgrad_ws_bytes(const Vol& g, int cin, int cout) {
-  const int mtiles = (27 + 128 / cin - 1) / (128 / cin);
-  const int nchunks = (g.g1 - g.g0 + 63) / 64;
-  const int ns = wgrad_splits(mtiles, nchunks < 1 ? 1 : nchunks);
-  return (size_t)ns * mtiles * 128 * cout * sizeof(float);
+  const int parts = cin == 16 ? 1 : 3;
+  const int nchunks = wgrad_chunks(g);
+  // 27 cin cout floats per split (all parts together)
+  return (size_t)wgrad_splits(parts, nchunks < 1 ? 1 : nchunks) * 27 * cin * cout * sizeof(float);
 }
 
 cudaError_t conv_wgrad(const uint16_t* x, const uint16_t* dy, float* dw, float* ws, const Vol& g,
