@@ -653,14 +653,12 @@ conv_fwd_zf_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
 }
 
 // ---- the folded z-marching kernel with warp-specialised roles -------------
-// Same work units, row-group triples, folded MMAs (N = 3 cout) and TMEM ring
-// of accumulators as conv_fwd_zf_kernel, but the three kinds of work no
-// longer wait for each other at a block barrier:
-//   warp 4 copies triples into a ring of ST slots (cp.async); once the next
-//          triple's copies are issued, each lane waits for its copies of the
-//          previous one, fences them to the async proxy and arrives on that
-//          slot's "full" mbarrier;
-//   warp 5 (one thread) issues the MMAs of a triple once it is full and the
+// Same work units, folded MMAs (N = 3 cout) and TMEM ring of accumulators as
+// conv_fwd_zf_kernel, with the three kinds of work on warps of their own:
+//   warp 5 (one thread) copies row-group triples into a ring of ST slots: one
+//          tensor-map copy of 130 voxels per row group, voxels outside the volume
+//          filled with zeros, and before them the 27 weight matrices;
+//   warp 4 (one thread) issues the MMAs of a triple once it is full and the
 //          slot of the output it starts is free, and commits to the triple's
 //          "empty" barrier and to the "full" barrier of the output the triple
 //          completes;
@@ -669,14 +667,24 @@ conv_fwd_zf_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
 //          rounding and the stores.
 // Every wait is bounded; a wait that runs out raises a shared abort flag that
 // every role checks, and the kernel records the timeout like the others.
+//
+// Voxels stay whole rows of cin channels in shared memory, in the copy engine's
+// swizzle of that width, which the tensor core reads directly: a tap is the row
+// group started dx rows later.  A layout of 8-channel blocks, which needs no
+// swizzle, has to be filled 16 bytes at a time: its copies, not the MMAs, set the
+// time (1,700 cycles per plane step and SM for 16 -> 16 against 400 for
+// the nine MMAs, each 32 + N / 4 cycles).
+// WSFIGURES
 template <int CIN, int COUT>
 struct WsCfg {
-  static constexpr int kST = zm_stages<CIN, COUT>();
-  static constexpr int kWTap = COUT * CIN * 2;
+  static constexpr int kRow = CIN * 2;
+  static constexpr int kWTap = COUT * kRow;
   static constexpr int kWBytes = 27 * kWTap;
-  static constexpr int kRGBytes = kRG * CIN * 2;
+  static constexpr int kRGBytes = (kRG * kRow + 1023) / 1024 * 1024;
   static constexpr int kTriple = 3 * kRGBytes;
-  static constexpr int kSmem = kWBytes + kST * kTriple;
+  // two CTAs per SM where two rings of three or more slots fit, else one
+  static constexpr int kST = CIN == 64 ? 2 : COUT == 64 ? 4 : CIN == 32 ? 3 : COUT == 32 ? 5 : 6;
+  static constexpr int kSmem = kWBytes + kST * kTriple + 1024;
   static constexpr int kR = 256 / COUT;
   static constexpr uint32_t kCols = 256;
   static_assert(kSmem <= 227 * 1024, "shared memory");
@@ -687,46 +695,43 @@ __device__ __forceinline__ void mbar_arrive1(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
 }
 
+struct RowMaps {
+  CUtensorMap a, b;
+};
+
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(192)
-conv_fwd_ws_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w,
-                   const float* __restrict__ bias, const uint16_t* __restrict__ mask,
-                   uint16_t* __restrict__ y, Vol g, int flags, ZmGrid zg) {
+conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict__ bias,
+                   const uint16_t* __restrict__ mask, uint16_t* __restrict__ y, Vol g, int flags,
+                   ZmGrid zg) {
   using Cfg = WsCfg<CIN, COUT>;
   constexpr int ST = Cfg::kST;
   constexpr int R = Cfg::kR;
-  constexpr int kc = CIN / 8;
-  constexpr int kChunks = 3 * kRG * kc;  // 16-byte copies per triple
-  extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ __align__(8) uint64_t tfull[ST], tempty[ST], afull[R], aempty[R], done_bar;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t tfull[ST], tempty[ST], afull[R], aempty[R], wfull, done_bar;
   __shared__ uint32_t tbase;
   __shared__ float sbias[COUT];
   __shared__ volatile int s_abort;
-  unsigned char* sW = sm;
-  unsigned char* sR = sm + Cfg::kWBytes;
+  unsigned char* sR = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char* sW = sR + ST * Cfg::kTriple;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  // weights in the folded order (see conv_fwd_zf_kernel)
-  for (int i = tid; i < 27 * COUT * kc; i += 192) {
-    const int c = i % kc, r = (i / kc) % COUT, t = i / (kc * COUT);
-    const int tt = (t % 9) * 3 + (2 - t / 9);
-    const uint4 v = *reinterpret_cast<const uint4*>(w + ((size_t)t * COUT + r) * CIN + c * 8);
-    *reinterpret_cast<uint4*>(sW + tt * Cfg::kWTap + tc::kmajor_off(r, c * 8, CIN)) = v;
-  }
   if (tid < COUT) sbias[tid] = bias ? bias[tid] : 0.f;
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) {
-      tc::mbar_init(&tfull[i], 32);
+      tc::mbar_init(&tfull[i], 1);
       tc::mbar_init(&tempty[i], 1);
     }
     for (int i = 0; i < R; ++i) {
       tc::mbar_init(&afull[i], 1);
       tc::mbar_init(&aempty[i], 4);
     }
+    tc::mbar_init(&wfull, 1);
     tc::mbar_init(&done_bar, 1);
     s_abort = 0;
   }
-  if (warp == 5) tc::tmem_alloc(&tbase, Cfg::kCols);
+  if (warp == 4) tc::tmem_alloc(&tbase, Cfg::kCols);
   tc::fence_proxy_async();
   tc::fence_before();
   __syncthreads();
@@ -740,54 +745,46 @@ conv_fwd_ws_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
     return false;
   };
 
-  if (warp == 4) {
-    // ---- copy warp -----------------------------------------------------------
-    // A triple is handed to the tensor core once the copies of the next one
-    // are issued: each lane waits for its own copies of the triple, makes
-    // them visible to the async proxy (the MMAs read shared memory through
-    // it), then arrives on the triple's "full" barrier.
-    int tg = 0, pend = -1;  // pend: slot of the triple whose arrival is due
-    auto hand_over = [&](bool last) {
-      if (pend < 0) return;
-      if (last) cp_wait_all();
-      else cp_wait_groups<1>();
-      tc::fence_proxy_async();
-      mbar_arrive1(&tfull[pend]);
-      pend = -1;
-    };
-    for (int u = blockIdx.x; u < zg.units && !s_abort; u += gridDim.x) {
-      const int bi = u % zg.nb, cz = u / zg.nb;
-      const int sidx = cz / zg.nzc;
-      const int z0 = (cz % zg.nzc) * zg.zc;
-      const int nout = min(zg.zc, g.nz - z0);
-      const int kp0 = sidx * g.dp + 1 + z0;
-      const int seg = bi * 128;
-      for (int j = 0; j < nout + 2; ++j, ++tg) {
-        const int s = tg % ST;
-        if (tg >= ST && !wait(&tempty[s], ((tg / ST) - 1) & 1)) break;
-        const int base = seg + (kp0 - 1 + j) * g.pp - g.wp - 1;
-        unsigned char* st = sR + s * Cfg::kTriple;
-        for (int i = lane; i < kChunks; i += 32) {
-          const int c = i % kc, v = (i / kc) % kRG, gi = i / (kc * kRG);
-          const int row = base + gi * g.wp + v;
-          const bool ok = row >= 0 && row < g.vp;
-          cp16z(st + gi * Cfg::kRGBytes + c * (kRG * 16) + v * 16,
-                x + (size_t)(ok ? row : 0) * CIN + c * 8, ok);
+  if (warp == 5) {
+    // ---- copies ---------------------------------------------------------------
+    if (lane == 0) {
+      // weights in the folded order (see conv_fwd_zf_kernel)
+      tc::mbar_expect(&wfull, Cfg::kWBytes);
+      for (int t = 0; t < 27; ++t)
+        tc::tma_2d(sW + ((t % 9) * 3 + (2 - t / 9)) * Cfg::kWTap, &maps.b, &wfull, 0, t * COUT);
+      int tg = 0;
+      for (int u = blockIdx.x; u < zg.units && !s_abort; u += gridDim.x) {
+        const int bi = u % zg.nb, cz = u / zg.nb;
+        const int sidx = cz / zg.nzc;
+        const int z0 = (cz % zg.nzc) * zg.zc;
+        const int nout = min(zg.zc, g.nz - z0);
+        const int kp0 = sidx * g.dp + 1 + z0;
+        const int seg = bi * 128;
+        bool stop = false;
+        for (int j = 0; j < nout + 2; ++j, ++tg) {
+          const int s = tg % ST;
+          if (tg >= ST && !wait(&tempty[s], ((tg / ST) - 1) & 1)) { stop = true; break; }
+          const int base = seg + (kp0 - 1 + j) * g.pp - g.wp - 1;  // first row of the triple
+          unsigned char* st = sR + s * Cfg::kTriple;
+          tc::mbar_expect(&tfull[s], 3 * kRG * Cfg::kRow);
+#pragma unroll
+          for (int gi = 0; gi < 3; ++gi)
+            tc::tma_2d(st + gi * Cfg::kRGBytes, &maps.a, &tfull[s], 0, base + gi * g.wp);
         }
-        cp_commit_group();
-        hand_over(false);  // the previous triple
-        pend = s;
+        if (stop) break;
       }
+      // no copy outlives the block: wait for the last (up to ST) triples and the weights
+      tc::mbar_wait(&wfull, 0, kWaitLimit);
+      for (int j = tg - 1; j >= 0 && j >= tg - ST; --j)
+        if (!tc::mbar_wait(&tfull[j % ST], (j / ST) & 1, kWaitLimit)) s_abort = 1;
     }
-    hand_over(true);
-    cp_wait_all();
-  } else if (warp == 5) {
+  } else if (warp == 4) {
     // ---- MMA thread --------------------------------------------------------
     if (lane == 0) {
-      const uint64_t adesc0 = tc::smem_desc(tc::smem_addr(sR), kRG * 16, 128);
-      const uint64_t bdesc0 = tc::smem_desc(tc::smem_addr(sW), 128, kc * 128);
+      const uint64_t adesc0 = tc::smem_desc_sw(tc::smem_addr(sR), 16, 8 * Cfg::kRow, Cfg::kRow);
+      const uint64_t bdesc0 = tc::smem_desc_sw(tc::smem_addr(sW), 16, 8 * Cfg::kRow, Cfg::kRow);
       int tg = 0, obase = 0;
-      bool stop = false;
+      bool stop = !wait(&wfull, 0);
       for (int u = blockIdx.x; u < zg.units && !stop; u += gridDim.x) {
         const int cz = u / zg.nb;
         const int z0 = (cz % zg.nzc) * zg.zc;
@@ -801,35 +798,41 @@ conv_fwd_ws_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
             if (oc >= R && !wait(&aempty[oc % R], ((oc / R) - 1) & 1)) { stop = true; break; }
           }
           tc::fence_after();
-          const uint64_t slot = adesc0 + (uint64_t)(s * (Cfg::kTriple >> 4));
-          auto mma_range = [&](int ka, int kb, uint64_t ad, int tile0, int ks, bool accum) {
-            int k = ka;
-            while (k <= kb) {
-              const int sl = (obase + k) % R;
-              const int n = min(kb - k + 1, R - sl);
-              const uint64_t bd =
-                  bdesc0 + (uint64_t)(((tile0 + (k - ka)) * Cfg::kWTap + ks * 256) >> 4);
-              tc::mma_bf16(acc0 + (uint32_t)(sl * COUT), ad, bd,
-                           tc::idesc_bf16_f32(128, n * COUT), accum);
-              k += n;
-            }
+          // Accumulator slots, instruction descriptors and operand addresses of
+          // the triple are the same for its 9 (dy, dx) x CIN / 16 steps up to
+          // constants, and formed once.
+          const int sl = (obase + klo) % R;
+          const int n1 = min(khi - klo + 1, R - sl), n2 = khi - klo + 1 - n1;
+          const uint32_t d1 = acc0 + (uint32_t)(sl * COUT);
+          const uint32_t i1 = tc::idesc_bf16_f32(128, n1 * COUT);
+          const uint32_t i2 = tc::idesc_bf16_f32(128, n2 * COUT);
+          const uint64_t a0 = adesc0 + (uint32_t)(s * (Cfg::kTriple >> 4));
+          const uint64_t b1 = bdesc0 + (uint32_t)((2 - j + klo) * (Cfg::kWTap >> 4));
+          const uint64_t b2 = b1 + (uint32_t)(n1 * (Cfg::kWTap >> 4));
+          // first step: output j starts with it, the outputs before j go on
+          if (khi == j) {
+            for (int k = klo; k <= j; ++k)
+              tc::mma_bf16(acc0 + (uint32_t)(((obase + k) % R) * COUT), a0,
+                           b1 + (uint32_t)((k - klo) * (Cfg::kWTap >> 4)),
+                           tc::idesc_bf16_f32(128, COUT), k < j);
+          } else {
+            tc::mma_bf16(d1, a0, b1, i1, true);
+            if (n2 > 0) tc::mma_bf16(acc0, a0, b2, i2, true);
+          }
+          auto step = [&](int st, bool two) {
+            const int gd = st / (CIN / 16), ks = st % (CIN / 16);  // gd = 3 gi + dx
+            const uint32_t ao = (gd / 3 * Cfg::kRGBytes + gd % 3 * Cfg::kRow + ks * 32) >> 4;
+            const uint32_t bo = (gd * 3 * Cfg::kWTap + ks * 32) >> 4;
+            tc::mma_bf16(d1, a0 + ao, b1 + bo, i1, true);
+            if (two) tc::mma_bf16(acc0, a0 + ao, b2 + bo, i2, true);
           };
+          if (n2 == 0) {
+#pragma unroll
+            for (int st = 1; st < 9 * (CIN / 16); ++st) step(st, false);
+          } else {
 #pragma unroll 1
-          for (int gi = 0; gi < 3; ++gi)
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-              for (int ks = 0; ks < CIN / 16; ++ks) {
-                const uint64_t ad =
-                    slot + (uint64_t)((gi * Cfg::kRGBytes + dx * 16 + ks * 2 * kRG * 16) >> 4);
-                const int grp = (gi * 3 + dx) * 3 + 2 - j;
-                if ((gi | dx | ks) == 0 && khi == j) {
-                  if (klo < j) mma_range(klo, j - 1, ad, grp + klo, ks, true);
-                  mma_range(j, j, ad, grp + j, ks, false);
-                } else {
-                  mma_range(klo, khi, ad, grp + klo, ks, true);
-                }
-              }
+            for (int st = 1; st < 9 * (CIN / 16); ++st) step(st, true);
+          }
           tc::mma_commit(&tempty[s]);
           if (j >= 2) tc::mma_commit(&afull[(obase + j - 2) % R]);  // output j-2 is final
         }
@@ -895,136 +898,142 @@ conv_fwd_ws_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
   tc::fence_before();
   __syncthreads();
   if (s_abort && tid == 0) atomicOr(&g_tc_timeout, 1);
-  if (warp == 5) tc::tmem_dealloc(acc0, Cfg::kCols);
+  if (warp == 4) tc::tmem_dealloc(acc0, Cfg::kCols);
 }
 
 // ---- weight gradient ---------------------------------------------------------
 // dw[t][co][ci] = sum_u dy[u - dx][co] x[u + (dz, dy)][ci]: a GEMM whose reduction
-// runs over voxels.  Rows are (dx, co) -- three copies of dy, each shifted by a
-// voxel -- and columns (dz, dy, ci), so that one MMA covers every tap of a (dx)
-// row set.  Both operands are staged as they lie in memory, 16 bytes (8
-// channels) per voxel, in blocks [8 channels][kKV voxels]: that is the MN-major
-// core-matrix layout (8 voxels of 16 bytes per core matrix, next 8 voxels 128
-// bytes on, next 8 channels kKV * 16 bytes on), which the tensor core transposes
-// itself.  16 -> 32 on 16 samples of 32^3 (GB300): 88 us and 11 us for the sum of
-// the partials; 1,008 and 15 us when 8 x 8 blocks went through movmatrix, which
-// left the tensor core idle.  Bound by the staging copies (every x voxel is
-// fetched for nine rows, from L2).
+// runs over voxels.  Rows are (dx, co) and columns (dz, dy, ci), so that one MMA
+// covers every tap of its columns.  Both operands are staged by the copy engine
+// as they lie in memory, voxel rows of all channels in the swizzle of that width,
+// and the tensor core reads them MN-major: a row of the stage is one step of the
+// reduction, and the next block of channels (lbo) is the next (dz, dy) row set
+// for x, and for dy the same rows started one voxel later, which makes the three
+// dx shifts out of one copy of dy.  Row blocks past the third (dx = 2, 3, ..) are
+// computed and ignored.
 // CTAs split the voxel range, write FP32 partial tiles, and a second kernel adds
 // the partials in a fixed order.
+// WGFIGURES
 template <int CIN, int COUT>
 struct WgCfg {
   static constexpr int kKV = 64;                   // voxels per stage
-  static constexpr int kS = 4;                     // stages
+  static constexpr int kS = 6;                     // stages
   static constexpr int kRg = CIN == 16 ? 9 : 3;    // (dz, dy) rows per CTA: all, or one dz
   static constexpr int kParts = 9 / kRg;
   static constexpr int kN = kRg * CIN;             // columns of the accumulator
   static constexpr int kRows = 3 * COUT;           // rows that mean something
   static constexpr int kMTiles = (kRows + 127) / 128;
-  static constexpr int kABlocks = kRows / 8, kBBlocks = kN / 8;
-  static constexpr int kBlock = kKV * 16;          // bytes of 8 channels of a stage
-  static constexpr int kABytes = kABlocks * kBlock;
-  static constexpr int kStage = (kABlocks + kBBlocks) * kBlock;
-  static constexpr int kSmem = kS * kStage;
+  static constexpr int kARow = COUT * 2, kBRow = CIN * 2;
+  static constexpr int kAVox = kKV + 8;            // voxels of dy a stage needs (and reads)
+  static constexpr int kABytes = (kAVox * kARow + 1023) / 1024 * 1024;
+  static constexpr int kBRg = kKV * kBRow;         // one (dz, dy) row set
+  static constexpr int kStage = kABytes + kRg * kBRg;
+  static constexpr uint32_t kTx = kAVox * kARow + kRg * kBRg;
+  static constexpr int kSmem = kS * kStage + 1024;
   static constexpr int kUse = kMTiles * kN;
   static constexpr uint32_t kCols = kUse <= 64 ? 64 : kUse <= 128 ? 128 : 256;
-  static constexpr int kThreads = 256;
-  // the MMA reads 16 row blocks per tile, those past the last from what follows
-  // in the stage (their accumulator rows are never read)
-  static_assert(kMTiles * 16 * kBlock <= kStage, "row blocks past the end stay in the stage");
+  // the last voxel read: 63 of the stage, plus the shift of the last row block
+  static_assert(kKV - 1 + 128 * kMTiles / COUT - 1 < kAVox, "row blocks stay in the stage");
+  static_assert(kBRg % 1024 == 0, "row sets start on a swizzle period");
   static_assert(kN % 16 == 0 && kN <= 256 && kUse <= 256 && kSmem <= 227 * 1024, "shape");
 };
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(256)
-conv_wgrad_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ dy,
-                  float* __restrict__ ws, Vol g, int nchunks) {
+__global__ void __launch_bounds__(192)
+conv_wgrad_kernel(const __grid_constant__ RowMaps maps, float* __restrict__ ws, Vol g,
+                  int nchunks) {
   using Cfg = WgCfg<CIN, COUT>;
   constexpr int kKV = Cfg::kKV, S = Cfg::kS;
-  constexpr int ka = COUT / 8, kb = CIN / 8;
-  constexpr int kACopies = Cfg::kABlocks * kKV, kBCopies = Cfg::kBBlocks * kKV;
-  extern __shared__ __align__(128) unsigned char sm[];
-  __shared__ __align__(8) uint64_t bars[S];
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t full[S], empty[S], done_bar;
   __shared__ uint32_t tbase;
+  __shared__ volatile int s_abort;
+  unsigned char* sm = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int part = blockIdx.x, split = blockIdx.y, nsplit = gridDim.y;
   const int my = (nchunks - split + nsplit - 1) / nsplit;
   const int u00 = g.g0 - 1;  // first voxel u: dy is not zero for u - dx in [g0, g1)
 
-  if (tid == 0)
-    for (int i = 0; i < S; ++i) tc::mbar_init(&bars[i], 1);
-  if (warp == 0) tc::tmem_alloc(&tbase, Cfg::kCols);
+  if (tid == 0) {
+    for (int i = 0; i < S; ++i) {
+      tc::mbar_init(&full[i], 1);
+      tc::mbar_init(&empty[i], 1);
+    }
+    tc::mbar_init(&done_bar, 1);
+    s_abort = 0;
+  }
+  if (warp == 4) tc::tmem_alloc(&tbase, Cfg::kCols);
+  tc::fence_proxy_async();
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t acc = tbase;
-
-  // copies of chunk i into stage i % S (one group per call, empty past the end)
-  auto load = [&](int i) {
-    if (i < my) {
-      const int u0 = u00 + (split + i * nsplit) * kKV;
-      unsigned char* sA = sm + (i % S) * Cfg::kStage;
-      unsigned char* sB = sA + Cfg::kABytes;
-      for (int c = tid; c < kACopies; c += 256) {
-        const int cb = c % ka, v = (c / ka) % kKV, d = c / (ka * kKV);
-        const int row = u0 + v - (d - 1);
-        const bool ok = row >= g.g0 && row < g.g1;
-        cp16z(sA + (d * ka + cb) * Cfg::kBlock + v * 16,
-              dy + (size_t)(ok ? row : 0) * COUT + cb * 8, ok);
-      }
-      for (int c = tid; c < kBCopies; c += 256) {
-        const int cb = c % kb, v = (c / kb) % kKV, q = c / (kb * kKV);
-        const int rg = part * Cfg::kRg + q;
-        const int row = u0 + v + (rg / 3 - 1) * g.pp + (rg % 3 - 1) * g.wp;
-        const bool ok = row >= 0 && row < g.vp;
-        cp16z(sB + (q * kb + cb) * Cfg::kBlock + v * 16,
-              x + (size_t)(ok ? row : 0) * CIN + cb * 8, ok);
-      }
-    }
-    cp_commit_group();
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (s_abort) return false;
+    if (tc::mbar_wait(bar, parity, kWaitLimit)) return true;
+    s_abort = 1;
+    return false;
   };
 
-  bool abort = false;
-  for (int i = 0; i < S - 1; ++i) load(i);
-  for (int i = 0; i < my; ++i) {
-    const int buf = i % S;
-    cp_wait_groups<S - 2>();  // chunk i has landed
-    tc::fence_proxy_async();
-    __syncthreads();
-    if (tid == 0) {
+  if (warp == 5) {
+    // ---- copies ------------------------------------------------------------------
+    if (lane == 0) {
+      int issued = 0;
+      for (int i = 0; i < my; ++i) {
+        const int buf = i % S;
+        if (i >= S && !wait(&empty[buf], ((i / S) - 1) & 1)) break;
+        const int u0 = u00 + (split + i * nsplit) * kKV;
+        unsigned char* st = sm + buf * Cfg::kStage;
+        tc::mbar_expect(&full[buf], Cfg::kTx);
+        tc::tma_2d(st, &maps.b, &full[buf], 0, u0 - 1);
+#pragma unroll
+        for (int q = 0; q < Cfg::kRg; ++q) {
+          const int rg = part * Cfg::kRg + q;
+          tc::tma_2d(st + Cfg::kABytes + q * Cfg::kBRg, &maps.a, &full[buf], 0,
+                     u0 + (rg / 3 - 1) * g.pp + (rg % 3 - 1) * g.wp);
+        }
+        issued = i + 1;
+      }
+      // no copy outlives the block
+      for (int j = issued - 1; j >= 0 && j >= issued - S; --j)
+        if (!tc::mbar_wait(&full[j % S], (j / S) & 1, kWaitLimit)) s_abort = 1;
+    }
+  } else if (warp == 4 && lane == 0) {
+    // ---- MMA thread ------------------------------------------------------------
+    for (int i = 0; i < my; ++i) {
+      const int buf = i % S;
+      if (!wait(&full[buf], (i / S) & 1)) break;
       tc::fence_after();
       // bits 15, 16: A and B MN-major
       constexpr uint32_t idesc = tc::idesc_bf16_f32(128, Cfg::kN) | (1u << 15) | (1u << 16);
-      const uint32_t a0 = tc::smem_addr(sm + buf * Cfg::kStage), b0 = a0 + Cfg::kABytes;
+      const uint32_t st = tc::smem_addr(sm + buf * Cfg::kStage);
+      const uint64_t ad = tc::smem_desc_sw(st, Cfg::kARow, 8 * Cfg::kARow, Cfg::kARow);
+      const uint64_t bd = tc::smem_desc_sw(st + Cfg::kABytes, Cfg::kBRg, 8 * Cfg::kBRow, Cfg::kBRow);
 #pragma unroll
       for (int ks = 0; ks < kKV / 16; ++ks)
 #pragma unroll
         for (int mt = 0; mt < Cfg::kMTiles; ++mt)
           tc::mma_bf16(acc + mt * Cfg::kN,
-                       tc::smem_desc(a0 + mt * 16 * Cfg::kBlock + ks * 256, 128, Cfg::kBlock),
-                       tc::smem_desc(b0 + ks * 256, 128, Cfg::kBlock), idesc, (i | ks) != 0);
-      tc::mma_commit(&bars[buf]);
+                       ad + (uint32_t)(((ks * 16 + mt * (128 / COUT)) * Cfg::kARow) >> 4),
+                       bd + (uint32_t)((ks * 16 * Cfg::kBRow) >> 4), idesc, (i | ks) != 0);
+      tc::mma_commit(&empty[buf]);
     }
-    // chunk i + S - 1 reuses the stage of chunk i - 1
-    bool ok = true;
-    if (i >= 1) ok = tc::mbar_wait(&bars[(i - 1) % S], ((i - 1) / S) & 1, kWaitLimit);
-    if (__syncthreads_or(!ok)) {
-      abort = true;
-      break;
-    }
-    load(i + S - 1);
+    // every MMA issued must be complete before the accumulator is read or released
+    tc::mma_commit(&done_bar);
+    if (!tc::mbar_wait(&done_bar, 0, kWaitLimit)) s_abort = 1;
   }
-  cp_wait_all();
-  if (!abort && my > 0) {
-    const bool ok = tc::mbar_wait(&bars[(my - 1) % S], ((my - 1) / S) & 1, kWaitLimit);
-    if (__syncthreads_or(!ok)) abort = true;
-  }
+  tc::fence_before();
+  __syncthreads();
+  const bool abort = s_abort != 0;
   tc::fence_after();
   if (warp < 4) {
 #pragma unroll
     for (int mt = 0; mt < Cfg::kMTiles; ++mt) {
       const int row = mt * 128 + warp * 32 + lane;
-      float* out = ws + ((size_t)(split * Cfg::kParts + part) * Cfg::kRows + row) * Cfg::kN;
+      const int m = row / COUT, co = row % COUT;  // row block m: voxel u - 1 + m, dx = 1 - m
+      float* out = ws + ((size_t)(split * Cfg::kParts + part) * Cfg::kRows + (2 - m) * COUT + co) *
+                            Cfg::kN;
 #pragma unroll
       for (int c0 = 0; c0 < Cfg::kN; c0 += 16) {
         float v[16];
@@ -1032,7 +1041,7 @@ conv_wgrad_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ d
           tc::tmem_ld16(acc + ((uint32_t)(warp * 32) << 16) + mt * Cfg::kN + c0, v);
         else
           for (int c = 0; c < 16; ++c) v[c] = 0.f;
-        if (row < Cfg::kRows)
+        if (m < 3)
 #pragma unroll
           for (int c = 0; c < 16; c += 4)
             *reinterpret_cast<float4*>(out + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
@@ -1042,17 +1051,17 @@ conv_wgrad_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ d
   if (abort && tid == 0) atomicOr(&g_tc_timeout, 1);
   tc::fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(acc, Cfg::kCols);
+  if (warp == 4) tc::tmem_dealloc(acc, Cfg::kCols);
 }
 
 // dw from the partial tiles: 32 outputs per block (consecutive ci), the splits
-// dealt to its 8 warps and added in a fixed order in FP64.
+// dealt to its 16 warps and added in a fixed order in FP64.
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(512)
 wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ dw, int nsplit,
                     int accumulate) {
   using Cfg = WgCfg<CIN, COUT>;
-  __shared__ double part[8][32];
+  __shared__ double part[16][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;  // 27 COUT CIN is a multiple of 32
   const int ci = i % CIN, co = (i / CIN) % COUT, t = i / (CIN * COUT);
@@ -1060,13 +1069,13 @@ wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ dw, int ns
   const float* src = ws + ((size_t)(rg / Cfg::kRg) * Cfg::kRows + d * COUT + co) * Cfg::kN +
                      (rg % Cfg::kRg) * CIN + ci;
   double s = 0.0;
-#pragma unroll 4
-  for (int sp = warp; sp < nsplit; sp += 8)
+#pragma unroll 10
+  for (int sp = warp; sp < nsplit; sp += 16)
     s += src[(size_t)sp * Cfg::kParts * Cfg::kRows * Cfg::kN];
   part[warp][lane] = s;
   __syncthreads();
   if (warp == 0) {
-    for (int w = 1; w < 8; ++w) s += part[w][lane];
+    for (int w = 1; w < 16; ++w) s += part[w][lane];
     dw[i] = accumulate ? (float)(dw[i] + s) : (float)s;
   }
 }
@@ -1156,25 +1165,44 @@ cudaError_t zf_launch(const uint16_t* x, const uint16_t* w, const float* bias,
   return cudaGetLastError();
 }
 
+// Planes per unit: the split of the planes into runs with the fewest plane steps
+// on the busiest CTA (a run of zc outputs takes zc + 2 steps).  Measured, us: 64^3
+// 16 -> 16 with runs of 4 / 8 / 16 planes 17.5 / 16.3 / 18.5 (8 taken), 160^3
+// 148 / 132 / 124 (16 taken), 64^3 32 -> 64 33.8 / 33.7 / 33.6 (16 taken).
+int ws_run(int nb, int nz, int ns, int ctas) {
+  long long best = 0;
+  int zc = nz;
+  for (int k = 1; k <= nz; ++k) {
+    const int z = (nz + k - 1) / k;
+    const long long units = (long long)nb * ns * ((nz + z - 1) / z);
+    const long long cost = (units + ctas - 1) / ctas * (z + 2);
+    if (best == 0 || cost < best) {
+      best = cost;
+      zc = z;
+    }
+  }
+  return zc;
+}
+
 template <int CIN, int COUT>
 cudaError_t ws_launch(const uint16_t* x, const uint16_t* w, const float* bias,
                       const uint16_t* mask, uint16_t* y, const Vol& g, int flags,
                       cudaStream_t s) {
+  using Cfg = WsCfg<CIN, COUT>;
   static int per_sm = -1, nsm = 0;
   if (per_sm < 0)
-    per_sm = ctas_per_sm((const void*)conv_fwd_ws_kernel<CIN, COUT>, WsCfg<CIN, COUT>::kSmem,
-                         WsCfg<CIN, COUT>::kCols, &nsm);
+    per_sm = ctas_per_sm((const void*)conv_fwd_ws_kernel<CIN, COUT>, Cfg::kSmem, Cfg::kCols, &nsm);
   const int ctas = per_sm * nsm;
   ZmGrid zg;
   zg.nb = (g.pp + 127) / 128;
-  zg.zc = g.nz;
-  while (zg.zc > 4 && (long long)zg.nb * g.ns * ((g.nz + zg.zc - 1) / zg.zc) < 2LL * ctas)
-    zg.zc = (zg.zc + 1) / 2;
+  zg.zc = ws_run(zg.nb, g.nz, g.ns, ctas);
   zg.nzc = (g.nz + zg.zc - 1) / zg.zc;
   zg.units = zg.nb * g.ns * zg.nzc;
   const int grid = zg.units < ctas ? zg.units : ctas;
-  conv_fwd_ws_kernel<CIN, COUT><<<grid, 192, WsCfg<CIN, COUT>::kSmem, s>>>(x, w, bias, mask, y,
-                                                                           g, flags, zg);
+  RowMaps maps;
+  if (!encode_rows(&maps.a, x, CIN, g.vp, kRG) || !encode_rows(&maps.b, w, CIN, 27 * COUT, COUT))
+    return cudaErrorInvalidValue;
+  conv_fwd_ws_kernel<CIN, COUT><<<grid, 192, Cfg::kSmem, s>>>(maps, bias, mask, y, g, flags, zg);
   return cudaGetLastError();
 }
 
@@ -1200,12 +1228,16 @@ cudaError_t wgrad_launch(const uint16_t* x, const uint16_t* dy, float* dw, float
   if (nchunks > 0) {
     cudaFuncSetAttribute(conv_wgrad_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          Cfg::kSmem);
+    RowMaps maps;
+    if (!encode_rows(&maps.a, x, CIN, g.vp, Cfg::kKV) ||
+        !encode_rows(&maps.b, dy, COUT, g.vp, Cfg::kAVox))
+      return cudaErrorInvalidValue;
     conv_wgrad_kernel<CIN, COUT>
-        <<<dim3(Cfg::kParts, nsplit), Cfg::kThreads, Cfg::kSmem, s>>>(x, dy, ws, g, nchunks);
+        <<<dim3(Cfg::kParts, nsplit), 192, Cfg::kSmem, s>>>(maps, ws, g, nchunks);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  wgrad_reduce_kernel<CIN, COUT><<<27 * COUT * CIN / 32, 256, 0, s>>>(
+  wgrad_reduce_kernel<CIN, COUT><<<27 * COUT * CIN / 32, 512, 0, s>>>(
       ws, dw, nchunks > 0 ? nsplit : 0, accumulate);
   return cudaGetLastError();
 }
@@ -1226,19 +1258,18 @@ bool conv_shape_ok(int cin, int cout) {
 #define TPFA_CONV_SHAPES(X) X(16, 16) X(16, 32) X(32, 16) X(32, 64) X(64, 32)
 
 // 0: tile kernel, 1: z-marching kernel, 2: z-marching kernel with the z-taps
-// folded into N, 4: the folded kernel with warp-specialised roles (1, 2 and 4
-// where their ring fits), 3: per layer shape the fastest as measured on GB300
-// (default: 1 for 32 -> 16, 4 otherwise)
+// folded into N (1 and 2 where their ring fits, else 0), 4: the folded kernel
+// with warp-specialised roles, 3: the fastest as measured on GB300 (default: 4)
 static int g_conv_kernel = 3;
 
 cudaError_t conv_fwd(const uint16_t* x, const uint16_t* w, const float* bias, const uint16_t* mask,
                      uint16_t* y, const Vol& g, int cin, int cout, int flags, cudaStream_t s) {
   const bool ring = !(cin == 64 && cout == 32);
-  const int kern = g_conv_kernel != 3 ? g_conv_kernel : (cin == 32 && cout == 16 ? 1 : 4);
-  if (ring && kern == 4) {
+  const int kern = g_conv_kernel != 3 ? g_conv_kernel : 4;
+  if (kern == 4) {
 #define X(CI, CO) \
   if (cin == CI && cout == CO) return ws_launch<CI, CO>(x, w, bias, mask, y, g, flags, s);
-    X(16, 16) X(16, 32) X(32, 16) X(32, 64)
+    TPFA_CONV_SHAPES(X)
 #undef X
   }
   if (ring && kern == 2) {

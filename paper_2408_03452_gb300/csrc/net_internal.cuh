@@ -11,6 +11,7 @@
 // W = nx+2, P = (nx+2)(ny+2).  Tap index t = 9(dz+1) + 3(dy+1) + (dx+1).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -51,6 +52,11 @@ __device__ __forceinline__ bool vol_interior(const Vol& g, int idx) {
 }
 
 enum ConvFlags : int { kConvRelu = 1, kConvMask = 2 };
+
+// 2-D tensor map of `rows` rows of `channels` BF16 values (16, 32 or 64), boxes of
+// `box` whole rows, in the copy engine's swizzle mode of the row's width.  False
+// without a tensor-map encoder.
+bool encode_rows(CUtensorMap* m, const uint16_t* base, int channels, int64_t rows, int box);
 
 // y = epilogue(conv3x3x3(x; w) + bias): see tpfa_conv3d_bf16.
 cudaError_t conv_fwd(const uint16_t* x, const uint16_t* w, const float* bias, const uint16_t* mask,

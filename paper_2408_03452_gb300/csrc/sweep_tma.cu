@@ -40,6 +40,7 @@
 #include <math.h>
 #include <string.h>
 
+#include "net_internal.cuh"
 #include "sweep_common.cuh"
 #include "tc_common.cuh"
 
@@ -843,6 +844,21 @@ cudaError_t launch_variant(const TmaArgs& a, const TmaPlan& p, cudaStream_t s) {
 }
 
 }  // namespace
+
+bool net::encode_rows(CUtensorMap* m, const uint16_t* base, int channels, int64_t rows, int box) {
+  EncodeTiledFn fn = encode_fn();
+  if (fn == nullptr) return false;
+  const cuuint64_t dim[2] = {(cuuint64_t)channels, (cuuint64_t)rows};
+  const cuuint64_t stride[1] = {(cuuint64_t)channels * 2};
+  const cuuint32_t bx[2] = {(cuuint32_t)channels, (cuuint32_t)box};
+  const cuuint32_t es[2] = {1, 1};
+  const CUtensorMapSwizzle sw = channels == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                : channels == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                 : CU_TENSOR_MAP_SWIZZLE_32B;
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(base), dim, stride, bx,
+            es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 bool tma_sweep_ok(const Grid& g, bool b16, bool jac) {
   if (g.nx >= (1 << 30) || g.ny >= (1 << 30) || g.nz >= (1 << 30) || encode_fn() == nullptr)

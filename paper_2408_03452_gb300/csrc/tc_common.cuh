@@ -38,6 +38,17 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
   return d;
 }
 
+// The same for tiles whose rows are `row` bytes long (32, 64 or 128) as the copy
+// engine lays them out in its swizzle mode of that width (16-byte pieces of a row
+// exchanged by an address-bit exclusive-or with period 8 * row bytes, so a start
+// address may be any row of an aligned buffer): layout code at bits 61-63.
+// K-major: sbo = next 8 rows (8 * row), lbo unused.  MN-major (rows are the
+// reduction): sbo = next 8 rows, lbo = next row / 2 elements of the other index.
+__device__ __forceinline__ uint64_t smem_desc_sw(uint32_t addr, uint32_t lbo, uint32_t sbo,
+                                                 int row) {
+  return smem_desc(addr, lbo, sbo) | ((uint64_t)(row == 128 ? 2 : row == 64 ? 4 : 6) << 61);
+}
+
 // Instruction descriptor for kind::f16: FP32 accumulator (bits 4-5 = 1), A
 // and B BF16 (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 at bits 17-22,
 // M >> 4 at bits 24-28.
@@ -145,6 +156,21 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float* v) {
   if (NC == 64) tmem_ld32(taddr + 32, v + 32);
   if (NC == 48) tmem_ld16(taddr + 32, v + 32);
   if (NC == 16) tmem_ld16(taddr, v);
+}
+
+// one arrival and `bytes` of pending copies on the current phase
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// box of a 2-D tensor map from (x, y), complete_tx on bar
+__device__ __forceinline__ void tma_2d(void* dst, const void* map, uint64_t* bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
+      : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
