@@ -243,7 +243,8 @@ struct ZmCfg {
 };
 
 struct ZmGrid {
-  int nb;   // 128-voxel segments per padded plane
+  int nb;   // 128-voxel segments (or tiles, nbx of them along x) per plane
+  int nbx;
   int zc;   // interior planes per unit
   int nzc;  // units per sample along z
   int units;
@@ -653,14 +654,15 @@ conv_fwd_zf_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
 }
 
 // ---- the folded z-marching kernel with warp-specialised roles -------------
-// Same work units, folded MMAs (N = 3 cout) and TMEM ring of accumulators as
-// conv_fwd_zf_kernel, with the three kinds of work on warps of their own:
-//   warp 5 (one thread) copies row-group triples into a ring of ST slots: one
-//          tensor-map copy of 130 voxels per row group, voxels outside the volume
-//          filled with zeros, and before them the 27 weight matrices;
-//   warp 4 (one thread) issues the MMAs of a triple once it is full and the
-//          slot of the output it starts is free, and commits to the triple's
-//          "empty" barrier and to the "full" barrier of the output the triple
+// Folded MMAs (N = 3 cout) and TMEM ring of accumulators as in
+// conv_fwd_zf_kernel, over tiles of 8 x 16 voxels (x, y) followed through zc
+// planes, with the three kinds of work on warps of their own:
+//   warp 5 (one thread) copies the tile's input planes, 10 x 18 voxels with their
+//          halo, into a ring of ST slots (one tensor-map copy each, voxels outside
+//          the volume filled with zeros), and before them the 27 weight matrices;
+//   warp 4 (one elected lane) issues the MMAs of a plane once it is full and the
+//          slot of the output it starts is free, and commits to the plane's
+//          "empty" barrier and to the "full" barrier of the output the plane
 //          completes;
 //   warps 0-3 (the four TMEM lane quarters) drain finished accumulators:
 //          load, release the slot ("empty"), then bias / ReLU / mask, BF16
@@ -669,22 +671,27 @@ conv_fwd_zf_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ 
 // every role checks, and the kernel records the timeout like the others.
 //
 // Voxels stay whole rows of cin channels in shared memory, in the copy engine's
-// swizzle of that width, which the tensor core reads directly: a tap is the row
-// group started dx rows later.  A layout of 8-channel blocks, which needs no
-// swizzle, has to be filled 16 bytes at a time: its copies, not the MMAs, set the
-// time (1,700 cycles per plane step and SM for 16 -> 16 against 400 for
-// the nine MMAs, each 32 + N / 4 cycles).
-// WSFIGURES
+// swizzle of that width, which the tensor core reads directly: operand row m is
+// voxel (m % 8, m / 8) of the tile (row groups of 8 voxels, 10 rows apart), and a
+// tap is the same rows started (dy, dx) later.
+// Small volumes are bound by launch and pipeline fill (16^3: 5.6 us), larger ones
+// by the one warp that issues the MMAs (each runs 32 + N / 4 cycles and takes
+// longer than that to issue) and by the voxel rows copied: a linear run of 128
+// voxels needs three runs of 130, this tile 180 rows.  16 -> 16, us: 64^3 21.8 in
+// 8-channel blocks filled 16 bytes at a time, 16.3 with linear runs of whole
+// rows, 14.4 now; 160^3 197, 129, 104 (350 TFLOP/s); 64 -> 32 at 64^3 160 -> 35.
 template <int CIN, int COUT>
 struct WsCfg {
+  static constexpr int kTX = 8, kTY = 16;
   static constexpr int kRow = CIN * 2;
+  static constexpr int kPitch = (kTX + 2) * kRow;              // next row of the tile
   static constexpr int kWTap = COUT * kRow;
   static constexpr int kWBytes = 27 * kWTap;
-  static constexpr int kRGBytes = (kRG * kRow + 1023) / 1024 * 1024;
-  static constexpr int kTriple = 3 * kRGBytes;
-  // two CTAs per SM where two rings of three or more slots fit, else one
-  static constexpr int kST = CIN == 64 ? 2 : COUT == 64 ? 4 : CIN == 32 ? 3 : COUT == 32 ? 5 : 6;
-  static constexpr int kSmem = kWBytes + kST * kTriple + 1024;
+  static constexpr int kTx = (kTY + 2) * kPitch;               // bytes of one plane
+  static constexpr int kPlane = (kTx + 1023) / 1024 * 1024;
+  // two CTAs per SM where the weights leave room, else one
+  static constexpr int kST = CIN == 64 ? 4 : COUT == 64 ? 8 : CIN == 32 ? 6 : 10;
+  static constexpr int kSmem = kWBytes + kST * kPlane + 1024;
   static constexpr int kR = 256 / COUT;
   static constexpr uint32_t kCols = 256;
   static_assert(kSmem <= 227 * 1024, "shared memory");
@@ -714,7 +721,7 @@ conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict
   __shared__ volatile int s_abort;
   unsigned char* sR = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char* sW = sR + ST * Cfg::kTriple;
+  unsigned char* sW = sR + ST * Cfg::kPlane;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid < COUT) sbias[tid] = bias ? bias[tid] : 0.f;
@@ -755,105 +762,104 @@ conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict
       int tg = 0;
       for (int u = blockIdx.x; u < zg.units && !s_abort; u += gridDim.x) {
         const int bi = u % zg.nb, cz = u / zg.nb;
-        const int sidx = cz / zg.nzc;
         const int z0 = (cz % zg.nzc) * zg.zc;
         const int nout = min(zg.zc, g.nz - z0);
-        const int kp0 = sidx * g.dp + 1 + z0;
-        const int seg = bi * 128;
+        const int p0 = cz / zg.nzc * g.dp + z0;  // padded plane of the first input plane
+        const int x0 = bi % zg.nbx * Cfg::kTX, y0 = bi / zg.nbx * Cfg::kTY;  // padded corner
         bool stop = false;
         for (int j = 0; j < nout + 2; ++j, ++tg) {
           const int s = tg % ST;
           if (tg >= ST && !wait(&tempty[s], ((tg / ST) - 1) & 1)) { stop = true; break; }
-          const int base = seg + (kp0 - 1 + j) * g.pp - g.wp - 1;  // first row of the triple
-          unsigned char* st = sR + s * Cfg::kTriple;
-          tc::mbar_expect(&tfull[s], 3 * kRG * Cfg::kRow);
-#pragma unroll
-          for (int gi = 0; gi < 3; ++gi)
-            tc::tma_2d(st + gi * Cfg::kRGBytes, &maps.a, &tfull[s], 0, base + gi * g.wp);
+          tc::mbar_expect(&tfull[s], Cfg::kTx);
+          tc::tma_4d(sR + s * Cfg::kPlane, &maps.a, &tfull[s], 0, x0, y0, p0 + j);
         }
         if (stop) break;
       }
-      // no copy outlives the block: wait for the last (up to ST) triples and the weights
+      // no copy outlives the block: wait for the last (up to ST) planes and the weights
       tc::mbar_wait(&wfull, 0, kWaitLimit);
       for (int j = tg - 1; j >= 0 && j >= tg - ST; --j)
         if (!tc::mbar_wait(&tfull[j % ST], (j / ST) & 1, kWaitLimit)) s_abort = 1;
     }
   } else if (warp == 4) {
-    // ---- MMA thread --------------------------------------------------------
-    if (lane == 0) {
-      const uint64_t adesc0 = tc::smem_desc_sw(tc::smem_addr(sR), 16, 8 * Cfg::kRow, Cfg::kRow);
-      const uint64_t bdesc0 = tc::smem_desc_sw(tc::smem_addr(sW), 16, 8 * Cfg::kRow, Cfg::kRow);
-      int tg = 0, obase = 0;
-      bool stop = !wait(&wfull, 0);
-      for (int u = blockIdx.x; u < zg.units && !stop; u += gridDim.x) {
-        const int cz = u / zg.nb;
-        const int z0 = (cz % zg.nzc) * zg.zc;
-        const int nout = min(zg.zc, g.nz - z0);
-        for (int j = 0; j < nout + 2; ++j, ++tg) {
-          const int s = tg % ST;
-          if (!wait(&tfull[s], (tg / ST) & 1)) { stop = true; break; }
-          const int klo = max(0, j - 2), khi = min(nout - 1, j);
-          if (khi == j) {  // output j starts here: its accumulator slot must be free
-            const int oc = obase + j;
-            if (oc >= R && !wait(&aempty[oc % R], ((oc / R) - 1) & 1)) { stop = true; break; }
-          }
-          tc::fence_after();
-          // Accumulator slots, instruction descriptors and operand addresses of
-          // the triple are the same for its 9 (dy, dx) x CIN / 16 steps up to
-          // constants, and formed once.
-          const int sl = (obase + klo) % R;
-          const int n1 = min(khi - klo + 1, R - sl), n2 = khi - klo + 1 - n1;
-          const uint32_t d1 = acc0 + (uint32_t)(sl * COUT);
-          const uint32_t i1 = tc::idesc_bf16_f32(128, n1 * COUT);
-          const uint32_t i2 = tc::idesc_bf16_f32(128, n2 * COUT);
-          const uint64_t a0 = adesc0 + (uint32_t)(s * (Cfg::kTriple >> 4));
-          const uint64_t b1 = bdesc0 + (uint32_t)((2 - j + klo) * (Cfg::kWTap >> 4));
-          const uint64_t b2 = b1 + (uint32_t)(n1 * (Cfg::kWTap >> 4));
-          // first step: output j starts with it, the outputs before j go on
-          if (khi == j) {
-            for (int k = klo; k <= j; ++k)
-              tc::mma_bf16(acc0 + (uint32_t)(((obase + k) % R) * COUT), a0,
-                           b1 + (uint32_t)((k - klo) * (Cfg::kWTap >> 4)),
-                           tc::idesc_bf16_f32(128, COUT), k < j);
-          } else {
-            tc::mma_bf16(d1, a0, b1, i1, true);
-            if (n2 > 0) tc::mma_bf16(acc0, a0, b2, i2, true);
-          }
-          auto step = [&](int st, bool two) {
-            const int gd = st / (CIN / 16), ks = st % (CIN / 16);  // gd = 3 gi + dx
-            const uint32_t ao = (gd / 3 * Cfg::kRGBytes + gd % 3 * Cfg::kRow + ks * 32) >> 4;
-            const uint32_t bo = (gd * 3 * Cfg::kWTap + ks * 32) >> 4;
-            tc::mma_bf16(d1, a0 + ao, b1 + bo, i1, true);
-            if (two) tc::mma_bf16(acc0, a0 + ao, b2 + bo, i2, true);
-          };
-          if (n2 == 0) {
-#pragma unroll
-            for (int st = 1; st < 9 * (CIN / 16); ++st) step(st, false);
-          } else {
-#pragma unroll 1
-            for (int st = 1; st < 9 * (CIN / 16); ++st) step(st, true);
-          }
-          tc::mma_commit(&tempty[s]);
-          if (j >= 2) tc::mma_commit(&afull[(obase + j - 2) % R]);  // output j-2 is final
+    // ---- MMA warp (one elected lane issues; everything it needs is uniform) ----
+    const uint64_t adesc0 = tc::smem_desc_sw(tc::smem_addr(sR), 16, Cfg::kPitch, Cfg::kRow);
+    const uint64_t bdesc0 = tc::smem_desc_sw(tc::smem_addr(sW), 16, 8 * Cfg::kRow, Cfg::kRow);
+    const uint32_t accu = __shfl_sync(0xffffffffu, acc0, 0);
+    auto waitw = [&](uint64_t* bar, uint32_t parity) -> bool {
+      if (tc::mbar_wait_warp(bar, parity, kWaitLimit)) return true;
+      s_abort = 1;
+      return false;
+    };
+    int tg = 0, obase = 0;
+    bool stop = !waitw(&wfull, 0);
+    for (int u = blockIdx.x; u < zg.units && !stop; u += gridDim.x) {
+      const int cz = u / zg.nb;
+      const int z0 = (cz % zg.nzc) * zg.zc;
+      const int nout = min(zg.zc, g.nz - z0);
+      for (int j = 0; j < nout + 2; ++j, ++tg) {
+        const int s = tg % ST;
+        if (!waitw(&tfull[s], (tg / ST) & 1)) { stop = true; break; }
+        const int klo = max(0, j - 2), khi = min(nout - 1, j);
+        if (khi == j) {  // output j starts here: its accumulator slot must be free
+          const int oc = obase + j;
+          if (oc >= R && !waitw(&aempty[oc % R], ((oc / R) - 1) & 1)) { stop = true; break; }
         }
-        obase += nout;
+        tc::fence_after();
+        // Accumulator slots, instruction descriptors and operand addresses of
+        // the plane are the same for its 9 (dy, dx) x CIN / 16 steps up to
+        // constants, and formed once.
+        const int sl = (obase + klo) % R;
+        const int n1 = min(khi - klo + 1, R - sl), n2 = khi - klo + 1 - n1;
+        const uint32_t d1 = accu + (uint32_t)(sl * COUT);
+        const uint32_t i1 = tc::idesc_bf16_f32(128, n1 * COUT);
+        const uint32_t i2 = tc::idesc_bf16_f32(128, n2 * COUT);
+        const uint64_t a0 = adesc0 + (uint32_t)(s * (Cfg::kPlane >> 4));
+        const uint64_t b1 = bdesc0 + (uint32_t)((2 - j + klo) * (Cfg::kWTap >> 4));
+        const uint64_t b2 = b1 + (uint32_t)(n1 * (Cfg::kWTap >> 4));
+        // first step: output j starts with it, the outputs before j go on
+        if (khi == j) {
+          for (int k = klo; k <= j; ++k)
+            tc::mma_bf16_warp(accu + (uint32_t)(((obase + k) % R) * COUT), a0,
+                              b1 + (uint32_t)((k - klo) * (Cfg::kWTap >> 4)),
+                              tc::idesc_bf16_f32(128, COUT), k < j);
+        } else {
+          tc::mma_bf16_warp(d1, a0, b1, i1, true);
+          if (n2 > 0) tc::mma_bf16_warp(accu, a0, b2, i2, true);
+        }
+        auto step = [&](int st, bool two) {
+          const int gd = st / (CIN / 16), ks = st % (CIN / 16);  // gd = 3 gi + dx
+          const uint32_t ao = (gd / 3 * Cfg::kPitch + gd % 3 * Cfg::kRow + ks * 32) >> 4;
+          const uint32_t bo = (gd * 3 * Cfg::kWTap + ks * 32) >> 4;
+          tc::mma_bf16_warp(d1, a0 + ao, b1 + bo, i1, true);
+          if (two) tc::mma_bf16_warp(accu, a0 + ao, b2 + bo, i2, true);
+        };
+        if (n2 == 0) {
+#pragma unroll
+          for (int st = 1; st < 9 * (CIN / 16); ++st) step(st, false);
+        } else {
+#pragma unroll 1
+          for (int st = 1; st < 9 * (CIN / 16); ++st) step(st, true);
+        }
+        tc::mma_commit_warp(&tempty[s]);
+        if (j >= 2) tc::mma_commit_warp(&afull[(obase + j - 2) % R]);  // output j-2 is final
       }
-      // every MMA issued must be complete before the TMEM is released
-      tc::mma_commit(&done_bar);
-      if (!tc::mbar_wait(&done_bar, 0, kWaitLimit)) s_abort = 1;
+      obase += nout;
     }
+    // every MMA issued must be complete before the TMEM is released
+    tc::mma_commit_warp(&done_bar);
+    if (!tc::mbar_wait_warp(&done_bar, 0, kWaitLimit)) s_abort = 1;
   } else {
     // ---- epilogue warps 0-3: TMEM lanes 32 warp .. 32 warp + 31 -------------
     int obase = 0;
     for (int u = blockIdx.x; u < zg.units && !s_abort; u += gridDim.x) {
       const int bi = u % zg.nb, cz = u / zg.nb;
-      const int sidx = cz / zg.nzc;
       const int z0 = (cz % zg.nzc) * zg.zc;
       const int nout = min(zg.zc, g.nz - z0);
-      const int kp0 = sidx * g.dp + 1 + z0;
-      const int poff = bi * 128 + warp * 32 + lane;
-      const int px = poff % g.wp, py = poff / g.wp;
-      const bool in_xy = poff < g.pp && px >= 1 && px <= g.nx && py >= 1 && py <= g.ny;
+      const int kp0 = cz / zg.nzc * g.dp + 1 + z0;  // padded plane of output 0
+      const int vx = bi % zg.nbx * Cfg::kTX + (lane & 7);
+      const int vy = bi / zg.nbx * Cfg::kTY + warp * 4 + (lane >> 3);
+      const int poff = (vy + 1) * g.wp + vx + 1;
+      const bool in_xy = vx < g.nx && vy < g.ny;
       bool stop = false;
       for (int k = 0; k < nout; ++k) {
         const int oc = obase + k;
@@ -913,7 +919,10 @@ conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict
 // computed and ignored.
 // CTAs split the voxel range, write FP32 partial tiles, and a second kernel adds
 // the partials in a fixed order.
-// WGFIGURES
+// 16 -> 32 on 16 samples of 32^3 (GB300): 41 us (bound by the
+// copies: 648 voxel rows per 64 voxels) and
+// 12 us for the sum of the partials; 1,008 and 15 us when 8 x 8 blocks went through
+// movmatrix.
 template <int CIN, int COUT>
 struct WgCfg {
   static constexpr int kKV = 64;                   // voxels per stage
@@ -999,11 +1008,15 @@ conv_wgrad_kernel(const __grid_constant__ RowMaps maps, float* __restrict__ ws, 
       for (int j = issued - 1; j >= 0 && j >= issued - S; --j)
         if (!tc::mbar_wait(&full[j % S], (j / S) & 1, kWaitLimit)) s_abort = 1;
     }
-  } else if (warp == 4 && lane == 0) {
-    // ---- MMA thread ------------------------------------------------------------
+  } else if (warp == 4) {
+    // ---- MMA warp (one elected lane issues) ------------------------------------
+    const uint32_t accu = __shfl_sync(0xffffffffu, acc, 0);
     for (int i = 0; i < my; ++i) {
       const int buf = i % S;
-      if (!wait(&full[buf], (i / S) & 1)) break;
+      if (!tc::mbar_wait_warp(&full[buf], (i / S) & 1, kWaitLimit)) {
+        s_abort = 1;
+        break;
+      }
       tc::fence_after();
       // bits 15, 16: A and B MN-major
       constexpr uint32_t idesc = tc::idesc_bf16_f32(128, Cfg::kN) | (1u << 15) | (1u << 16);
@@ -1014,14 +1027,14 @@ conv_wgrad_kernel(const __grid_constant__ RowMaps maps, float* __restrict__ ws, 
       for (int ks = 0; ks < kKV / 16; ++ks)
 #pragma unroll
         for (int mt = 0; mt < Cfg::kMTiles; ++mt)
-          tc::mma_bf16(acc + mt * Cfg::kN,
-                       ad + (uint32_t)(((ks * 16 + mt * (128 / COUT)) * Cfg::kARow) >> 4),
-                       bd + (uint32_t)((ks * 16 * Cfg::kBRow) >> 4), idesc, (i | ks) != 0);
-      tc::mma_commit(&empty[buf]);
+          tc::mma_bf16_warp(accu + mt * Cfg::kN,
+                            ad + (uint32_t)(((ks * 16 + mt * (128 / COUT)) * Cfg::kARow) >> 4),
+                            bd + (uint32_t)((ks * 16 * Cfg::kBRow) >> 4), idesc, (i | ks) != 0);
+      tc::mma_commit_warp(&empty[buf]);
     }
     // every MMA issued must be complete before the accumulator is read or released
-    tc::mma_commit(&done_bar);
-    if (!tc::mbar_wait(&done_bar, 0, kWaitLimit)) s_abort = 1;
+    tc::mma_commit_warp(&done_bar);
+    if (!tc::mbar_wait_warp(&done_bar, 0, kWaitLimit)) s_abort = 1;
   }
   tc::fence_before();
   __syncthreads();
@@ -1129,6 +1142,7 @@ cudaError_t zm_launch(const uint16_t* x, const uint16_t* w, const float* bias,
                          ZmCfg<CIN, COUT>::kCols, &nsm);
   const int ctas = per_sm * nsm;
   ZmGrid zg;
+  zg.nbx = 0;
   zg.nb = (g.pp + 127) / 128;
   zg.zc = g.nz;
   // shorter z runs until there are at least two units per resident CTA
@@ -1152,6 +1166,7 @@ cudaError_t zf_launch(const uint16_t* x, const uint16_t* w, const float* bias,
                          ZfCfg<CIN, COUT>::kCols, &nsm);
   const int ctas = per_sm * nsm;
   ZmGrid zg;
+  zg.nbx = 0;
   zg.nb = (g.pp + 127) / 128;
   zg.zc = g.nz;
   // shorter z runs until there are at least two units per resident CTA
@@ -1168,7 +1183,8 @@ cudaError_t zf_launch(const uint16_t* x, const uint16_t* w, const float* bias,
 // Planes per unit: the split of the planes into runs with the fewest plane steps
 // on the busiest CTA (a run of zc outputs takes zc + 2 steps).  Measured, us: 64^3
 // 16 -> 16 with runs of 4 / 8 / 16 planes 17.5 / 16.3 / 18.5 (8 taken), 160^3
-// 148 / 132 / 124 (16 taken), 64^3 32 -> 64 33.8 / 33.7 / 33.6 (16 taken).
+// 148 / 132 / 124 (16 taken), 64^3 32 -> 64 33.8 / 33.7 / 33.6 (16 taken; linear
+// runs).
 int ws_run(int nb, int nz, int ns, int ctas) {
   long long best = 0;
   int zc = nz;
@@ -1194,13 +1210,15 @@ cudaError_t ws_launch(const uint16_t* x, const uint16_t* w, const float* bias,
     per_sm = ctas_per_sm((const void*)conv_fwd_ws_kernel<CIN, COUT>, Cfg::kSmem, Cfg::kCols, &nsm);
   const int ctas = per_sm * nsm;
   ZmGrid zg;
-  zg.nb = (g.pp + 127) / 128;
+  zg.nbx = (g.nx + Cfg::kTX - 1) / Cfg::kTX;
+  zg.nb = zg.nbx * ((g.ny + Cfg::kTY - 1) / Cfg::kTY);
   zg.zc = ws_run(zg.nb, g.nz, g.ns, ctas);
   zg.nzc = (g.nz + zg.zc - 1) / zg.zc;
   zg.units = zg.nb * g.ns * zg.nzc;
   const int grid = zg.units < ctas ? zg.units : ctas;
   RowMaps maps;
-  if (!encode_rows(&maps.a, x, CIN, g.vp, kRG) || !encode_rows(&maps.b, w, CIN, 27 * COUT, COUT))
+  if (!encode_volume(&maps.a, x, CIN, g, Cfg::kTX + 2, Cfg::kTY + 2) ||
+      !encode_rows(&maps.b, w, CIN, 27 * COUT, COUT))
     return cudaErrorInvalidValue;
   conv_fwd_ws_kernel<CIN, COUT><<<grid, 192, Cfg::kSmem, s>>>(maps, bias, mask, y, g, flags, zg);
   return cudaGetLastError();

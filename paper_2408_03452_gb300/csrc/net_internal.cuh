@@ -58,6 +58,11 @@ enum ConvFlags : int { kConvRelu = 1, kConvMask = 2 };
 // without a tensor-map encoder.
 bool encode_rows(CUtensorMap* m, const uint16_t* base, int channels, int64_t rows, int box);
 
+// The same for a haloed volume as a 4-D tensor (channels, x, y, plane), boxes of bx x
+// by voxels of one plane.
+bool encode_volume(CUtensorMap* m, const uint16_t* base, int channels, const Vol& g, int bx,
+                   int by);
+
 // y = epilogue(conv3x3x3(x; w) + bias): see tpfa_conv3d_bf16.
 cudaError_t conv_fwd(const uint16_t* x, const uint16_t* w, const float* bias, const uint16_t* mask,
                      uint16_t* y, const Vol& g, int cin, int cout, int flags, cudaStream_t s);

@@ -845,6 +845,12 @@ cudaError_t launch_variant(const TmaArgs& a, const TmaPlan& p, cudaStream_t s) {
 
 }  // namespace
 
+static CUtensorMapSwizzle row_swizzle(int channels) {
+  return channels == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+         : channels == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                          : CU_TENSOR_MAP_SWIZZLE_32B;
+}
+
 bool net::encode_rows(CUtensorMap* m, const uint16_t* base, int channels, int64_t rows, int box) {
   EncodeTiledFn fn = encode_fn();
   if (fn == nullptr) return false;
@@ -852,12 +858,24 @@ bool net::encode_rows(CUtensorMap* m, const uint16_t* base, int channels, int64_
   const cuuint64_t stride[1] = {(cuuint64_t)channels * 2};
   const cuuint32_t bx[2] = {(cuuint32_t)channels, (cuuint32_t)box};
   const cuuint32_t es[2] = {1, 1};
-  const CUtensorMapSwizzle sw = channels == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
-                                : channels == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                                 : CU_TENSOR_MAP_SWIZZLE_32B;
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(base), dim, stride, bx,
-            es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+            es, CU_TENSOR_MAP_INTERLEAVE_NONE, row_swizzle(channels),
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool net::encode_volume(CUtensorMap* m, const uint16_t* base, int channels, const Vol& g, int bx,
+                        int by) {
+  EncodeTiledFn fn = encode_fn();
+  if (fn == nullptr) return false;
+  const cuuint64_t row = (cuuint64_t)channels * 2;
+  const cuuint64_t dim[4] = {(cuuint64_t)channels, (cuuint64_t)g.wp, (cuuint64_t)g.hp,
+                             (cuuint64_t)g.dp * (cuuint64_t)g.ns};
+  const cuuint64_t stride[3] = {row, row * (cuuint64_t)g.wp, row * (cuuint64_t)g.pp};
+  const cuuint32_t box[4] = {(cuuint32_t)channels, (cuuint32_t)bx, (cuuint32_t)by, 1};
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t*>(base), dim, stride, box,
+            es, CU_TENSOR_MAP_INTERLEAVE_NONE, row_swizzle(channels),
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool tma_sweep_ok(const Grid& g, bool b16, bool jac) {
