@@ -51,6 +51,7 @@ struct tpfa_ctx {
   int loop_key_zc, loop_key_mode, loop_key_chunk, loop_key_sweep, loop_key_tile;
   unsigned long long* comm;  // exchange buffers of the resident CG (allocated on first use)
   size_t comm_words;
+  float2* packed;    // coefficients of the resident CG with tall bricks (on first use)
   int resident_off;  // the device refused a cooperative launch of this size
   TmaMaps* maps;     // tensor maps of the TMA-staged sweep (host copy, built with the loop)
   TmaPlan tplan;
@@ -484,6 +485,7 @@ int tpfa_destroy(tpfa_ctx* c) {
   if (c->r64) cudaFree(c->r64);
   if (c->dinv) cudaFree(c->dinv);
   if (c->comm) cudaFree(c->comm);
+  if (c->packed) cudaFree(c->packed);
   if (c->vec4) cudaFree(c->vec4);
   delete c->maps;
   if (c->partials) cudaFree(c->partials);
@@ -742,6 +744,12 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
   rc = ensure_r64(c);
   if (!rc) rc = resident ? ensure_comm(c, rp.words) : ensure_vectors(c);
   if (rc) return rc;
+  if (resident && rp.packed > 0 && c->packed == nullptr &&
+      cudaMalloc(&c->packed, rp.packed) != cudaSuccess) {
+    cudaGetLastError();
+    c->packed = nullptr;
+    return TPFA_ENOMEM;
+  }
   if (b16 && c->precond && c->dinv == nullptr) {
     if (cudaMalloc(&c->dinv, n * sizeof(float)) != cudaSuccess) {
       cudaGetLastError();
@@ -800,10 +808,10 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
         // launch waits for can need the lock
         std::lock_guard<std::mutex> lock(resident_mutex(c->device));
         CK(cudaEventRecord(c->ev[2], s));
-        const cudaError_t e =
-            launch_resident(make_res_prob(c->g, rp, coef, b16, c->dinv, c->r64, x, c->st, rtol,
-                                          (long long)(maxit - total_iters), c->comm),
-                            c->precond == 1, s);
+        ResProb prob = make_res_prob(c->g, rp, coef, b16, c->dinv, c->r64, x, c->st, rtol,
+                                     (long long)(maxit - total_iters), c->comm);
+        prob.packed = c->packed;
+        const cudaError_t e = launch_resident(prob, c->precond == 1, s);
         if (e == cudaErrorCooperativeLaunchTooLarge && outer == 0) {
           // fewer SMs than the device reports: this context keeps the sweeps
           cudaGetLastError();

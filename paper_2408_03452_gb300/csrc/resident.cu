@@ -121,13 +121,14 @@ struct ResShared {
 
 // the block's sums of four values, sent to every block and added up in a fixed
 // order; the neighbours' face words arrive in the same wait
-template <int CZ>
+// (NH: words a thread waits for; EARLY: first look before the sums are sent)
+template <int NH, bool EARLY>
 struct ResComm {
   uint2* part;
   const uint2* face;
   uint32_t* abort;
   int nblk, blk;
-  int hoff[5];  // face words this thread reads (index in one buffer), -1: none
+  int hoff[NH];  // face words this thread reads (index in one buffer), -1: none
   size_t face_buf;
 
   // warp-wide transposing sum of four pairs: lane l ends with value (l >> 3)
@@ -160,7 +161,7 @@ struct ResComm {
   // neighbours' face words.  The totals are there in warp 0 only.  Returns
   // false when the wait ran out (or another block gave up).
   __device__ __forceinline__ bool exchange(const Dfl (&mine)[4], uint32_t epoch, Dfl (&tot)[4],
-                                           float (&qh)[5], ResShared& sh) {
+                                           float (&qh)[NH], ResShared& sh) {
     auto& sA = sh.a;
     auto& sB = sh.b;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -175,16 +176,16 @@ struct ResComm {
     // while warp 0 sends the sums (64^3: 2.89 -> 2.66 us per iteration); with
     // tall ones the loads would only hold up those (128x128x64: 5.3 against 5.9)
     unsigned need = 0u;
-    uint2 f[5];
+    uint2 f[NH];
     auto look = [&]() {
 #pragma unroll
-      for (int j = 0; j < 5; ++j)
+      for (int j = 0; j < NH; ++j)
         if (hoff[j] >= 0) {
           need |= 1u << j;
           f[j] = ll_load(fb + hoff[j]);
         }
     };
-    if (CZ <= 8) look();
+    if (EARLY) look();
     if (warp == 0) {
       const Dfl t = warps16(sA);
       if (lane < 4) {
@@ -192,7 +193,7 @@ struct ResComm {
         ll_store(pb + ((size_t)blk * 4 + lane) * 2 + 1, t.l, epoch);
       }
     }
-    if (CZ > 8) look();
+    if (!EARLY) look();
     bool ok = true;
     uint32_t polls = 0;
     auto give_up = [&]() -> bool {
@@ -201,7 +202,7 @@ struct ResComm {
     };
     while (need != 0u) {
 #pragma unroll
-      for (int j = 0; j < 5; ++j)
+      for (int j = 0; j < NH; ++j)
         if (((need >> j) & 1u) && f[j].y == epoch) {
           qh[j] = __uint_as_float(f[j].x);
           need &= ~(1u << j);
@@ -211,7 +212,7 @@ struct ResComm {
         break;
       }
 #pragma unroll
-      for (int j = 0; j < 5; ++j)
+      for (int j = 0; j < NH; ++j)
         if ((need >> j) & 1u) f[j] = ll_load(fb + hoff[j]);
     }
     // the sums of every block: item = 4 block + value, in order
@@ -240,6 +241,110 @@ struct ResComm {
         tot[v] = {__shfl_sync(kFull, t.h, v), __shfl_sync(kFull, t.l, v)};
     }
     return true;
+  }
+};
+
+// Power-of-two scale of the operator: the largest D of the grid, from every
+// block's, scaled into [1, 2).
+__device__ __forceinline__ float operator_scale(const ResProb& a, int blk, float dmax,
+                                                uint32_t epoch, ResShared& sh, bool& fault) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto& sMax = sh.mx;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, o));
+  if (lane == 0) sMax[warp] = dmax;
+  __syncthreads();
+  for (int w = 0; w < kRW; ++w) dmax = fmaxf(dmax, sMax[w]);
+  uint2* pb = a.part + (size_t)(epoch & 1u) * a.nblk * 8;
+  if (tid == 0) ll_store(pb + (size_t)blk * 8, dmax, epoch);
+  uint32_t polls = 0;
+  for (int i = tid; i < a.nblk && !fault; i += kRT) {
+    for (;;) {
+      const uint2 v = ll_load(pb + (size_t)i * 8);
+      if (v.y == epoch) {
+        dmax = fmaxf(dmax, __uint_as_float(v.x));
+        break;
+      }
+      if ((++polls & 1023u) == 0u && (polls >= kPollLimit || *(volatile uint32_t*)a.abort != 0u)) {
+        fault = true;
+        break;
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, o));
+  if (lane == 0) sMax[warp] = dmax;
+  fault = __syncthreads_or(fault);
+  for (int w = 0; w < kRW; ++w) dmax = fmaxf(dmax, sMax[w]);
+  if (!(dmax > 0.f && isfinite(dmax))) return 1.f;
+  int e = ilogbf(dmax);
+  e = e > 120 ? 120 : (e < -120 ? -120 : e);
+  return exp2f((float)-e);
+}
+
+// Scalars of an iteration, kept by warp 0: alpha, beta and the stop test (as
+// cg_finish).
+struct ResScalars {
+  Dfl rho, rho0, thresh;
+  long long iter, sweeps;
+  float alpha, beta;
+  int done;
+
+  __device__ __forceinline__ void init() {
+    rho = rho0 = thresh = {0.f, 0.f};
+    iter = sweeps = 0;
+    alpha = beta = 0.f;
+    done = kRunning;
+  }
+  __device__ __forceinline__ void update(const Dfl (&tot)[4], double rtol2, long long maxit) {
+    rho = tot[0];
+    if (iter == 0) {
+      const float h = (float)rtol2, l = (float)(rtol2 - (double)h);
+      rho0 = rho;
+      thresh = df_add(df_mulf(rho0, h), df_mulf(rho0, l));
+    }
+    // alpha is the FP32 step the vectors take, so that rho - 2 alpha r'q +
+    // alpha^2 q'q is the norm of the residual it leaves
+    const float al = quot(rho.h, tot[1].h);
+    const Dfl u = df_mulf(tot[3], al);
+    const Dfl v = df_mulf(df_add({2.f * tot[2].h, 2.f * tot[2].l}, {-u.h, -u.l}), al);
+    Dfl rn = df_add(rho, {-v.h, -v.l});
+    if (rn.h < 0.f) rn = {0.f, 0.f};
+    alpha = al;
+    beta = quot(rn.h, rho.h);
+    // 0 unless one of the sums is infinite or NaN
+    const float bad = fmaf(tot[0].h, 0.f, fmaf(tot[1].h, 0.f, fmaf(tot[2].h, 0.f, tot[3].h * 0.f)));
+    const bool stay = bad == 0.f && tot[1].h > 0.f && !df_le(rho, thresh);
+    ++iter;
+    if (!stay || df_le(rn, thresh) || iter >= maxit || ++sweeps > 2 * maxit + 64) {
+      done = stay ? (df_le(rn, thresh) ? kConvEst : iter >= maxit ? kMaxit : kGuard)
+                  : (bad != 0.f ? kNonFinite : df_le(rho, thresh) ? kConvTrue : kBreakdown);
+      if (!stay) {
+        alpha = 0.f;
+        --iter;
+      }
+    }
+  }
+  // after the last step: the true r'r of the residual it leaves; if the estimate
+  // that stopped the loop was too optimistic, go on with the exact continuation
+  __device__ __forceinline__ void finish(const Dfl (&tot)[4], long long maxit) {
+    const Dfl prev = rho;
+    rho = tot[0];
+    if (done == kConvEst && !df_le(rho, thresh) && iter < maxit && isfinite(rho.h) && prev.h > 0.f) {
+      beta = quot(rho.h, prev.h);
+      done = kRunning;
+    }
+    alpha = 0.f;
+  }
+  __device__ __forceinline__ void report(CgState* st, double scale, bool fault) const {
+    st->rho = (double)rho.h + (double)rho.l;
+    st->rho0 = (double)rho0.h + (double)rho0.l;
+    st->scale = scale;
+    st->iter = iter;
+    st->launches = 1;
+    st->done = fault ? (int)kGuard : done;
+    st->fault = fault ? 1 : 0;
   }
 };
 
@@ -304,7 +409,7 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
   }
   for (int i = tid; i < CZ * (kRW + 2) * 34; i += kRT) sP[i] = 0.f;
 
-  ResComm<CZ> cm;
+  ResComm<5, (CZ <= 8)> cm;
   cm.part = a.part;
   cm.face = a.face;
   cm.abort = a.abort;
@@ -355,47 +460,9 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     x[k] = 0.f;
   }
 
-  // ---- power-of-two scale of the operator: the largest D of the grid ----------
   uint32_t epoch = *(volatile uint32_t*)a.ctl;
   bool fault = false;
-  float tscale = 1.f;
-  {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, o));
-    auto& sMax = sh.mx;
-    if (lane == 0) sMax[warp] = dmax;
-    __syncthreads();
-    for (int w = 0; w < kRW; ++w) dmax = fmaxf(dmax, sMax[w]);
-    ++epoch;
-    uint2* pb = a.part + (size_t)(epoch & 1u) * a.nblk * 8;
-    if (tid == 0) ll_store(pb + (size_t)blk * 8, dmax, epoch);
-    uint32_t polls = 0;
-    for (int i = tid; i < a.nblk && !fault; i += kRT) {
-      for (;;) {
-        const uint2 v = ll_load(pb + (size_t)i * 8);
-        if (v.y == epoch) {
-          dmax = fmaxf(dmax, __uint_as_float(v.x));
-          break;
-        }
-        if ((++polls & 1023u) == 0u &&
-            (polls >= kPollLimit || *(volatile uint32_t*)a.abort != 0u)) {
-          fault = true;
-          break;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, o));
-    if (lane == 0) sMax[warp] = dmax;
-    fault = __syncthreads_or(fault);
-    for (int w = 0; w < kRW; ++w) dmax = fmaxf(dmax, sMax[w]);
-    if (dmax > 0.f && isfinite(dmax)) {
-      int e = ilogbf(dmax);
-      e = e > 120 ? 120 : (e < -120 ? -120 : e);
-      tscale = exp2f((float)-e);
-    }
-  }
+  const float tscale = operator_scale(a, blk, dmax, ++epoch, sh, fault);
   const float mscale = 1.f / tscale;  // exact: a power of two
   tzlo *= tscale;
 #pragma unroll
@@ -413,12 +480,10 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     for (int j = 0; j < 5; ++j) mh[j] *= mscale;
 
   // ---- iterations -------------------------------------------------------------
-  const float rtol2h = (float)a.rtol2, rtol2l = (float)(a.rtol2 - (double)rtol2h);
   float alpha = 0.f, beta = 0.f;
-  Dfl rho = {0.f, 0.f}, rho0 = {0.f, 0.f}, thresh = {0.f, 0.f};
-  long long iter = 0, sweeps = 0;  // (warp 0)
-  const long long maxit = a.maxit, guard = 2 * maxit + 64;
   int done = kRunning;
+  ResScalars sc;  // (warp 0)
+  sc.init();
   ResNext& sNext = sh.next;
   uint2* fmine = a.face + (size_t)blk * LY::kFaces;
   const bool fy0 = warp == 0 && by > 0, fy1 = warp == kRW - 1 && by + 1 < a.nby;
@@ -523,36 +588,11 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
       fault = true;
       break;
     }
-    // alpha, beta and the stop test (as cg_finish), formed by warp 0 alone: in
-    // all 16 warps the same chain takes twice as long
+    // the scalars are formed by warp 0 alone: in all 16 warps the same chain takes
+    // twice as long
     if (warp == 0) {
-      rho = tot[0];
-      if (iter == 0) {
-        rho0 = rho;
-        thresh = df_add(df_mulf(rho0, rtol2h), df_mulf(rho0, rtol2l));
-      }
-      // alpha is the FP32 step the vectors take, so that rho - 2 alpha r'q +
-      // alpha^2 q'q is the norm of the residual it leaves
-      const float al = quot(rho.h, tot[1].h);
-      const Dfl u = df_mulf(tot[3], al);
-      const Dfl v = df_mulf(df_add({2.f * tot[2].h, 2.f * tot[2].l}, {-u.h, -u.l}), al);
-      Dfl rn = df_add(rho, {-v.h, -v.l});
-      if (rn.h < 0.f) rn = {0.f, 0.f};
-      alpha = al;
-      beta = quot(rn.h, rho.h);
-      // 0 unless one of the sums is infinite or NaN
-      const float bad = fmaf(tot[0].h, 0.f, fmaf(tot[1].h, 0.f, fmaf(tot[2].h, 0.f, tot[3].h * 0.f)));
-      const bool stay = bad == 0.f && tot[1].h > 0.f && !df_le(rho, thresh);
-      ++iter;
-      if (!stay || df_le(rn, thresh) || iter >= maxit || ++sweeps > guard) {
-        done = stay ? (df_le(rn, thresh) ? kConvEst : iter >= maxit ? kMaxit : kGuard)
-                    : (bad != 0.f ? kNonFinite : df_le(rho, thresh) ? kConvTrue : kBreakdown);
-        if (!stay) {
-          alpha = 0.f;
-          --iter;
-        }
-      }
-      if (lane == 0) sNext = {alpha, beta, done};
+      sc.update(tot, a.rtol2, a.maxit);
+      if (lane == 0) sNext = {sc.alpha, sc.beta, sc.done};
     }
     __syncthreads();
     alpha = sNext.alpha;
@@ -581,15 +621,8 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
       break;
     }
     if (warp == 0) {
-      const Dfl prev = rho;
-      rho = tot[0];
-      if (done == kConvEst && !df_le(rho, thresh) && iter < a.maxit && isfinite(rho.h) &&
-          prev.h > 0.f) {
-        // the estimate was too optimistic: go on with the exact continuation
-        beta = quot(rho.h, prev.h);
-        done = kRunning;
-      }
-      if (lane == 0) sNext = {0.f, beta, done};
+      sc.finish(tot, a.maxit);
+      if (lane == 0) sNext = {sc.alpha, sc.beta, sc.done};
     }
     __syncthreads();
     alpha = sNext.alpha;
@@ -610,17 +643,353 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
       }
   }
   if (blk == 0 && tid == 0) {
-    st->rho = (double)rho.h + (double)rho.l;
-    st->rho0 = (double)rho0.h + (double)rho0.l;
-    st->scale = scale;
-    st->iter = iter;
-    st->launches = 1;
-    st->done = done;
-    st->fault = fault ? 1 : 0;
+    sc.report(st, scale, fault);
     *(volatile uint32_t*)a.ctl = epoch;
   }
 }
 
+// ---- bricks of up to 32 planes -------------------------------------------------
+// The same iteration for grids of up to twice that size (2.5 M cells on GB300).
+// r and q are in registers, p, x and Ty in shared memory, and the other
+// coefficients (Tx, Tz, D: 12 bytes per cell) are read every iteration from a
+// packed copy, which each thread writes for itself at the start and which stays
+// in L2; loads run four planes ahead of the stencil.  The Jacobi variant is plain
+// CG on S A S with S = M^-1/2 (the same iterates: r'M^-1 r is the norm of S r), so
+// that neither M^-1 nor a second vector is needed.
+template <int CZ>
+struct BigLayout {
+  static constexpr int kP = 0;                                  // [CZ][W + 2][34]
+  static constexpr int kX = kP + CZ * (kRW + 2) * 34;           // [CZ][W][32]
+  static constexpr int kTy = kX + CZ * kRW * 32;                // [CZ][W + 1][32], row 0: y - 1
+  static constexpr int kTx = kTy + CZ * (kRW + 1) * 32;         // [CZ][W]: Tx of x - 1, lane 0
+  static constexpr int kFx = CZ * kRW, kFy = CZ * 32, kFz = kRW * 32;
+  static constexpr int kFaces = 2 * (kFx + kFy + kFz);
+  static constexpr int kNY = CZ / 8, kNX = 2, kNH = 2 + kNY + kNX;  // halo cells per thread
+  static constexpr int kRh = kTx + CZ * kRW;                    // r of the y and x halo cells
+  static constexpr int kFloats = kRh + (kNY + kNX) * kRT;
+  static_assert(CZ % 8 == 0 && CZ <= 32, "halo rows per warp");
+};
+
+template <int CZ, bool JAC>
+__global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_constant__ ResProb a) {
+  using LY = BigLayout<CZ>;
+  constexpr int NH = LY::kNH;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ ResShared sh;
+  float* sP = sm + LY::kP;
+  float* sX = sm + LY::kX;
+  float* sTy = sm + LY::kTy;
+  float* sTx = sm + LY::kTx;
+  float* sRh = sm + LY::kRh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int blk = blockIdx.x;
+  const int bx = blk % a.nbx, by = (blk / a.nbx) % a.nby, bz = blk / (a.nbx * a.nby);
+  const Grid g = a.g;
+  const int64_t gx = 32 * bx + lane, gy = kRW * by + warp, Z0 = (int64_t)CZ * bz;
+  const bool inxy = gx < g.nx && gy < g.ny;
+  const int64_t c0 = gx + g.nx * gy;
+  CgState* st = a.st;
+  const double scale = st->rr64 > 0.0 ? 1.0 / sqrt(st->rr64) : 1.0;
+
+  const float4* c32 = static_cast<const float4*>(a.coef);
+  const uint2* c16 = static_cast<const uint2*>(a.coef);
+  auto inside = [&](int64_t x, int64_t y, int64_t z) {
+    return x >= 0 && y >= 0 && z >= 0 && x < g.nx && y < g.ny && z < g.nz;
+  };
+  auto rec = [&](int64_t x, int64_t y, int64_t z) -> float4 {
+    if (!inside(x, y, z)) return make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t c = x + g.nx * y + g.plane * z;
+    if (!a.b16) return __ldg(c32 + c);
+    const uint2 u = __ldg(c16 + c);
+    return make_float4(bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y));
+  };
+  // S of a cell (Jacobi): the root of M^-1; 1 without preconditioner, 0 outside
+  auto root = [&](int64_t x, int64_t y, int64_t z) -> float {
+    if (!inside(x, y, z)) return 0.f;
+    if (!JAC) return 1.f;
+    const int64_t c = x + g.nx * y + g.plane * z;
+    return __fsqrt_rn(a.b16 ? __ldg(a.dinv + c) : jac_inv(__ldg(c32 + c).w));
+  };
+  // D of an own cell (BF16 records: formed from the faces as the sweeps do)
+  auto diag = [&](int64_t z, const float4& cf) -> float {
+    if (!a.b16) return cf.w;
+    const float txm = rec(gx - 1, gy, z).x, tym = rec(gx, gy - 1, z).y, tzm = rec(gx, gy, z - 1).z;
+    return (((((txm + cf.x) + tym) + cf.y) + tzm) + cf.z) + cf.w;
+  };
+
+  // ---- scale, packed coefficients -----------------------------------------------
+  uint32_t epoch = *(volatile uint32_t*)a.ctl;
+  bool fault = false;
+  float tscale = 1.f;
+  {
+    float dmax = JAC ? 1.f : 0.f;  // S A S has a unit diagonal
+    if (!JAC && inxy)
+      for (int k = 0; k < CZ && Z0 + k < g.nz; ++k)
+        dmax = fmaxf(dmax, diag(Z0 + k, rec(gx, gy, Z0 + k)));
+    tscale = operator_scale(a, blk, dmax, ++epoch, sh, fault);
+  }
+  // every face value is (T s_low) s_high in both its cells
+  float2* pk = a.packed + ((size_t)blk * CZ * kRW + warp) * 32 + lane;           // (Tx, Tz)
+  float* pd = reinterpret_cast<float*>(a.packed + (size_t)a.nblk * CZ * kRT) +
+              ((size_t)blk * CZ * kRW + warp) * 32 + lane;                         // D
+  const float tzlo = inxy ? rec(gx, gy, Z0 - 1).z * tscale * root(gx, gy, Z0 - 1) *
+                                root(gx, gy, Z0) : 0.f;
+#pragma unroll 1
+  for (int k = 0; k < CZ; ++k) {
+    const int64_t z = Z0 + k;
+    const float4 cf = rec(gx, gy, z);
+    const float sc = root(gx, gy, z);
+    const bool in = inxy && z < g.nz;
+    const float D = in ? diag(z, cf) : 0.f;
+    pk[(size_t)k * kRT] = make_float2(cf.x * tscale * sc * root(gx + 1, gy, z),
+                                      cf.z * tscale * sc * root(gx, gy, z + 1));
+    pd[(size_t)k * kRT] = D * tscale * sc * sc;
+    sTy[(k * (kRW + 1) + warp + 1) * 32 + lane] = cf.y * tscale * sc * root(gx, gy + 1, z);
+    if (warp == 0)
+      sTy[k * (kRW + 1) * 32 + lane] = rec(gx, gy - 1, z).y * tscale * root(gx, gy - 1, z) * sc;
+    if (lane == 0)
+      sTx[k * kRW + warp] = rec(gx - 1, gy, z).x * tscale * root(gx - 1, gy, z) * sc;
+    sX[(k * kRW + warp) * 32 + lane] = 0.f;
+  }
+  for (int i = tid; i < CZ * (kRW + 2) * 34; i += kRT) sP[i] = 0.f;
+  __syncthreads();
+
+  // ---- halo cells: 0, 1 below and above; kNY y rows; kNX x cells -------------------
+  ResComm<NH, false> cm;
+  cm.part = a.part;
+  cm.face = a.face;
+  cm.abort = a.abort;
+  cm.nblk = a.nblk;
+  cm.blk = blk;
+  cm.face_buf = (size_t)a.nblk * LY::kFaces;
+  float rz[2] = {0.f, 0.f}, pz[2] = {0.f, 0.f}, qh[NH];
+  // y rows: row id warp + 16 j counts (side, k); x cells: tid + 512 j counts (side, w, k)
+  auto yk = [&](int j) { return (warp + kRW * j) % CZ; };
+  auto yhi = [&](int j) { return warp + kRW * j >= CZ; };
+  auto xk = [&](int j) { return (tid + kRT * j) % LY::kFx % CZ; };
+  auto xw = [&](int j) { return (tid + kRT * j) % LY::kFx / CZ; };
+  auto xhi = [&](int j) { return tid + kRT * j >= LY::kFx; };
+  auto halo_r = [&](int64_t x, int64_t y, int64_t z) -> float {
+    if (!inside(x, y, z)) return 0.f;
+    return (float)(scale * a.r64[x + g.nx * y + g.plane * z]) * root(x, y, z);
+  };
+  {
+    const int fz = 2 * (LY::kFx + LY::kFy), fy = 2 * LY::kFx;
+    cm.hoff[0] = bz > 0 ? (blk - a.nbx * a.nby) * LY::kFaces + fz + LY::kFz + tid : -1;
+    cm.hoff[1] = bz + 1 < a.nbz ? (blk + a.nbx * a.nby) * LY::kFaces + fz + tid : -1;
+    rz[0] = halo_r(gx, gy, Z0 - 1);
+    rz[1] = halo_r(gx, gy, Z0 + CZ);
+#pragma unroll
+    for (int j = 0; j < LY::kNY; ++j) {
+      const int w = yk(j) * 32 + lane;
+      cm.hoff[2 + j] = yhi(j) ? (by + 1 < a.nby ? (blk + a.nbx) * LY::kFaces + fy + w : -1)
+                              : (by > 0 ? (blk - a.nbx) * LY::kFaces + fy + LY::kFy + w : -1);
+      sRh[j * kRT + tid] =
+          halo_r(gx, kRW * (int64_t)by + (yhi(j) ? kRW : -1), Z0 + yk(j));
+    }
+#pragma unroll
+    for (int j = 0; j < LY::kNX; ++j) {
+      const bool use = tid + kRT * j < 2 * LY::kFx;
+      const int w = xw(j) * CZ + xk(j);
+      cm.hoff[2 + LY::kNY + j] =
+          !use ? -1
+               : xhi(j) ? (bx + 1 < a.nbx ? (blk + 1) * LY::kFaces + w : -1)
+                        : (bx > 0 ? (blk - 1) * LY::kFaces + LY::kFx + w : -1);
+      sRh[(LY::kNY + j) * kRT + tid] =
+          use ? halo_r(32 * (int64_t)bx + (xhi(j) ? 32 : -1), kRW * (int64_t)by + xw(j), Z0 + xk(j))
+              : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < NH; ++j) qh[j] = 0.f;
+  }
+
+  float r[CZ], q[CZ];
+#pragma unroll
+  for (int k = 0; k < CZ; ++k) {
+    r[k] = halo_r(gx, gy, Z0 + k);
+    q[k] = 0.f;
+  }
+
+  float alpha = 0.f, beta = 0.f;
+  int done = kRunning;
+  ResScalars sc;  // (warp 0)
+  sc.init();
+  uint2* fmine = a.face + (size_t)blk * LY::kFaces;
+
+  auto step = [&](bool dir, Acc& s0) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (cm.hoff[j] < 0) continue;
+      rz[j] = fmaf(-alpha, qh[j], rz[j]);
+      if (dir) pz[j] = fmaf(beta, pz[j], rz[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < LY::kNY + LY::kNX; ++j) {
+      if (cm.hoff[2 + j] < 0) continue;
+      const float rn = fmaf(-alpha, qh[2 + j], sRh[j * kRT + tid]);
+      sRh[j * kRT + tid] = rn;
+      if (!dir) continue;
+      const int i = j - LY::kNY;
+      float* ps = j < LY::kNY ? sP + (yk(j) * (kRW + 2) + (yhi(j) ? kRW + 1 : 0)) * 34 + lane + 1
+                              : sP + (xk(i) * (kRW + 2) + xw(i) + 1) * 34 + (xhi(i) ? 33 : 0);
+      *ps = fmaf(beta, *ps, rn);
+    }
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < CZ; ++k) {
+      float* ps = sP + (k * (kRW + 2) + warp + 1) * 34 + lane + 1;
+      float* xs = sX + (k * kRW + warp) * 32 + lane;
+      const float p0 = *ps;
+      *xs = fmaf(alpha, p0, *xs);
+      r[k] = fmaf(-alpha, q[k], r[k]);
+      if (dir) *ps = fmaf(beta, p0, r[k]);
+      s = fmaf(r[k], r[k], s);
+      if ((k & 3) == 3) {
+        kadd(s0, s);
+        s = 0.f;
+      }
+    }
+  };
+
+  while (!fault) {
+    Acc acc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    // the first planes' coefficients, in flight during the step
+    constexpr int kPre = 4;
+    float2 tc[kPre];
+    float dc[kPre];
+#pragma unroll
+    for (int k = 0; k < kPre; ++k) {
+      tc[k] = __ldcg(pk + (size_t)k * kRT);
+      dc[k] = __ldcg(pd + (size_t)k * kRT);
+    }
+    step(true, acc[0]);
+    __syncthreads();
+    ++epoch;
+    uint2* fo = fmine + (epoch & 1u) * cm.face_buf;
+    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    float tz0 = tzlo, pm = pz[0];
+    float pc = sP[(warp + 1) * 34 + lane + 1];
+#pragma unroll
+    for (int k = 0; k < CZ; ++k) {
+      const float* ps = sP + (k * (kRW + 2) + warp + 1) * 34 + lane + 1;
+      const float pp = k + 1 < CZ ? ps[(kRW + 2) * 34] : pz[1];
+      const float* ty = sTy + (k * (kRW + 1) + warp) * 32 + lane;
+      const float2 t = tc[k % kPre];
+      const float D = dc[k % kPre];
+      if (k + kPre < CZ) {
+        tc[k % kPre] = __ldcg(pk + (size_t)(k + kPre) * kRT);
+        dc[k % kPre] = __ldcg(pd + (size_t)(k + kPre) * kRT);
+      }
+      float txm = __shfl_up_sync(kFull, t.x, 1);
+      if (lane == 0) txm = sTx[k * kRW + warp];
+      const float4 cf = make_float4(t.x, ty[32], t.y, D);
+      const float v = stencil7(cf, txm, ty[0], tz0, pc, ps[1], ps[-1], ps[34], ps[-34], pp, pm);
+      q[k] = v;
+      s1 = fmaf(pc, v, s1);
+      s2 = fmaf(r[k], v, s2);
+      s3 = fmaf(v, v, s3);
+      if ((k & 3) == 3) {
+        kadd(acc[1], s1);
+        kadd(acc[2], s2);
+        kadd(acc[3], s3);
+        s1 = s2 = s3 = 0.f;
+      }
+      tz0 = t.y;
+      pm = pc;
+      pc = pp;
+    }
+    if (bz > 0) ll_store(fo + 2 * (LY::kFx + LY::kFy) + tid, q[0], epoch);
+    if (bz + 1 < a.nbz) ll_store(fo + 2 * (LY::kFx + LY::kFy) + LY::kFz + tid, q[CZ - 1], epoch);
+    if ((warp == 0 && by > 0) || (warp == kRW - 1 && by + 1 < a.nby)) {
+      uint2* f = fo + 2 * LY::kFx + (warp == 0 ? 0 : LY::kFy) + lane;
+#pragma unroll
+      for (int k = 0; k < CZ; ++k) ll_store(f + k * 32, q[k], epoch);
+    }
+    if (bx > 0 || bx + 1 < a.nbx) {
+#pragma unroll
+      for (int h = 0; h < CZ; h += 16) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = h; k < h + 16 && k < CZ; ++k) {
+          const float t = __shfl_sync(kFull, q[k], lane < 16 ? 0 : 31);
+          if ((lane & 15) == k - h) v = t;
+        }
+        if (h + (lane & 15) < CZ && (lane < 16 ? bx > 0 : bx + 1 < a.nbx))
+          ll_store(fo + (lane < 16 ? 0 : LY::kFx) + warp * CZ + h + (lane & 15), v, epoch);
+      }
+    }
+    Dfl mine[4], tot[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) mine[v] = df_fast(acc[v].s, -acc[v].c);
+    if (!cm.exchange(mine, epoch, tot, qh, sh)) {
+      fault = true;
+      break;
+    }
+    if (warp == 0) {
+      sc.update(tot, a.rtol2, a.maxit);
+      if (lane == 0) sh.next = {sc.alpha, sc.beta, sc.done};
+    }
+    __syncthreads();
+    alpha = sh.next.alpha;
+    beta = sh.next.beta;
+    done = sh.next.done;
+    if (done == kRunning) continue;
+    if (done != kConvEst && done != kMaxit) break;
+    // the last step, and the true r'r of the residual it leaves (no face words)
+    Acc s0 = {0.f, 0.f};
+    step(false, s0);
+    ++epoch;
+    int keep[NH];
+#pragma unroll
+    for (int j = 0; j < NH; ++j) {
+      keep[j] = cm.hoff[j];
+      cm.hoff[j] = -1;
+    }
+    mine[0] = df_fast(s0.s, -s0.c);
+    mine[1] = mine[2] = mine[3] = {0.f, 0.f};
+    const bool ok = cm.exchange(mine, epoch, tot, qh, sh);
+#pragma unroll
+    for (int j = 0; j < NH; ++j) cm.hoff[j] = keep[j];
+    if (!ok) {
+      fault = true;
+      break;
+    }
+    if (warp == 0) {
+      sc.finish(tot, a.maxit);
+      if (lane == 0) sh.next = {sc.alpha, sc.beta, sc.done};
+    }
+    __syncthreads();
+    alpha = sh.next.alpha;
+    beta = sh.next.beta;
+    done = sh.next.done;
+    if (done != kRunning) break;
+  }
+
+  if (fault) done = kGuard;
+  if (done != kNonFinite && done != kGuard && inxy) {
+    const double inv = (double)tscale / scale;
+    for (int k = 0; k < CZ && Z0 + k < g.nz; ++k) {
+      const int64_t c = c0 + g.plane * (Z0 + k);
+      const double e = (double)sX[(k * kRW + warp) * 32 + lane] * (double)root(gx, gy, Z0 + k);
+      a.x64[c] = fma(e, inv, a.x64[c]);
+    }
+  }
+  if (blk == 0 && tid == 0) {
+    sc.report(st, scale, fault);
+    *(volatile uint32_t*)a.ctl = epoch;
+  }
+}
+
+template <int CZ>
+cudaError_t launch_big(ResProb& a, bool jac, cudaStream_t s) {
+  constexpr int smem = BigLayout<CZ>::kFloats * 4;
+  const void* fn = jac ? (const void*)resident_big_kernel<CZ, true>
+                       : (const void*)resident_big_kernel<CZ, false>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel(fn, dim3(a.nblk), dim3(kRT), args, smem, s);
+}
 template <int CZ, bool JAC>
 __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant__ ResProb a) {
   extern __shared__ __align__(16) float sm[];
@@ -795,9 +1164,9 @@ size_t sched_words(int nprob, int nblocks) {  // 8-byte words after the sums and
 bool plan_resident(const Grid& g, int num_sms, bool dense, ResPlan* p) {
   const int64_t bx = (g.nx + 31) / 32, by = (g.ny + kRW - 1) / kRW;
   if (bx * by > num_sms) return false;
-  constexpr int fast[] = {1, 2, 4, 6, 8, 12, 16}, packed[] = {4, 8, 16};
+  constexpr int fast[] = {1, 2, 4, 6, 8, 12, 16, 24, 32}, packed[] = {4, 8, 16};
   const int* heights = dense ? packed : fast;
-  const int nh = dense ? 3 : 7;
+  const int nh = dense ? 3 : 9;
   double best = 0.0;
   int cz = 0;
   for (int h = 0; h < nh; ++h) {
@@ -818,6 +1187,7 @@ bool plan_resident(const Grid& g, int num_sms, bool dense, ResPlan* p) {
   // control words, sums, faces (two buffers each)
   p->words = 32 + (size_t)2 * p->nblk * 8 +
              (size_t)2 * p->nblk * (2 * ((size_t)cz * kRW + (size_t)cz * 32 + kRW * 32));
+  p->packed = cz > 16 ? (size_t)p->nblk * cz * kRT * 12 : 0;
   return true;
 }
 
@@ -844,6 +1214,7 @@ ResProb make_res_prob(const Grid& g, const ResPlan& p, const void* coef, bool b1
   a.part = reinterpret_cast<uint2*>(comm + 32);
   a.face = a.part + (size_t)2 * p.nblk * 8;
   a.team = nullptr;
+  a.packed = nullptr;
   return a;
 }
 
@@ -857,6 +1228,8 @@ cudaError_t launch_resident(const ResProb& prob, bool jac, cudaStream_t s) {
     case 8: return launch_cz<8>(a, jac, s);
     case 12: return launch_cz<12>(a, jac, s);
     case 16: return launch_cz<16>(a, jac, s);
+    case 24: return launch_big<24>(a, jac, s);
+    case 32: return launch_big<32>(a, jac, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -226,6 +226,7 @@ cudaError_t launch_apply_batch(const BatchInst* inst, int ninst, int64_t nblocks
 struct ResPlan {
   int cz, nbx, nby, nbz, nblk;  // brick height, bricks per axis, bricks
   size_t words;                 // 8-byte words of exchange buffers
+  size_t packed;                // bytes of the packed coefficients (bricks above 16 planes)
 };
 struct ResProb {
   Grid g;
@@ -243,6 +244,7 @@ struct ResProb {
   uint32_t* ctl;          // last epoch used
   uint32_t* abort;        // set by a block whose wait ran out
   int* team;              // batched: [nblk] blocks that run it
+  float2* packed;         // bricks above 16 planes: p.packed bytes of workspace
 };
 // Bricks for one grid; false when it does not fit at one brick per SM.
 // dense = false: the lowest bricks that fit (shortest iterations of a solve that

@@ -2,7 +2,7 @@
 the cp.async sweep, which does the same per-cell arithmetic, and the oracle.
 
 Shapes: one cell, single brick columns and planes, bricks with ragged edges on
-every axis, several bricks along every axis, every brick height (1 to 16
+every axis, several bricks along every axis, every brick height (1 to 32
 planes), the largest grid that fits one brick per SM and the first that does
 not (which keeps the sweeps)."""
 import numpy as np
@@ -56,7 +56,8 @@ def _resident(info):
 SHAPES = [((1, 1, 1), "wells"), ((5, 3, 2), "wells"), ((32, 16, 1), "wells"), ((33, 17, 9), "dirx"),
           ((31, 15, 40), "wells"), ((64, 1, 300), "wells"), ((1, 200, 7), "wells"),
           ((100, 30, 41), "wells"), ((65, 47, 90), "dirx"), ((48, 24, 200), "wells"),
-          ((96, 96, 48), "dirx"), ((128, 128, 64), "wells")]
+          ((96, 96, 48), "dirx"), ((128, 128, 64), "wells"), ((65, 33, 300), "dirx"),
+          ((128, 128, 128), "wells")]
 
 
 @pytest.mark.parametrize("b16,jac", [(False, 0), (False, 1), (True, 0), (True, 1)],
@@ -85,8 +86,8 @@ def test_resident_iterates_and_solution(tp, oracle_mod, shape, kind, b16, jac):
 
 
 def test_grid_beyond_the_chip_keeps_the_sweeps(tp):
-    c = _case((160, 160, 96), 12, "wells")
-    _, info = _solve(tp, (160, 160, 96), c, 1e-4, 1000, {"precond": 1})
+    c = _case((192, 160, 96), 12, "wells")
+    _, info = _solve(tp, (192, 160, 96), c, 1e-4, 1000, {"precond": 1})
     assert info["code"] == 0 and not _resident(info)
 
 
