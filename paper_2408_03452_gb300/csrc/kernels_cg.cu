@@ -58,20 +58,26 @@ struct SweepArgs {
 // With Jacobi preconditioning and FP32 records the stage also holds D of the
 // halo rows -1 and VY (the records of the own rows carry theirs); with BF16
 // records, which do not store D, it holds M^-1 of every row -1 .. VY.
-template <int VY, bool B16, bool JAC = false>
+// The plain operator (CG = false) stages p alone: 2,944 instead of 4,992 bytes per
+// warp and plane, so that twice as many warps keep copies in flight (375 x 497 x
+// 461, rows not a multiple of 16 bytes: 360 -> 329 us).
+template <int VY, bool B16, bool JAC = false, bool CG = true>
 struct StageLayout {
   static constexpr int kRec = B16 ? 8 : 16;
   static constexpr int kCoef = 0;                               // record [VY][32]
-  static constexpr int kVec = VY * 32 * kRec;                   // float [3][VY+2][32]
-  static constexpr int kE = kVec + 3 * (VY + 2) * 32 * 4;       // float [VY][32]
-  static constexpr int kTy = kE + VY * 32 * 4;                  // 32-bit word [32]
+  static constexpr int kVec = VY * 32 * kRec;                   // float [3 or 1][VY+2][32]
+  static constexpr int kPv = CG ? 2 * (VY + 2) : 0;             // first row of p
+  static constexpr int kE = kVec + (CG ? 3 : 1) * (VY + 2) * 32 * 4;  // float [VY][32] (CG)
+  static constexpr int kTy = kE + (CG ? VY * 32 * 4 : 0);       // 32-bit word [32]
   static constexpr int kDh = kTy + 32 * 4;                      // float [2 or VY+2][32] (JAC)
   static constexpr int kDhRows = JAC ? (B16 ? VY + 2 : 2) : 0;
   static constexpr int kBytes = kDh + kDhRows * 32 * 4;
 };
 
-template <int VY, int S, bool B16, bool JAC = false>
-constexpr int sweep_smem_bytes() { return kSweepWarps * S * StageLayout<VY, B16, JAC>::kBytes; }
+template <int VY, int S, bool B16, bool JAC = false, bool CG = true>
+constexpr int sweep_smem_bytes() {
+  return kSweepWarps * S * StageLayout<VY, B16, JAC, CG>::kBytes;
+}
 
 // A staged record as (Tx, Ty, Tz, w): w = D for FP32 records, w = E (the
 // diagonal beyond the six face terms) for BF16 records.
@@ -109,7 +115,7 @@ sweep_kernel(const SweepArgs a) {
   static_assert(!JAC || CG, "Jacobi preconditioning is for CG sweeps");
   static_assert(!BATCH || (!B16 && !COND), "batched sweeps use FP32 records, no graph condition");
   static_assert(!BATCH || !JAC || CG, "the batched operator has no preconditioner");
-  using LY = StageLayout<VY, B16, JAC>;
+  using LY = StageLayout<VY, B16, JAC, CG>;
   extern __shared__ __align__(16) unsigned char smem[];
   Grid g = a.g;
   int64_t nwx = a.nwx, nwy = a.nwy, nwarps = a.nwarps, zcr = a.zc, off = 0;
@@ -205,9 +211,9 @@ sweep_kernel(const SweepArgs a) {
           if (CG) {
             cp4(sv + (0 * (VY + 2) + jj + 1) * 32 + lane, rin + src, ok);
             cp4(sv + (1 * (VY + 2) + jj + 1) * 32 + lane, qin + src, ok);
-            cp4(sv + (2 * (VY + 2) + jj + 1) * 32 + lane, pin + src, ok);
+            cp4(sv + (LY::kPv + jj + 1) * 32 + lane, pin + src, ok);
           } else {
-            cp4(sv + (2 * (VY + 2) + jj + 1) * 32 + lane, pin + src, ok);
+            cp4(sv + (LY::kPv + jj + 1) * 32 + lane, pin + src, ok);
           }
           if (jj == -1) {
             if (B16) cp4(sty + lane, a.coef16 + src, ok);  // word 0 = Tx | Ty << 16
@@ -240,7 +246,7 @@ sweep_kernel(const SweepArgs a) {
       const int64_t zo = g.plane * z;
 #pragma unroll
       for (int jj = -1; jj <= VY; ++jj) {
-        const float p0 = sv[(2 * (VY + 2) + jj + 1) * 32 + lane];
+        const float p0 = sv[(LY::kPv + jj + 1) * 32 + lane];
         float p_ = p0, r_ = 0.f;
         if (CG) {
           const float r0 = sv[(0 * (VY + 2) + jj + 1) * 32 + lane];
@@ -543,7 +549,7 @@ static SweepArgs sweep_args(const Grid& g, const Sweep& sw, const float4* coef) 
 
 template <int VY, int S, bool CG, bool COND, bool B16, bool JAC = false, bool BATCH = false>
 static cudaError_t launch_t(const SweepArgs& a, const Sweep& sw, cudaStream_t s) {
-  constexpr int smem = sweep_smem_bytes<VY, S, B16, JAC>();
+  constexpr int smem = sweep_smem_bytes<VY, S, B16, JAC, CG>();
   cudaError_t e = cudaFuncSetAttribute(sweep_kernel<VY, S, CG, COND, B16, JAC, BATCH>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
