@@ -40,6 +40,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "net_internal.cuh"
 #include "sweep_common.cuh"
 #include "tc_common.cuh"
@@ -806,8 +808,18 @@ cudaError_t launch_apply_t(const ApplyArgs& a, int64_t nblocks, cudaStream_t s) 
   constexpr int S = apply_stages<DM>();
   constexpr int smem = apply_smem_bytes<4, 4, S, B16, DM < 0 ? 0 : 2 + DM>();
   auto fn = apply_tma_kernel<4, 4, S, B16, BATCH, DM>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // the attribute is set on the first launch of a device (it costs as much as the
+  // rest of the launch)
+  static std::atomic<uint64_t> set{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+  if ((set.load(std::memory_order_acquire) & bit) == 0) {
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    set.fetch_or(bit, std::memory_order_release);
+  }
   fn<<<(unsigned)nblocks, 5 * 32, smem, s>>>(a);
   return cudaGetLastError();
 }
