@@ -706,11 +706,11 @@ struct RowMaps {
   CUtensorMap a, b;
 };
 
-template <int CIN, int COUT>
+template <int CIN, int COUT, int FUSE = kFuseNone>
 __global__ void __launch_bounds__(192)
 conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict__ bias,
                    const uint16_t* __restrict__ mask, uint16_t* __restrict__ y, Vol g, int flags,
-                   ZmGrid zg) {
+                   ZmGrid zg, const ConvFuse fuse) {
   using Cfg = WsCfg<CIN, COUT>;
   constexpr int ST = Cfg::kST;
   constexpr int R = Cfg::kR;
@@ -860,6 +860,8 @@ conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict
       const int vy = bi / zg.nbx * Cfg::kTY + warp * 4 + (lane >> 3);
       const int poff = (vy + 1) * g.wp + vx + 1;
       const bool in_xy = vx < g.nx && vy < g.ny;
+      float psum[FUSE == kFusePool ? COUT : 1];  // pool: sums of the even plane
+      (void)psum;
       bool stop = false;
       for (int k = 0; k < nout; ++k) {
         const int oc = obase + k;
@@ -871,29 +873,102 @@ conv_fwd_ws_kernel(const __grid_constant__ RowMaps maps, const float* __restrict
         tc::fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive1(&aempty[sl]);
-        if (in_xy) {
-          const size_t idx = (size_t)(kp0 + k) * g.pp + poff;
+        uint32_t ov[COUT / 2];  // the output voxel in BF16
+        const size_t idx = (size_t)(kp0 + k) * g.pp + poff;
 #pragma unroll
-          for (int c0 = 0; c0 < COUT; c0 += 8) {
-            const float* v = va + c0;
-            uint4 mk = make_uint4(0, 0, 0, 0);
-            if (flags & kConvMask) mk = *reinterpret_cast<const uint4*>(mask + idx * COUT + c0);
-            const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
-            uint32_t ov[4];
+        for (int c0 = 0; c0 < COUT; c0 += 8) {
+          const float* v = va + c0;
+          uint4 mk = make_uint4(0, 0, 0, 0);
+          if (FUSE == kFuseNone && (flags & kConvMask) && in_xy)
+            mk = *reinterpret_cast<const uint4*>(mask + idx * COUT + c0);
+          const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              float a = v[2 * h] + sbias[c0 + 2 * h], b = v[2 * h + 1] + sbias[c0 + 2 * h + 1];
-              if (flags & kConvRelu) {
-                a = fmaxf(a, 0.f);
-                b = fmaxf(b, 0.f);
-              }
-              if (flags & kConvMask) {
-                if (!bf16_positive(mw[h] & 0xffffu)) a = 0.f;
-                if (!bf16_positive(mw[h] >> 16)) b = 0.f;
-              }
-              ov[h] = pack_bf16(a, b);
+          for (int h = 0; h < 4; ++h) {
+            float a = v[2 * h] + sbias[c0 + 2 * h], b = v[2 * h + 1] + sbias[c0 + 2 * h + 1];
+            if (flags & kConvRelu) {
+              a = fmaxf(a, 0.f);
+              b = fmaxf(b, 0.f);
             }
-            *reinterpret_cast<uint4*>(y + idx * COUT + c0) = make_uint4(ov[0], ov[1], ov[2], ov[3]);
+            if (FUSE == kFuseNone && (flags & kConvMask)) {
+              if (!bf16_positive(mw[h] & 0xffffu)) a = 0.f;
+              if (!bf16_positive(mw[h] >> 16)) b = 0.f;
+            }
+            ov[c0 / 2 + h] = pack_bf16(a, b);
+          }
+          if (FUSE != kFuseCells && in_xy)
+            *reinterpret_cast<uint4*>(y + idx * COUT + c0) =
+                make_uint4(ov[c0 / 2], ov[c0 / 2 + 1], ov[c0 / 2 + 2], ov[c0 / 2 + 3]);
+        }
+        if (FUSE == kFuseCells && in_xy) {
+          const int s_ = cz / zg.nzc;
+          fuse.z[(((size_t)s_ * g.nz + z0 + k) * g.ny + vy) * g.nx + vx] =
+              fuse.rms[s_] * __uint_as_float(ov[0] << 16);
+        }
+        if (FUSE == kFusePool) {
+          // children in the order (dz, dy, dx): x neighbours are lanes 1 apart, y
+          // neighbours 8 apart, z neighbours consecutive outputs of the unit
+#pragma unroll
+          for (int h = 0; h < COUT / 2; ++h) {
+            const uint32_t w0 = ov[h];
+            const uint32_t w1 = __shfl_down_sync(0xffffffffu, w0, 1);
+            const uint32_t w2 = __shfl_down_sync(0xffffffffu, w0, 8);
+            const uint32_t w3 = __shfl_down_sync(0xffffffffu, w0, 9);
+            float lo = (k & 1) ? psum[2 * h] : 0.f, hi = (k & 1) ? psum[2 * h + 1] : 0.f;
+            lo += __uint_as_float(w0 << 16);
+            hi += __uint_as_float(w0 & 0xffff0000u);
+            lo += __uint_as_float(w1 << 16);
+            hi += __uint_as_float(w1 & 0xffff0000u);
+            lo += __uint_as_float(w2 << 16);
+            hi += __uint_as_float(w2 & 0xffff0000u);
+            lo += __uint_as_float(w3 << 16);
+            hi += __uint_as_float(w3 & 0xffff0000u);
+            psum[2 * h] = lo;
+            psum[2 * h + 1] = hi;
+          }
+          if ((k & 1) && in_xy && (vx & 1) == 0 && (vy & 1) == 0) {
+            const Vol& gc = fuse.g2;
+            const size_t vc = ((size_t)(cz / zg.nzc * gc.dp + (z0 + k) / 2 + 1) * gc.hp + vy / 2 + 1) *
+                                  gc.wp + vx / 2 + 1;
+#pragma unroll
+            for (int c0 = 0; c0 < COUT; c0 += 8) {
+              uint32_t o[4];
+#pragma unroll
+              for (int h = 0; h < 4; ++h)
+                o[h] = pack_bf16(psum[c0 + 2 * h] * 0.125f, psum[c0 + 2 * h + 1] * 0.125f);
+              *reinterpret_cast<uint4*>(fuse.out + vc * COUT + c0) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+          }
+        }
+        if (FUSE == kFuseUpadd && in_xy) {
+          const Vol& gf = fuse.g2;
+          const size_t vf = ((size_t)(cz / zg.nzc * gf.dp + 2 * (z0 + k) + 1) * gf.hp + 2 * vy + 1) *
+                                gf.wp + 2 * vx + 1;
+#pragma unroll
+          for (int dz = 0; dz < 2; ++dz) {
+            uint4 sk[4][COUT / 8];  // the four children of a plane: loads first
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+              for (int c = 0; c < COUT / 8; ++c)
+                sk[j][c] = __ldg(reinterpret_cast<const uint4*>(
+                    fuse.skip + (vf + (size_t)dz * gf.pp + (j >> 1) * gf.wp + (j & 1)) * COUT) + c);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+              for (int c = 0; c < COUT / 8; ++c) {
+                const uint32_t sw[4] = {sk[j][c].x, sk[j][c].y, sk[j][c].z, sk[j][c].w};
+                uint32_t o[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                  const uint32_t b = ov[4 * c + h];
+                  o[h] = pack_bf16(__uint_as_float(sw[h] << 16) + __uint_as_float(b << 16),
+                                   __uint_as_float(sw[h] & 0xffff0000u) +
+                                       __uint_as_float(b & 0xffff0000u));
+                }
+                *(reinterpret_cast<uint4*>(
+                      fuse.out + (vf + (size_t)dz * gf.pp + (j >> 1) * gf.wp + (j & 1)) * COUT) + c) =
+                    make_uint4(o[0], o[1], o[2], o[3]);
+              }
           }
         }
       }
@@ -1200,19 +1275,20 @@ int ws_run(int nb, int nz, int ns, int ctas) {
   return zc;
 }
 
-template <int CIN, int COUT>
+template <int CIN, int COUT, int FUSE = kFuseNone>
 cudaError_t ws_launch(const uint16_t* x, const uint16_t* w, const float* bias,
                       const uint16_t* mask, uint16_t* y, const Vol& g, int flags,
-                      cudaStream_t s) {
+                      cudaStream_t s, const ConvFuse& fuse = ConvFuse()) {
   using Cfg = WsCfg<CIN, COUT>;
+  const auto fn = conv_fwd_ws_kernel<CIN, COUT, FUSE>;
   static int per_sm = -1, nsm = 0;
-  if (per_sm < 0)
-    per_sm = ctas_per_sm((const void*)conv_fwd_ws_kernel<CIN, COUT>, Cfg::kSmem, Cfg::kCols, &nsm);
+  if (per_sm < 0) per_sm = ctas_per_sm((const void*)fn, Cfg::kSmem, Cfg::kCols, &nsm);
   const int ctas = per_sm * nsm;
   ZmGrid zg;
   zg.nbx = (g.nx + Cfg::kTX - 1) / Cfg::kTX;
   zg.nb = zg.nbx * ((g.ny + Cfg::kTY - 1) / Cfg::kTY);
   zg.zc = ws_run(zg.nb, g.nz, g.ns, ctas);
+  if (FUSE == kFusePool) zg.zc += zg.zc & 1;  // pairs of planes stay in a unit
   zg.nzc = (g.nz + zg.zc - 1) / zg.zc;
   zg.units = zg.nb * g.ns * zg.nzc;
   const int grid = zg.units < ctas ? zg.units : ctas;
@@ -1220,7 +1296,7 @@ cudaError_t ws_launch(const uint16_t* x, const uint16_t* w, const float* bias,
   if (!encode_volume(&maps.a, x, CIN, g, Cfg::kTX + 2, Cfg::kTY + 2) ||
       !encode_rows(&maps.b, w, CIN, 27 * COUT, COUT))
     return cudaErrorInvalidValue;
-  conv_fwd_ws_kernel<CIN, COUT><<<grid, 192, Cfg::kSmem, s>>>(maps, bias, mask, y, g, flags, zg);
+  fn<<<grid, 192, Cfg::kSmem, s>>>(maps, bias, mask, y, g, flags, zg, fuse);
   return cudaGetLastError();
 }
 
@@ -1307,6 +1383,19 @@ cudaError_t conv_fwd(const uint16_t* x, const uint16_t* w, const float* bias, co
   TPFA_CONV_SHAPES(X)
 #undef X
   return cudaErrorInvalidValue;
+}
+
+cudaError_t conv_fwd_fused(const uint16_t* x, const uint16_t* w, const float* bias, uint16_t* y,
+                           const Vol& g, int cin, int cout, int flags, const ConvFuse& f,
+                           cudaStream_t s) {
+  if (g_conv_kernel < 3) return cudaErrorNotSupported;
+#define X(CI, CO, F) \
+  if (cin == CI && cout == CO && f.mode == F) \
+    return ws_launch<CI, CO, F>(x, w, bias, nullptr, y, g, flags, s, f);
+  X(16, 16, kFusePool) X(16, 32, kFusePool) X(64, 32, kFuseUpadd) X(32, 16, kFuseUpadd)
+  X(16, 16, kFuseCells)
+#undef X
+  return cudaErrorNotSupported;
 }
 
 size_t conv_wgrad_ws_bytes(const Vol& g, int cin, int cout) {

@@ -63,9 +63,31 @@ bool encode_rows(CUtensorMap* m, const uint16_t* base, int channels, int64_t row
 bool encode_volume(CUtensorMap* m, const uint16_t* base, int channels, const Vol& g, int bx,
                    int by);
 
+// What the epilogue of a forward convolution does besides y (values rounded exactly
+// as by separate passes over the stored y):
+//   pool   out[V] = mean of the 2x2x2 children of V in y; g2 the coarser volume
+//          (extents of y even)
+//   upadd  out[v] = skip[v] + y[parent(v)]; g2 the finer volume
+//   cells  z[c] = rms[sample] * y[v][0] for every cell, and y is not written
+enum ConvFuseMode : int { kFuseNone = 0, kFusePool = 1, kFuseUpadd = 2, kFuseCells = 3 };
+struct ConvFuse {
+  int mode = kFuseNone;
+  Vol g2;
+  const uint16_t* skip = nullptr;
+  uint16_t* out = nullptr;
+  const float* rms = nullptr;
+  float* z = nullptr;
+};
+
 // y = epilogue(conv3x3x3(x; w) + bias): see tpfa_conv3d_bf16.
 cudaError_t conv_fwd(const uint16_t* x, const uint16_t* w, const float* bias, const uint16_t* mask,
                      uint16_t* y, const Vol& g, int cin, int cout, int flags, cudaStream_t s);
+// The same with a fused second output, for the layers of the network that have
+// one: pool (16,16) (16,32); upadd (64,32) (32,16); cells (16,16).
+// cudaErrorNotSupported when the kernel that does it is not the selected one.
+cudaError_t conv_fwd_fused(const uint16_t* x, const uint16_t* w, const float* bias, uint16_t* y,
+                           const Vol& g, int cin, int cout, int flags, const ConvFuse& f,
+                           cudaStream_t s);
 // workspace bytes conv_wgrad needs for this shape
 size_t conv_wgrad_ws_bytes(const Vol& g, int cin, int cout);
 // dw[t][co][ci] (+)= sum_v dy[v][co] x[v + off_t][ci]

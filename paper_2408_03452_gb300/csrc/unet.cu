@@ -103,12 +103,17 @@ int rms_blocks(int per) {
   return b < 1 ? 1 : (b > kRmsBlocks ? kRmsBlocks : b);
 }
 
-__global__ void sumsq_partial_kernel(const float* __restrict__ r, int n, double* partials) {
+// Blocks (x: parts of a sample, y: samples); the last block of a sample adds the
+// partial sums (strided sums, then a tree, in a fixed order) and writes its rms.
+// counters: one per sample, zero before and after.
+__global__ void rms_kernel(const float* __restrict__ r, int n, double* partials,
+                           unsigned int* counters, float* rms) {
   __shared__ double sh[kThreads];
-  const int s = blockIdx.y;
+  __shared__ bool last;
+  const int s = blockIdx.y, nb = gridDim.x;
   const float* rs = r + (size_t)s * n;
   double acc = 0.0;
-  for (int c = blockIdx.x * kThreads + threadIdx.x; c < n; c += gridDim.x * kThreads) {
+  for (int c = blockIdx.x * kThreads + threadIdx.x; c < n; c += nb * kThreads) {
     const double v = rs[c];
     acc += v * v;
   }
@@ -118,15 +123,16 @@ __global__ void sumsq_partial_kernel(const float* __restrict__ r, int n, double*
     if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partials[s * gridDim.x + blockIdx.x] = sh[0];
-}
-
-// one block per sample: strided sums, then a tree, in a fixed order
-__global__ void rms_finish_kernel(const double* partials, int nb, int n, float* rms) {
-  __shared__ double sh[kThreads];
-  const int s = blockIdx.x;
+  if (threadIdx.x == 0) {
+    partials[s * nb + blockIdx.x] = sh[0];
+    __threadfence();
+    last = atomicAdd(counters + s, 1u) == (unsigned)nb - 1u;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   double t = 0.0;
-  for (int b = threadIdx.x; b < nb; b += kThreads) t += partials[s * nb + b];
+  for (int b = threadIdx.x; b < nb; b += kThreads) t += __ldcg(partials + s * nb + b);
   sh[threadIdx.x] = t;
   __syncthreads();
   for (int w = kThreads / 2; w > 0; w >>= 1) {
@@ -136,6 +142,7 @@ __global__ void rms_finish_kernel(const double* partials, int nb, int n, float* 
   if (threadIdx.x == 0) {
     const double v = sqrt(sh[0] / n);
     rms[s] = v > 0.0 ? (float)v : 1.0f;  // a zero residual maps to a zero input
+    counters[s] = 0u;
   }
 }
 
@@ -396,6 +403,7 @@ struct tpfa_unet {
   size_t ws_bytes;
   float* rms;
   double* partials;
+  unsigned int* counters;  // blocks of rms_kernel done, per sample
   bool have_params, have_forward;
 };
 
@@ -416,6 +424,7 @@ void unet_free(tpfa_unet* u) {
   cudaFree(u->ws);
   cudaFree(u->rms);
   cudaFree(u->partials);
+  cudaFree(u->counters);
   delete u;
 }
 
@@ -443,6 +452,19 @@ int conv(tpfa_unet* u, const Vol* gv, int layer, const uint16_t* x, const uint16
   else
     e = tpfa::net::conv_fwd(x, u->wb[layer], nullptr, mask, y, g, d.cop, d.cip, flags, s);
   return e == cudaSuccess ? TPFA_OK : TPFA_ECUDA;
+}
+
+// forward convolution with the fused second output f; 1 when only y was written and
+// the pass that f stands for is still to be done
+int conv_then(tpfa_unet* u, const Vol* gv, int layer, const uint16_t* x, uint16_t* y, int flags,
+              const tpfa::net::ConvFuse& f, cudaStream_t s) {
+  const LayerDef& d = kDefs[layer];
+  const cudaError_t e = tpfa::net::conv_fwd_fused(x, u->wf[layer], u->bias[layer], y, gv[d.level],
+                                                  d.cip, d.cop, flags, f, s);
+  if (e == cudaSuccess) return TPFA_OK;
+  if (e != cudaErrorNotSupported) return TPFA_ECUDA;
+  const int rc = conv(u, gv, layer, x, nullptr, y, flags, false, s);
+  return rc ? rc : 1;
 }
 
 int layer_grads(tpfa_unet* u, int layer, const uint16_t* x, const uint16_t* dpre, float* grad,
@@ -533,7 +555,8 @@ int tpfa_unet_create(int nx, int ny, int nz, int ns, int train, tpfa_unet** out)
   }
   const size_t np = (size_t)ns * kRmsBlocks > 64 * kBiasBlocks ? (size_t)ns * kRmsBlocks
                                                                   : 64 * kBiasBlocks;
-  ok = ok && alloc_zero((void**)&u->rms, (size_t)ns * 4) && alloc_zero((void**)&u->partials, np * 8);
+  ok = ok && alloc_zero((void**)&u->rms, (size_t)ns * 4) && alloc_zero((void**)&u->partials, np * 8) &&
+       alloc_zero((void**)&u->counters, (size_t)ns * 4);
   if (!ok) {
     cudaGetLastError();
     unet_free(u);
@@ -589,30 +612,57 @@ int tpfa_unet_forward_samples(tpfa_unet* u, int ns, const float* r, const float*
   cudaStream_t s = (cudaStream_t)stream;
   const int per = g0.nx * g0.ny * g0.nz;
   const int nrb = rms_blocks(per);
-  sumsq_partial_kernel<<<dim3(nrb, g0.ns), kThreads, 0, s>>>(r, per, u->partials);
-  rms_finish_kernel<<<g0.ns, kThreads, 0, s>>>(u->partials, nrb, per, u->rms);
+  rms_kernel<<<dim3(nrb, g0.ns), kThreads, 0, s>>>(r, per, u->partials, u->counters, u->rms);
   prep_input_kernel<<<blocks_for(n0), kThreads, 0, s>>>(r, lnk, u->rms, u->in16, g0);
   if (elem_launch_ok()) return TPFA_ECUDA;
   using tpfa::net::kConvRelu;
   int rc;
   u->have_forward = false;
-  if ((rc = conv(u, gv, 0, u->in16, nullptr, u->e0, kConvRelu, false, s))) return rc;
-  pool_kernel<<<blocks_for((long long)cells(g1) * 2), kThreads, 0, s>>>(u->e0, u->p0, 16, g0, g1);
-  if ((rc = elem_launch_ok())) return rc;
-  if ((rc = conv(u, gv, 1, u->p0, nullptr, u->e1, kConvRelu, false, s))) return rc;
-  pool_kernel<<<blocks_for((long long)cells(g2) * 4), kThreads, 0, s>>>(u->e1, u->p1, 32, g1, g2);
-  if ((rc = elem_launch_ok())) return rc;
+  // pooling, upsampling with the skip and the output cells come out of the
+  // convolutions before them; the separate passes serve the kernels without that
+  tpfa::net::ConvFuse f;
+  f.mode = tpfa::net::kFusePool;
+  f.g2 = g1;
+  f.out = u->p0;
+  if ((rc = conv_then(u, gv, 0, u->in16, u->e0, kConvRelu, f, s)) > 0) {
+    pool_kernel<<<blocks_for((long long)cells(g1) * 2), kThreads, 0, s>>>(u->e0, u->p0, 16, g0, g1);
+    rc = elem_launch_ok();
+  }
+  if (rc) return rc;
+  f.g2 = g2;
+  f.out = u->p1;
+  if ((rc = conv_then(u, gv, 1, u->p0, u->e1, kConvRelu, f, s)) > 0) {
+    pool_kernel<<<blocks_for((long long)cells(g2) * 4), kThreads, 0, s>>>(u->e1, u->p1, 32, g1, g2);
+    rc = elem_launch_ok();
+  }
+  if (rc) return rc;
   if ((rc = conv(u, gv, 2, u->p1, nullptr, u->e2, kConvRelu, false, s))) return rc;
-  if ((rc = conv(u, gv, 3, u->e2, nullptr, u->d2, kConvRelu, false, s))) return rc;
-  upadd_kernel<<<blocks_for((long long)cells(g1) * 4), kThreads, 0, s>>>(u->d2, u->e1, u->s1, 32, g1, g2);
-  if ((rc = elem_launch_ok())) return rc;
-  if ((rc = conv(u, gv, 4, u->s1, nullptr, u->d1, kConvRelu, false, s))) return rc;
-  upadd_kernel<<<blocks_for((long long)n0 * 2), kThreads, 0, s>>>(u->d1, u->e0, u->s0, 16, g0, g1);
-  if ((rc = elem_launch_ok())) return rc;
+  f.mode = tpfa::net::kFuseUpadd;
+  f.g2 = g1;
+  f.skip = u->e1;
+  f.out = u->s1;
+  if ((rc = conv_then(u, gv, 3, u->e2, u->d2, kConvRelu, f, s)) > 0) {
+    upadd_kernel<<<blocks_for((long long)cells(g1) * 4), kThreads, 0, s>>>(u->d2, u->e1, u->s1, 32, g1, g2);
+    rc = elem_launch_ok();
+  }
+  if (rc) return rc;
+  f.g2 = g0;
+  f.skip = u->e0;
+  f.out = u->s0;
+  if ((rc = conv_then(u, gv, 4, u->s1, u->d1, kConvRelu, f, s)) > 0) {
+    upadd_kernel<<<blocks_for((long long)n0 * 2), kThreads, 0, s>>>(u->d1, u->e0, u->s0, 16, g0, g1);
+    rc = elem_launch_ok();
+  }
+  if (rc) return rc;
   if ((rc = conv(u, gv, 5, u->s0, nullptr, u->d0, kConvRelu, false, s))) return rc;
-  if ((rc = conv(u, gv, 6, u->d0, nullptr, u->o16, 0, false, s))) return rc;
-  out_extract_kernel<<<blocks_for(n0), kThreads, 0, s>>>(u->o16, u->rms, z, g0);
-  if ((rc = elem_launch_ok())) return rc;
+  f.mode = tpfa::net::kFuseCells;
+  f.rms = u->rms;
+  f.z = z;
+  if ((rc = conv_then(u, gv, 6, u->d0, u->o16, 0, f, s)) > 0) {
+    out_extract_kernel<<<blocks_for(n0), kThreads, 0, s>>>(u->o16, u->rms, z, g0);
+    rc = elem_launch_ok();
+  }
+  if (rc) return rc;
   // the backward pass needs the activations of every sample
   u->have_forward = ns == u->g[0].ns;
   return TPFA_OK;
