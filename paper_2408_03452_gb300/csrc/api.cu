@@ -819,6 +819,11 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
         } else {
           CK(e);
           CK(cudaEventRecord(c->ev[3], s));
+          // the residual of the corrected x right behind it: one wait for both (after
+          // a solve that ended without a correction it is the old one)
+          CK(launch_residual64(c->g, coef64, b, x, c->r64, nullptr, c->st, c->partials, c->counter,
+                               c->elem_nblocks, s));
+          launches += 1;
           rc = read_state(c, s);
           if (rc) return rc;
           float ms = 0.f;
@@ -871,17 +876,16 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
       if (inner_status == kGuard) { status = TPFA_EINTERNAL; break; }
       if (inner_status == kNonFinite) { status = TPFA_ENONFINITE; break; }
       if (inner_status == kBreakdown && hs->iter == 0) { status = TPFA_EBREAKDOWN; break; }
-      // x += e / scale;  r64 = b - A x
-      if (!resident) {  // the resident kernel has added its correction
-        CK(launch_correct(c->g, vecs, x, c->st, s));
-        launches += 1;
-      }
-      CK(launch_residual64(c->g, coef64, b, x, c->r64, nullptr, c->st, c->partials, c->counter,
-                           c->elem_nblocks, s));
-      launches += 1;
+      // x += e / scale;  r64 = b - A x  (the resident path has done both)
       ++outer;
-      rc = read_state(c, s);
-      if (rc) return rc;
+      if (!resident) {
+        CK(launch_correct(c->g, vecs, x, c->st, s));
+        CK(launch_residual64(c->g, coef64, b, x, c->r64, nullptr, c->st, c->partials, c->counter,
+                             c->elem_nblocks, s));
+        launches += 2;
+        rc = read_state(c, s);
+        if (rc) return rc;
+      }
       rr = hs->rr64;
       rel = sqrt(rr / bb);
       if (!isfinite(rel)) { status = TPFA_ENONFINITE; break; }

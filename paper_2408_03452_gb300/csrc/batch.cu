@@ -51,13 +51,13 @@ bool batch_tma(const tpfa_batch* b) {
 }
 
 // The inner solves run in the resident kernel when every instance fits on the
-// chip, unless a sweep, a tile or z-runs are asked for.
+// chip, unless a sweep or a tile is asked for (z-runs are those of the sweeps).
 bool batch_resident(const tpfa_batch* b) {
   if (b->sweep_sel != 0 || b->tma_tile != 0 || b->resident_off || b->ninst > kResMaxProb)
     return false;
   ResPlan p;
   for (int i = 0; i < b->ninst; ++i)
-    if (b->zc_req[i] > 0 || !plan_resident(b->g[i], b->num_sms, true, &p)) return false;
+    if (!plan_resident(b->g[i], b->num_sms, true, &p)) return false;
   return true;
 }
 
