@@ -382,7 +382,7 @@ double ctx_option(const tpfa_ctx* c, int option) {
 // The TMA-staged operator's plan for tpfa_apply's arguments (coef, p 16-byte
 // aligned; dots: the variant fused with the flexible-CG dot products), or
 // false when tpfa_apply would take the cp.async kernel.
-bool ctx_apply_tma_plan(const tpfa_ctx* c, TmaPlan* p, Grid* g, bool dots) {
+bool ctx_apply_tma_plan(const tpfa_ctx* c, TmaPlan* p, Grid* g, int dots) {
   if (!use_tma_apply(c, false)) return false;
   *g = c->g;
   *p = plan_tma(c->g, 0, c->zc, c->num_sms, false, false, true, dots);

@@ -193,11 +193,29 @@ __global__ void finish_dots_kernel(const double* __restrict__ part, int nb, int 
   }
 }
 
+// The network term u on the 2^lev coarser grid (each cell has its ancestor's
+// value); v = nullptr: u is given on the fine grid.  Extents of fewer than 2^31
+// cells, nx a multiple of 4, all divisible by 2^lev.
+struct CoarseU {
+  const float* v;
+  int lev, nx4, ny;   // fine extents: nx / 4, ny
+  int cx, cplane;     // coarse extents: row, plane
+
+  // of the four cells of float4 i
+  __device__ __forceinline__ float4 at(int i) const {
+    const int row = i / nx4, x = 4 * (i - row * nx4), z = row / ny, y = row - z * ny;
+    const float* b = v + (int64_t)(z >> lev) * cplane + (y >> lev) * cx;
+    const float lo = __ldg(b + (x >> lev)), hi = lev > 1 ? lo : __ldg(b + (x >> 1) + 1);
+    return make_float4(lo, lo, hi, hi);
+  }
+};
+
 // p = w + c u + sum_j beta_j p_j; partial p'r (four elements per step)
 template <int M>
 __global__ void dir_kernel(const float* __restrict__ r, const float* __restrict__ dinv,
-                           const float* __restrict__ u, Dirs pd, const Scal* __restrict__ sc,
-                           int jac, int net, float* p, int64_t n, double* part) {
+                           const float* __restrict__ u, CoarseU uc, Dirs pd,
+                           const Scal* __restrict__ sc, int jac, int net, float* p, int64_t n,
+                           double* part) {
   // p may be the oldest retained direction (read, then overwritten, per element)
   const float c = (float)sc->c;
   float beta[M > 0 ? M : 1];
@@ -217,7 +235,9 @@ __global__ void dir_kernel(const float* __restrict__ r, const float* __restrict_
   for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * kT) {
     const float4 r4 = reinterpret_cast<const float4*>(r)[i];
     const float4 d4 = jac ? reinterpret_cast<const float4*>(dinv)[i] : z4;
-    const float4 u4 = net ? reinterpret_cast<const float4*>(u)[i] : z4;
+    const float4 u4 = !net              ? z4
+                      : uc.v != nullptr ? uc.at((int)i)
+                                        : reinterpret_cast<const float4*>(u)[i];
     float4 p4[M > 0 ? M : 1];
 #pragma unroll
     for (int j = 0; j < M; ++j) p4[j] = reinterpret_cast<const float4*>(pd.v[j])[i];
@@ -337,11 +357,11 @@ void launch_dots(int m, int nb, cudaStream_t s, const float* r, const float* coe
 }
 
 void launch_dir(int m, int nb, cudaStream_t s, const float* r, const float* coef, const float* u,
-                const Dirs& pd, const Scal* sc, int jac, int net, float* p, int64_t n,
+                const CoarseU& uc, const Dirs& pd, const Scal* sc, int jac, int net, float* p, int64_t n,
                 double* part) {
   switch (m) {
 #define X(M) \
-  case M: dir_kernel<M><<<nb, kT, 0, s>>>(r, coef, u, pd, sc, jac, net, p, n, part); break;
+  case M: dir_kernel<M><<<nb, kT, 0, s>>>(r, coef, u, uc, pd, sc, jac, net, p, n, part); break;
     TPFA_FCG_M0(X)
 #undef X
     default: break;
@@ -506,8 +526,8 @@ struct Result {
 
 enum PrecMode { kIdentity = 0, kJacobi = 1, kBlend = 2 };
 
-// the network term u of the blend (into w.z) and, unless the fused operator
-// takes it, A u (into w.au, u'Au into w.uau)
+// the network term u of the blend: into w.z with A u (into w.au, u'Au into w.uau)
+// unless the fused operator takes it, which reads a coarser u where it is
 int network_term(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, Work& w,
                  bool with_apply) {
   int rc;
@@ -517,9 +537,12 @@ int network_term(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* ln
                            nullptr, 0, 0, 0);
     rc = tpfa_unet_forward(net, w.rl[L], w.lnkc, w.ul[L], w.s);
     if (rc) return rc;
-    launch_prolong_levels(L, w.nb, w.s, w.ul[L], w.z, w.dims[0], w.dims[1], w.dims[2], 1, nullptr,
-                          0, 0, 0, true);
-    w.launches += 17;
+    w.launches += 16;
+    if (with_apply) {
+      launch_prolong_levels(L, w.nb, w.s, w.ul[L], w.z, w.dims[0], w.dims[1], w.dims[2], 1,
+                            nullptr, 0, 0, 0, true);
+      ++w.launches;
+    }
   } else {
     rc = tpfa_unet_forward(net, w.r, lnk, w.z, w.s);
     if (rc) return rc;
@@ -536,7 +559,7 @@ int setup_fused(const tpfa_ctx* c, const float* coef, Work& w) {
   using namespace tpfa;
   TmaPlan p;
   Grid g;
-  if (!ctx_apply_tma_plan(c, &p, &g, true) || reinterpret_cast<uintptr_t>(coef) % 16 != 0 ||
+  if (!ctx_apply_tma_plan(c, &p, &g, w.levels > 0 ? 2 : 1) || reinterpret_cast<uintptr_t>(coef) % 16 != 0 ||
       w.m > kMaxDirs)
     return TPFA_OK;
   const int per = 4 + 2 * w.m;
@@ -610,12 +633,23 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
     // with the network, the TMA-staged operator A u also forms the dot
     // products (A u itself is not stored)
     const bool fused = with_net && w.fused && stored <= tpfa::kApplyMaxDirs;
+    CoarseU uc{};
+    if (fused && w.levels > 0) {
+      const int L = w.levels;
+      uc.v = w.ul[L];
+      uc.lev = L;
+      uc.nx4 = w.dims[0] / 4;  // the fused operator's grids have nx % 4 == 0
+      uc.ny = w.dims[1];
+      uc.cx = w.dims[0] >> L;
+      uc.cplane = uc.cx * (w.dims[1] >> L);
+    }
     if (with_net) {
       int rc = network_term(c, net, coef, lnk, w, !fused);
       if (rc) return rc;
       if (fused) {
         if (launch_apply_dots_tma_batch(w.finst, 1, w.fblocks, 0, w.fact, 1, w.own0, qmap, stored,
-                                        w.uau, w.fdots, w.fpart, w.fcnt, w.s) != cudaSuccess)
+                                        w.uau, w.fdots, w.fpart, w.fcnt, w.s, uc.v, uc.lev) !=
+            cudaSuccess)
           return TPFA_ECUDA;
         ++w.launches;
       }
@@ -631,7 +665,7 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
     }
     float* p = w.P + (size_t)head * w.slot_stride();
     float* q = w.Q + (size_t)head * w.slot_stride();
-    launch_dir(stored, w.nb, w.s, w.r, w.dinv, w.z, pd, w.sc, jac, with_net, p, w.n, w.part);
+    launch_dir(stored, w.nb, w.s, w.r, w.dinv, w.z, uc, pd, w.sc, jac, with_net, p, w.n, w.part);
     int rc = tpfa_apply(c, coef, p, q, w.pq, w.s);
     if (rc) return rc;
     finish_alpha_kernel<<<1, kT, 0, w.s>>>(w.part, w.nb, w.pq, w.sc, head);

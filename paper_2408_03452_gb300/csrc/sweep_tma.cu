@@ -395,12 +395,13 @@ cg_sweep_tma_kernel(const __grid_constant__ TmaArgs a) {
 constexpr int kPX = 40;  // p box width: X0-4 .. X0+35
 
 // NE: further FP32 fields staged for the own cells only ([TY rows][32 floats]
-// from (X0, Y0) per own plane), for the fused dot products
-template <int W, int VY, bool B16, int NE = 0>
+// from (X0, Y0) per own plane), for the fused dot products; P: p is staged (it is
+// not when the kernel reads it from a coarser grid)
+template <int W, int VY, bool B16, int NE = 0, bool P = true>
 struct ApplyLayout {
   using RC = Rec<B16, false>;
   static constexpr int TY = W * VY;
-  static constexpr int kPBytes = (TY + 2) * kPX * 4;
+  static constexpr int kPBytes = P ? (TY + 2) * kPX * 4 : 0;
   static constexpr int kRecBytes = (TY + 1) * RC::kX * RC::kBytes;
   static constexpr int kOwnBytes = TY * 32 * 4;  // one own-cell field
   static constexpr int al(int b) { return (b + 127) / 128 * 128; }
@@ -412,9 +413,9 @@ struct ApplyLayout {
   static constexpr uint32_t kTxOwn = kTx + NE * kOwnBytes;  // own planes
 };
 
-template <int W, int VY, int S, bool B16, int NE = 0>
+template <int W, int VY, int S, bool B16, int NE = 0, bool P = true>
 constexpr int apply_smem_bytes() {
-  return S * ApplyLayout<W, VY, B16, NE>::kStage + 2 * S * 8 + 128;
+  return S * ApplyLayout<W, VY, B16, NE, P>::kStage + 2 * S * 8 + 128;
 }
 
 struct ApplyArgs {
@@ -438,22 +439,33 @@ struct ApplyArgs {
   // Flexible-CG dot products fused into the batched operator (DM >= 0 in the
   // kernel): with u the input, q = A u (not stored) and w = M^-1 r, per
   // instance u'q, u'r, q'w, w'q_j and u'q_j (j < DM) into
-  // dots[id * kApplyDotsStride + ...], u'q also into pAp[id].  r, M^-1 and
-  // the q_j are staged like p, own cells only, from the instance's maps
-  // own0 (r), own0 + 1 (M^-1) and own0 + 2 + qmap[j].
+  // dots[id * kApplyDotsStride + ...], u'q also into pAp[id].  r and the q_j
+  // are staged like p, own cells only, from the instance's maps own0 (r) and
+  // own0 + 2 + qmap[j]; M^-1 = 1 / D comes from the cell's record.
   int own0;
   int qmap[kApplyMaxDirs];
   double* dots;
+  // the input on the 2^lev coarser grid, each cell having its ancestor's value
+  // (CRS in the kernel; one instance, extents divisible by 2^lev)
+  const float* uc;
+  int lev;
 };
 
-template <int W, int VY, int S, bool B16, bool BATCH, int DM = -1>
+// CRS: the input u is constant on the blocks of a coarser grid (a.uc) and read from
+// there through the caches, a plane ahead; neither a fine copy nor its traffic is
+// needed, and a plane of the ring is consumed as soon as it has landed (no wait for
+// the one above it).  256^3 with two directions: 124 us + 15 for the fine copy with
+// u and M^-1 staged, 106 without (four blocks per SM; with a fourth stage and three
+// blocks 109, with 8 warps of two rows 122).
+template <int W, int VY, int S, bool B16, bool BATCH, int DM = -1, bool CRS = false>
 __global__ void __launch_bounds__((W + 1) * 32)
 apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
   static_assert(!BATCH || !B16, "batched operator: FP32 records");
   static_assert(DM < 0 || (BATCH && DM <= kApplyMaxDirs), "fused dots: batched, few directions");
-  constexpr int NE = DM < 0 ? 0 : 2 + DM;       // own-cell fields: r, M^-1, q_j
+  static_assert(!CRS || (DM >= 0 && VY % 2 == 0), "coarse input: fused dots, rows in pairs");
+  constexpr int NE = DM < 0 ? 0 : 1 + DM;       // own-cell fields: r, q_j
   constexpr int NV = DM < 0 ? 1 : 3 + 2 * DM;   // reduced values
-  using LY = ApplyLayout<W, VY, B16, NE>;
+  using LY = ApplyLayout<W, VY, B16, NE, !CRS>;
   using RC = Rec<B16, false>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* smem =
@@ -494,7 +506,7 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
   const int X0 = 32 * bx, Y0 = LY::TY * by;
   const int64_t z0 = (int64_t)bz * zc;
   const int64_t z1 = min(z0 + (int64_t)zc, g.nz);
-  const int L = (int)(z1 - z0) + 2;  // planes z0-1 .. z1
+  const int L = (int)(z1 - z0) + (CRS ? 1 : 2);  // planes z0-1 .. z1 (CRS: z1 - 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -521,18 +533,17 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
           break;
         }
         const int z = (int)(z0 - 1 + j);
-        const bool own = NE > 0 && j >= 1 && j <= L - 2;
+        const bool own = NE > 0 && j >= 1 && z < z1;
         unsigned char* sb = smem + s * LY::kStage;
         mbar_expect_tx(&full[s], own ? LY::kTxOwn : LY::kTx);
         // x coordinates in 4-byte elements, multiples of 4 (16 bytes)
-        tma_3d(sb + LY::kP, mp, &full[s], X0 - 4, Y0 - 1, z);
+        if (!CRS) tma_3d(sb + LY::kP, mp, &full[s], X0 - 4, Y0 - 1, z);
         tma_3d(sb + LY::kC, mc, &full[s], (RC::kBytes / 4) * (X0 - RC::kC0), Y0 - 1, z);
         if (own) {
           tma_3d(sb + LY::kE, mown, &full[s], X0, Y0, z);                        // r
-          tma_3d(sb + LY::kE + LY::kOwnBytes, mown + 1, &full[s], X0, Y0, z);    // M^-1
 #pragma unroll
           for (int q = 0; q < (DM > 0 ? DM : 0); ++q)
-            tma_3d(sb + LY::kE + (2 + q) * LY::kOwnBytes, mown + 2 + a.qmap[q], &full[s], X0, Y0,
+            tma_3d(sb + LY::kE + (1 + q) * LY::kOwnBytes, mown + 2 + a.qmap[q], &full[s], X0, Y0,
                    z);
         }
         issued = j + 1;
@@ -555,9 +566,58 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
     const int hc = lane == 0 ? 3 : 36;  // p box column of this lane's x-halo cell
     float* out = a.Ap + off;
 
+    // CRS: u of this lane's column at rows -1, 0, 2, .., VY (the rows of a pair have
+    // one ancestor) and of the x-halo cell at the pairs; zero outside the grid, as
+    // the copies give it
+    constexpr int NR = VY / 2 + 2;
+    struct Coarse {
+      float v[NR], h[VY / 2];
+    };
+    int co[NR], ch[VY / 2];
+    int64_t cplane = 0;
+    if constexpr (CRS) {
+      const int cx = (int)(g.nx >> a.lev);
+      cplane = (g.nx >> a.lev) * (g.ny >> a.lev);
+      const int hx = lane == 0 ? X0 - 1 : lane == 31 ? X0 + 32 : -1;
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        const int y = Y0 + jw + (k == 0 ? -1 : 2 * (k - 1));
+        const bool iny = y >= 0 && y < g.ny;
+        co[k] = inx && iny ? (y >> a.lev) * cx + (gx >> a.lev) : -1;
+        if (k >= 1 && k <= VY / 2)
+          ch[k - 1] = hx >= 0 && hx < g.nx && iny ? (y >> a.lev) * cx + (hx >> a.lev) : -1;
+      }
+    }
+    auto fetch = [&](int j) {
+      Coarse u{};
+      const int64_t z = z0 - 1 + j;
+      if (z >= 0 && z < g.nz) {
+        const float* base = a.uc + (z >> a.lev) * cplane;
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+          if (co[k] >= 0) u.v[k] = __ldg(base + co[k]);
+#pragma unroll
+        for (int k = 0; k < VY / 2; ++k)
+          if (ch[k] >= 0) u.h[k] = __ldg(base + ch[k]);
+      }
+      return u;
+    };
+    Coarse un{};  // of the next plane to load
+
     // p of plane j for rows -1..VY of this lane's column, and of the x-halo
     // cell of the own rows
     auto load = [&](int j, float (&P)[VY + 2], float (&H)[VY]) {
+      if constexpr (CRS) {
+        P[0] = un.v[0];
+        P[VY + 1] = un.v[NR - 1];
+#pragma unroll
+        for (int jj = 0; jj < VY; ++jj) {
+          P[1 + jj] = un.v[1 + jj / 2];
+          H[jj] = un.h[jj / 2];
+        }
+        un = fetch(j + 1);
+        return;
+      }
       const float* sp = reinterpret_cast<const float*>(smem + (j % S) * LY::kStage + LY::kP);
 #pragma unroll
       for (int jj = -1; jj <= VY; ++jj) {
@@ -576,6 +636,7 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
 
     float Pm[VY], P0[VY + 2], H0[VY], Tzm[VY];
     int64_t zdone = z0;  // first plane of the run not yet written
+    if constexpr (CRS) un = fetch(0);
     if (!wait_full(0)) fault = true;
     if (!fault) {  // plane z0 - 1: p below the first plane, and its Tz
       float Pt[VY + 2], Ht[VY];
@@ -586,14 +647,14 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
         Tzm[jj] = srec<B16>(smem + LY::kC, (jw + jj + 1) * RC::kX + lane + RC::kC0).z;
       }
       release(0);
-      if (!wait_full(1)) fault = true;
+      if (!CRS && !wait_full(1)) fault = true;
     }
     if (!fault) load(1, P0, H0);
 
     for (int64_t z = z0; z < z1 && !fault; ++z) {
       const int jc = (int)(z - z0) + 1;  // plane z
       const int jf = jc + 1;             // plane z + 1
-      if (!wait_full(jf)) { fault = true; break; }
+      if (!wait_full(CRS ? jc : jf)) { fault = true; break; }
       float Pp[VY + 2], Hp[VY];
       load(jf, Pp, Hp);
       const unsigned char* sb = smem + (jc % S) * LY::kStage;
@@ -625,13 +686,13 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
             // the dot products of the flexible-CG step at this cell (u = pc)
             const float* se = reinterpret_cast<const float*>(sb + LY::kE) + (jw + jj) * 32 + lane;
             const float rv = se[0];
-            const float wv = rv * se[LY::kOwnBytes / 4];
+            const float wv = rv * (1.0f / cf.w);
             sd[0] = fmaf(pc, q, sd[0]);
             sd[1] = fmaf(pc, rv, sd[1]);
             sd[2] = fmaf(q, wv, sd[2]);
 #pragma unroll
             for (int k = 0; k < (DM > 0 ? DM : 0); ++k) {
-              const float qv = se[(2 + k) * (LY::kOwnBytes / 4)];
+              const float qv = se[(1 + k) * (LY::kOwnBytes / 4)];
               sd[3 + k] = fmaf(wv, qv, sd[3 + k]);
               sd[3 + DM + k] = fmaf(pc, qv, sd[3 + DM + k]);
             }
@@ -654,7 +715,7 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
       for (int jj = 0; jj < VY + 2; ++jj) P0[jj] = Pp[jj];
     }
     if (!fault) {
-      release(L - 1);  // the last plane (z1) was only read
+      if (!CRS) release(L - 1);  // the last plane (z1) was only read
     } else {
       // a copy that never landed: the cells this warp did not write become
       // NaN, and so do the dot products, so that the failure cannot pass
@@ -786,15 +847,18 @@ int apply_blocks_per_sm_t() {
 }
 
 // stages of the operator's ring: 4; 3 with the fused dot products, whose
-// stages also hold the own-cell boxes (three blocks per SM instead of two)
+// stages also hold the own-cell boxes (three blocks per SM instead of two; four
+// where u is read from a coarser grid)
 template <int DM>
 constexpr int apply_stages() {
   return DM < 0 ? 4 : 3;
 }
 
+template <bool CRS>
 int apply_dots_blocks_per_sm_t() {
-  constexpr int smem = apply_smem_bytes<4, 4, apply_stages<2>(), false, 4>();
-  auto fn = apply_tma_kernel<4, 4, apply_stages<2>(), false, true, 2>;
+  constexpr int S = apply_stages<2>();
+  constexpr int smem = apply_smem_bytes<4, 4, S, false, 3, !CRS>();
+  auto fn = apply_tma_kernel<4, 4, S, false, true, 2, CRS>;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return 0;
   int nb = 0;
@@ -803,11 +867,11 @@ int apply_dots_blocks_per_sm_t() {
   return nb;
 }
 
-template <bool B16, bool BATCH, int DM = -1>
+template <bool B16, bool BATCH, int DM = -1, bool CRS = false>
 cudaError_t launch_apply_t(const ApplyArgs& a, int64_t nblocks, cudaStream_t s) {
   constexpr int S = apply_stages<DM>();
-  constexpr int smem = apply_smem_bytes<4, 4, S, B16, DM < 0 ? 0 : 2 + DM>();
-  auto fn = apply_tma_kernel<4, 4, S, B16, BATCH, DM>;
+  constexpr int smem = apply_smem_bytes<4, 4, S, B16, DM < 0 ? 0 : 1 + DM, !CRS>();
+  auto fn = apply_tma_kernel<4, 4, S, B16, BATCH, DM, CRS>;
   // the attribute is set on the first launch of a device (it costs as much as the
   // rest of the launch)
   static std::atomic<uint64_t> set{0};
@@ -901,11 +965,11 @@ bool tma_sweep_ok(const Grid& g, bool b16, bool jac) {
 int tma_tile_count() { return kNumTmaTiles; }
 
 TmaPlan plan_tma(const Grid& g, int tile, int zc_opt, int num_sms, bool b16, bool jac,
-                 bool apply, bool dots) {
+                 bool apply, int dots) {
   TmaPlan p{};
   if (tile < 0 || tile >= kNumTmaTiles || b16 || jac || apply) tile = 0;
   if (apply) jac = false;
-  p.dots = apply && dots && !b16;
+  p.dots = apply && !b16 ? dots : 0;
   const TileShape ts = kTmaTiles[tile];
   p.tile = tile;
   p.b16 = b16;
@@ -952,20 +1016,20 @@ TmaPlan plan_tma(const Grid& g, int tile, int zc_opt, int num_sms, bool b16, boo
 int tma_blocks_per_sm(const TmaPlan& p) {
   // host-side occupancy queries cost microseconds; the answer is fixed per
   // device and kernel, so it is kept (index: device, kernel variant)
-  constexpr int kDevs = 64, kVariants = 3 + kNumTmaTiles + 3;
+  constexpr int kDevs = 64, kVariants = 3 + kNumTmaTiles + 4;
   static int memo[kDevs][kVariants] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     dev = -1;
   }
-  const int var = p.dots ? 3 + kNumTmaTiles + 2
+  const int var = p.dots ? 3 + kNumTmaTiles + 1 + p.dots
                   : p.apply ? 3 + kNumTmaTiles + (p.b16 ? 1 : 0)
                   : (p.b16 && p.jac) ? 0 : p.b16 ? 1 : p.jac ? 2 : 3 + p.tile;
   if (dev >= 0 && dev < kDevs && var >= 0 && var < kVariants && memo[dev][var] > 0)
     return memo[dev][var];
   int nb = 0;
-  if (p.dots) nb = apply_dots_blocks_per_sm_t();
+  if (p.dots) nb = p.dots == 2 ? apply_dots_blocks_per_sm_t<true>() : apply_dots_blocks_per_sm_t<false>();
   else if (p.apply) nb = p.b16 ? apply_blocks_per_sm_t<true>() : apply_blocks_per_sm_t<false>();
   else if (p.b16 && p.jac) nb = tma_blocks_per_sm_t<4, 4, 4, true, true>();
   else if (p.b16) nb = tma_blocks_per_sm_t<4, 4, 4, true, false>();
@@ -1094,8 +1158,8 @@ bool make_own_maps(const Grid& g, const TmaPlan& p, const float* const* in, int 
 cudaError_t launch_apply_dots_tma_batch(const TmaInst* inst, int ninst, int64_t nblocks,
                                         int which, const int* act, int need, int own0,
                                         const int* qmap, int ndirs, double* uq, double* dots,
-                                        double* partials, unsigned int* counters,
-                                        cudaStream_t s) {
+                                        double* partials, unsigned int* counters, cudaStream_t s,
+                                        const float* uc, int lev) {
   if (ndirs < 0 || ndirs > kApplyMaxDirs) return cudaErrorInvalidValue;
   ApplyArgs a;
   memset(&a, 0, sizeof(a));
@@ -1110,6 +1174,19 @@ cudaError_t launch_apply_dots_tma_batch(const TmaInst* inst, int ninst, int64_t 
   a.own0 = own0;
   for (int j = 0; j < ndirs; ++j) a.qmap[j] = qmap[j];
   a.dots = dots;
+  if (uc != nullptr) {
+    if (ninst != 1) return cudaErrorInvalidValue;
+    a.uc = uc;
+    a.lev = lev;
+    switch (ndirs) {
+      case 0: return launch_apply_t<false, true, 0, true>(a, nblocks, s);
+      case 1: return launch_apply_t<false, true, 1, true>(a, nblocks, s);
+      case 2: return launch_apply_t<false, true, 2, true>(a, nblocks, s);
+      case 3: return launch_apply_t<false, true, 3, true>(a, nblocks, s);
+      case 4: return launch_apply_t<false, true, 4, true>(a, nblocks, s);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   switch (ndirs) {
     case 0: return launch_apply_t<false, true, 0>(a, nblocks, s);
     case 1: return launch_apply_t<false, true, 1>(a, nblocks, s);

@@ -82,7 +82,7 @@ struct TmaPlan {
   int tile;    // index of the (w, vy, stages) choice
   bool b16, jac;
   bool apply;  // the operator application q = A p (tile 0), not a CG sweep
-  bool dots;   // ... fused with the flexible-CG dot products (its own ring depth)
+  int dots;    // ... fused with the flexible-CG dot products (its own ring depth), 2: of a coarser u
   int w, vy, stages, zc;
   int64_t nbx, nby, nbz, nblocks;
 };
@@ -96,7 +96,7 @@ struct TmaMaps {
 bool tma_sweep_ok(const Grid& g, bool b16, bool jac);
 int tma_tile_count();
 TmaPlan plan_tma(const Grid& g, int tile, int zc_opt, int num_sms, bool b16, bool jac,
-                 bool apply = false, bool dots = false);
+                 bool apply = false, int dots = 0);
 int tma_blocks_per_sm(const TmaPlan& p);
 bool make_tma_maps(const Grid& g, const TmaPlan& p, const void* coef, const float* dinv,
                    const CgVecs& v, TmaMaps* m);
@@ -137,9 +137,11 @@ bool make_apply_maps(const Grid& g, const TmaPlan& p, const void* coef, const fl
 // (act[id] & need) == need, with u its input `which`, q = A u and w = M^-1 r:
 // u'q into uq[id] and, at dots + id * kApplyDotsStride, u'q, u'r, q'w, then
 // w'q_j and u'q_j (j < ndirs <= kApplyMaxDirs).  The instance's maps from
-// index own0 on are own-cell maps (make_own_maps) of r, M^-1 and the
-// direction slots; q_j is slot qmap[j].  partials: 3 + 2 ndirs doubles per
-// block.
+// index own0 on are own-cell maps (make_own_maps) of r, M^-1 (not read: it is
+// 1 / D of the records) and the direction slots; q_j is slot qmap[j].
+// partials: 3 + 2 ndirs doubles per block.  With uc (one instance only) u is
+// the value of each cell's ancestor on the 2^lev coarser grid, lev >= 1, and
+// input `which` is not read.
 constexpr int kApplyMaxDirs = 4;
 constexpr int kApplyDotsStride = 3 + 2 * kApplyMaxDirs;
 bool make_own_maps(const Grid& g, const TmaPlan& p, const float* const* in, int nin,
@@ -147,8 +149,8 @@ bool make_own_maps(const Grid& g, const TmaPlan& p, const float* const* in, int 
 cudaError_t launch_apply_dots_tma_batch(const TmaInst* inst, int ninst, int64_t nblocks,
                                         int which, const int* act, int need, int own0,
                                         const int* qmap, int ndirs, double* uq, double* dots,
-                                        double* partials, unsigned int* counters,
-                                        cudaStream_t s);
+                                        double* partials, unsigned int* counters, cudaStream_t s,
+                                        const float* uc = nullptr, int lev = 0);
 // Batched operator through the TMA-staged kernel: inst[k].maps as from
 // make_apply_maps, input `which`; the table may list any subset of the batch's
 // instances (inst[k].id, bstart consecutive through the table); only instances
@@ -276,7 +278,7 @@ std::mutex& resident_mutex(int device);
 int64_t ctx_cells(const tpfa_ctx* c);
 void ctx_dims(const tpfa_ctx* c, int64_t* d3);
 double ctx_option(const tpfa_ctx* c, int option);
-bool ctx_apply_tma_plan(const tpfa_ctx* c, TmaPlan* p, Grid* g, bool dots = false);
+bool ctx_apply_tma_plan(const tpfa_ctx* c, TmaPlan* p, Grid* g, int dots = 0);
 bool dev_ok(const void* p, size_t bytes, size_t align, int device);
 bool opt_dev_ok(const void* p, size_t bytes, size_t align, int device);
 int elem_blocks(const Grid& g, int num_sms);
