@@ -86,7 +86,8 @@ typedef struct tpfa_ctx tpfa_ctx;
 enum tpfa_option {
   TPFA_OPT_INNER_RTOL = 1,   /* lower bound on the inner FP32 CG relative tolerance (default 1e-6) */
   TPFA_OPT_MAX_OUTER = 2,    /* maximum FP64 refinement steps (default 20)                        */
-  TPFA_OPT_LOOP = 3,         /* 0 = CUDA-graph while node (default), 1 = host-polled graph chunks */
+  TPFA_OPT_LOOP = 3,         /* loop of the sweeps: 0 = CUDA-graph while node (default), 1 =
+                                host-polled graph chunks (resident solves have no host loop)      */
   TPFA_OPT_TILE_VY = 4,      /* rows per warp in the stencil sweeps: 4 or 8 (default 4; 8 sets 3 stages) */
   TPFA_OPT_TILE_ZC = 5,      /* planes per warp in the stencil sweeps, 0 = automatic              */
   TPFA_OPT_CHUNK = 6,        /* CG iterations per graph launch when TPFA_OPT_LOOP = 1 (default 32) */
@@ -103,9 +104,10 @@ enum tpfa_option {
   TPFA_OPT_FCG_FALLBACK = 14, /* fcg_solve with a network, after breakdown or stagnation:
                                 0 = unpreconditioned CG (default); 1 = drop the network, keep
                                 Jacobi                                                            */
-  TPFA_OPT_SWEEP = 15,       /* CG sweep kernel of cg_solve: 0 = automatic (default: the TMA-staged
-                                sweep for unpreconditioned CG on FP32 records, else the
-                                cp.async-staged sweep), 1 = cp.async-staged sweep, 2 = TMA-staged
+  TPFA_OPT_SWEEP = 15,       /* CG kernel of the solves: 0 = automatic (default: the resident
+                                kernel where the grid fits on the chip, see cg_solve; else the
+                                TMA-staged sweep where it can run, else the cp.async-staged
+                                sweep), 1 = cp.async-staged sweep, 2 = TMA-staged
                                 sweep (cg_solve returns TPFA_EINVAL where it cannot run: BF16
                                 records, Jacobi, or a driver without the tensor-map encoder).
                                 The TMA-staged sweep keeps r, q, p, x of a cell in one 16-byte
@@ -118,7 +120,9 @@ enum tpfa_option {
                                 2 = 8 x 4, 3 stages; 3 = 4 x 2, 6 stages                         */
 };
 
-/* The stencil-sweep tiling a context uses, for inspection and tests.
+/* The stencil-sweep tiling a context uses, for inspection and tests (a grid
+ * that is solved by the resident kernel reports the sweep it would take
+ * otherwise).
  * which: 0 = the CG loop of cg_solve with FP32 records, 1 = the CG loop of
  * cg_solve_bf16, 2 = tpfa_apply, 3 = tpfa_apply_bf16 (for 16-byte aligned
  * arguments).  out: host array of 6 values:
@@ -226,7 +230,14 @@ int tpfa_residual64(tpfa_ctx* ctx, const double* coef64, const double* b, const 
  * Solve A x = b (Alg. 1) to ||b - A x||_2 <= tol ||b||_2 measured in FP64.
  * Inner solver: unpreconditioned CG in FP32 on coef, one fused sweep per
  * iteration (operator, both vector updates and the single reduction), run
- * inside a CUDA graph whose while-loop condition is set on the device.
+ * inside a CUDA graph whose while-loop condition is set on the device.  Grids
+ * that fit on the chip (about one 32 x 16 x 32 brick per SM, 2.5 M cells on
+ * GB300) run a whole inner solve as one cooperative launch with the vectors in
+ * registers and shared memory, unless TPFA_OPT_SWEEP or TPFA_OPT_TILE_VY asks
+ * for a sweep; it needs a few MB of context memory, 12 bytes per cell more
+ * above 1.2 M cells, and falls back to the sweeps where that cannot be had.
+ * An explicit TPFA_OPT_TILE_ZC takes the bricks of a batch, so that results
+ * are bit-identical to it.
  * Outer loop: FP64 residual with coef64, FP32 correction solve, FP64 update
  * (iterative refinement) until tol is met.
  * coef    dev 4N floats; coef64 dev 4N doubles (both from tpfa_build_trans).
@@ -286,7 +297,10 @@ int cg_solve_bf16(tpfa_ctx* ctx, const uint16_t* coef16, const double* coef64, c
  * innermost inside the instance.  The CG iterations of all instances run as
  * one sweep launch per iteration inside one CUDA-graph while loop; each
  * instance has its own scalars and convergence flag, and the blocks of a
- * converged instance return immediately.
+ * converged instance return immediately.  A batch whose instances each fit on
+ * the chip (1.2 M cells on GB300) runs its inner solves in one cooperative
+ * launch instead, whose SMs take the instances one after another (see cg_solve
+ * for when; explicit z-runs are the sweeps' and do not matter there).
  */
 typedef struct tpfa_batch tpfa_batch;
 
@@ -375,13 +389,13 @@ int tpfa_conv3d_wgrad_bf16(const uint16_t* x, const uint16_t* dy, float* dw, int
  *     (dy, dx) offset to the three output planes an input plane feeds
  *     (accumulators in a TMEM ring), so every staged input row is read by the
  *     tensor core 9 instead of 27 times;
- * 4 = kernel 2 with warp-specialised roles: a copy warp fills the ring of
- *     triples, one thread issues the MMAs, four epilogue warps drain a ring
- *     of TMEM accumulators, joined by mbarriers instead of block barriers;
- * 3 = per layer shape, the fastest on GB300 (default): 1 for 32 -> 16, 4 for
- *     the others.
- * (cin, cout) = (64, 32) always uses kernel 0.  Returns TPFA_EINVAL for
- * another value. */
+ * 4 = kernel 2 with warp-specialised roles on tiles of 8 x 16 voxels: one
+ *     tensor-map copy per input plane fills swizzled voxel rows that the tensor
+ *     core reads directly, one warp issues the MMAs, four epilogue warps drain a
+ *     ring of TMEM accumulators, joined by mbarriers instead of block barriers;
+ * 3 = the fastest on GB300 for every layer shape (default): 4.
+ * Kernels 1 and 2 do not cover (cin, cout) = (64, 32), which takes kernel 0
+ * there.  Returns TPFA_EINVAL for another value. */
 int tpfa_conv3d_select(int kernel);
 /* Waits for the stream; TPFA_EINTERNAL (and clears the flag) if any
  * tensor-core wait of the convolution kernels gave up since the last call. */

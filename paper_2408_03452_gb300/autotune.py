@@ -16,7 +16,9 @@ so it is measured on the real solve:
      fixed.
 Each candidate is timed with CUDA events over a complete batched solve to the
 target tolerance.  Results can be cached in a JSON file keyed by the device
-name, the preconditioner, the tolerance and the size mix.
+name, the preconditioner, the tolerance and the size mix.  A batch whose
+instances fit on the chip is solved without sweeps unless TPFA_OPT_SWEEP asks for
+them (the cp.async candidate does), so its tilings time alike.
 """
 from __future__ import annotations
 

@@ -4,7 +4,8 @@
 // the instance).  The CG iterations of all instances run as one sweep launch
 // per iteration inside one CUDA-graph while loop; each instance keeps its
 // own scalars, completion counter and convergence flag, and the blocks of a
-// converged instance return at once.  Coefficients, right-hand sides, FP64
+// converged instance return at once.  Batches whose instances fit on the chip run
+// their inner solves in one cooperative launch instead (resident.cu).  Coefficients, right-hand sides, FP64
 // residuals and the refinement steps are launched per instance (a handful of
 // launches per refinement step).
 #include <math.h>

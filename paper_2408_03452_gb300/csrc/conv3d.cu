@@ -1470,7 +1470,7 @@ extern "C" int tpfa_conv3d_wgrad_bf16(const uint16_t* x, const uint16_t* dy, flo
 
 // Selects the forward convolution kernel: 0 = 128-voxel tiles with all nine
 // row groups per tile, 1 = z-marching ring where it fits, 2 = z-marching ring
-// with the z-taps folded into N, 3 = per layer shape (default), 4 = the folded
+// with the z-taps folded into N, 3 = the default (4), 4 = the folded
 // ring with warp-specialised roles.
 extern "C" int tpfa_conv3d_select(int kernel) {
   if (kernel < 0 || kernel > 4) return TPFA_EINVAL;

@@ -210,14 +210,16 @@ struct CoarseU {
   }
 };
 
-// p = w + c u + sum_j beta_j p_j; partial p'r (four elements per step)
+// p = w + c u + sum_j beta_j p_j; partial p'r (four elements per step).  With e
+// (M > 0) the previous iteration's e += alpha p_0 is made here, where p_0 is read
+// anyway: 4 of the 24 bytes per cell that a separate update moves.
 template <int M>
 __global__ void dir_kernel(const float* __restrict__ r, const float* __restrict__ dinv,
                            const float* __restrict__ u, CoarseU uc, Dirs pd,
-                           const Scal* __restrict__ sc, int jac, int net, float* p, int64_t n,
-                           double* part) {
+                           const Scal* __restrict__ sc, int jac, int net, float* p,
+                           float* __restrict__ e, int64_t n, double* part) {
   // p may be the oldest retained direction (read, then overwritten, per element)
-  const float c = (float)sc->c;
+  const float c = (float)sc->c, alpha = (float)sc->alpha;  // alpha of the previous iteration
   float beta[M > 0 ? M : 1];
 #pragma unroll
   for (int j = 0; j < M; ++j) beta[j] = (float)sc->beta[j];
@@ -241,6 +243,16 @@ __global__ void dir_kernel(const float* __restrict__ r, const float* __restrict_
     float4 p4[M > 0 ? M : 1];
 #pragma unroll
     for (int j = 0; j < M; ++j) p4[j] = reinterpret_cast<const float4*>(pd.v[j])[i];
+    if constexpr (M > 0) {
+      if (e != nullptr) {
+        float4 e4 = reinterpret_cast<float4*>(e)[i];
+        e4.x = fmaf(alpha, p4[0].x, e4.x);
+        e4.y = fmaf(alpha, p4[0].y, e4.y);
+        e4.z = fmaf(alpha, p4[0].z, e4.z);
+        e4.w = fmaf(alpha, p4[0].w, e4.w);
+        reinterpret_cast<float4*>(e)[i] = e4;
+      }
+    }
     float pv[M > 0 ? M : 1];
     float4 o;
 #pragma unroll
@@ -262,6 +274,9 @@ __global__ void dir_kernel(const float* __restrict__ r, const float* __restrict_
     float pv[M > 0 ? M : 1];
 #pragma unroll
     for (int j = 0; j < M; ++j) pv[j] = pd.v[j][i];
+    if constexpr (M > 0) {
+      if (e != nullptr) e[i] = fmaf(alpha, pv[0], e[i]);
+    }
     p[i] = one(r[i], jac ? dinv[i] : 0.f, net ? u[i] : 0.f, pv);
   }
   double pr[1] = {prf};
@@ -301,27 +316,19 @@ __global__ void finish_alpha_kernel(const double* __restrict__ part, int nb,
   }
 }
 
-// e += alpha p; r -= alpha q; partial r'r (four elements per step)
-__global__ void update_kernel(float* __restrict__ e, float* __restrict__ r,
-                              const float* __restrict__ p, const float* __restrict__ q,
+// r -= alpha q; partial r'r (four elements per step)
+__global__ void update_kernel(float* __restrict__ r, const float* __restrict__ q,
                               const Scal* __restrict__ sc, int64_t n, double* part) {
   const float alpha = (float)sc->alpha;
   float rrf = 0.f;
   const int64_t n4 = n / 4;
   for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * kT) {
-    float4 e4 = reinterpret_cast<float4*>(e)[i];
     float4 r4 = reinterpret_cast<float4*>(r)[i];
-    const float4 p4 = reinterpret_cast<const float4*>(p)[i];
     const float4 q4 = reinterpret_cast<const float4*>(q)[i];
-    e4.x = fmaf(alpha, p4.x, e4.x);
-    e4.y = fmaf(alpha, p4.y, e4.y);
-    e4.z = fmaf(alpha, p4.z, e4.z);
-    e4.w = fmaf(alpha, p4.w, e4.w);
     r4.x = fmaf(-alpha, q4.x, r4.x);
     r4.y = fmaf(-alpha, q4.y, r4.y);
     r4.z = fmaf(-alpha, q4.z, r4.z);
     r4.w = fmaf(-alpha, q4.w, r4.w);
-    reinterpret_cast<float4*>(e)[i] = e4;
     reinterpret_cast<float4*>(r)[i] = r4;
     rrf = fmaf(r4.x, r4.x, rrf);
     rrf = fmaf(r4.y, r4.y, rrf);
@@ -330,13 +337,81 @@ __global__ void update_kernel(float* __restrict__ e, float* __restrict__ r,
   }
   for (int64_t i = 4 * n4 + (int64_t)blockIdx.x * kT + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * kT) {
-    e[i] = fmaf(alpha, p[i], e[i]);
     const float v = fmaf(-alpha, q[i], r[i]);
     r[i] = v;
     rrf = fmaf(v, v, rrf);
   }
   double rr[1] = {rrf};
   block_sum_m<1>(rr, part);
+}
+
+// The same with r restricted to the 2^L coarser grid (L = 1, 2; the value of
+// block_mean<L>, bit for bit) for the network's next input: one thread per coarse
+// cell, whose rows are 16 bytes at L = 2, so a warp reads whole lines.  HBM bounds
+// it; 256^3: update 57 us (with e) + restriction 17 before, 33 so.
+template <int L>
+__global__ void update_restrict_kernel(float* __restrict__ r, const float* __restrict__ q,
+                                       const Scal* __restrict__ sc, float* __restrict__ coarse,
+                                       int nx, int ny, int nz, double* part) {
+  static_assert(L == 1 || L == 2, "blocks of 2 or 4 cells a side");
+  const float alpha = (float)sc->alpha;
+  const int cx = nx >> L, cy = ny >> L, nc = cx * cy * (nz >> L);
+  float rrf = 0.f;
+  for (int c = blockIdx.x * kT + threadIdx.x; c < nc; c += gridDim.x * kT) {
+    const int t = c / cx, i = c - t * cx, k = t / cy, j = t - k * cy;
+    const size_t base = ((size_t)(k << L) * ny + (j << L)) * nx + (i << L);
+    if constexpr (L == 1) {
+      float acc = 0.f;
+#pragma unroll
+      for (int row = 0; row < 4; ++row) {
+        const size_t o = base + ((size_t)(row >> 1) * ny + (row & 1)) * nx;
+        float2 v = *reinterpret_cast<float2*>(r + o);
+        const float2 w = *reinterpret_cast<const float2*>(q + o);
+        v.x = fmaf(-alpha, w.x, v.x);
+        v.y = fmaf(-alpha, w.y, v.y);
+        *reinterpret_cast<float2*>(r + o) = v;
+        rrf = fmaf(v.x, v.x, rrf);
+        rrf = fmaf(v.y, v.y, rrf);
+        acc += v.x + v.y;
+      }
+      coarse[c] = __fmul_rn(0.125f, acc);
+    } else {
+      float acc = 0.f;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {  // pairs of 2 x 2 x 2 blocks, next to each other in x
+        float lo = 0.f, hi = 0.f;
+#pragma unroll
+        for (int row = 0; row < 4; ++row) {
+          const size_t o = base + ((size_t)(2 * (b >> 1) + (row >> 1)) * ny + 2 * (b & 1) + (row & 1)) * nx;
+          float4 v = *reinterpret_cast<float4*>(r + o);
+          const float4 w = *reinterpret_cast<const float4*>(q + o);
+          v.x = fmaf(-alpha, w.x, v.x);
+          v.y = fmaf(-alpha, w.y, v.y);
+          v.z = fmaf(-alpha, w.z, v.z);
+          v.w = fmaf(-alpha, w.w, v.w);
+          *reinterpret_cast<float4*>(r + o) = v;
+          rrf = fmaf(v.x, v.x, rrf);
+          rrf = fmaf(v.y, v.y, rrf);
+          rrf = fmaf(v.z, v.z, rrf);
+          rrf = fmaf(v.w, v.w, rrf);
+          lo += v.x + v.y;
+          hi += v.z + v.w;
+        }
+        acc += __fmul_rn(0.125f, lo) + __fmul_rn(0.125f, hi);
+      }
+      coarse[c] = __fmul_rn(0.125f, acc);
+    }
+  }
+  double rr[1] = {rrf};
+  block_sum_m<1>(rr, part);
+}
+
+// e += alpha p: the update that no direction pass follows
+__global__ void flush_kernel(float* __restrict__ e, const float* __restrict__ p,
+                             const Scal* __restrict__ sc, int64_t n) {
+  const float alpha = (float)sc->alpha;
+  for (int64_t i = (int64_t)blockIdx.x * kT + threadIdx.x; i < n; i += (int64_t)gridDim.x * kT)
+    e[i] = fmaf(alpha, p[i], e[i]);
 }
 
 // r'r of this iteration into its history slot
@@ -357,11 +432,11 @@ void launch_dots(int m, int nb, cudaStream_t s, const float* r, const float* coe
 }
 
 void launch_dir(int m, int nb, cudaStream_t s, const float* r, const float* coef, const float* u,
-                const CoarseU& uc, const Dirs& pd, const Scal* sc, int jac, int net, float* p, int64_t n,
-                double* part) {
+                const CoarseU& uc, const Dirs& pd, const Scal* sc, int jac, int net, float* p,
+                float* e, int64_t n, double* part) {
   switch (m) {
 #define X(M) \
-  case M: dir_kernel<M><<<nb, kT, 0, s>>>(r, coef, u, uc, pd, sc, jac, net, p, n, part); break;
+  case M: dir_kernel<M><<<nb, kT, 0, s>>>(r, coef, u, uc, pd, sc, jac, net, p, e, n, part); break;
     TPFA_FCG_M0(X)
 #undef X
     default: break;
@@ -528,16 +603,20 @@ enum PrecMode { kIdentity = 0, kJacobi = 1, kBlend = 2 };
 
 // the network term u of the blend: into w.z with A u (into w.au, u'Au into w.uau)
 // unless the fused operator takes it, which reads a coarser u where it is
+// (restricted: the last update left r on the network's grid)
 int network_term(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, Work& w,
-                 bool with_apply) {
+                 bool with_apply, bool restricted) {
   int rc;
   if (w.levels > 0) {
     const int L = w.levels;
-    launch_restrict_levels(L, w.nb, w.s, w.r, w.rl[L], w.dims[0], w.dims[1], w.dims[2], 1,
-                           nullptr, 0, 0, 0);
+    if (!restricted) {
+      launch_restrict_levels(L, w.nb, w.s, w.r, w.rl[L], w.dims[0], w.dims[1], w.dims[2], 1,
+                             nullptr, 0, 0, 0);
+      ++w.launches;
+    }
     rc = tpfa_unet_forward(net, w.rl[L], w.lnkc, w.ul[L], w.s);
     if (rc) return rc;
-    w.launches += 16;
+    w.launches += 9;
     if (with_apply) {
       launch_prolong_levels(L, w.nb, w.s, w.ul[L], w.z, w.dims[0], w.dims[1], w.dims[2], 1,
                             nullptr, 0, 0, 0, true);
@@ -546,7 +625,7 @@ int network_term(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* ln
   } else {
     rc = tpfa_unet_forward(net, w.r, lnk, w.z, w.s);
     if (rc) return rc;
-    w.launches += 15;
+    w.launches += 9;
   }
   if (!with_apply) return TPFA_OK;
   rc = tpfa_apply(c, coef, w.z, w.au, w.uau, w.s);
@@ -617,9 +696,16 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
   const int m = w.m;
   double rr = rr0;
   int stored = 0, head = 0, pending = 0;
+  bool restricted = false;  // r on the network's grid is that of the current r
   PrecMode mode = net == nullptr ? kIdentity : (res->fallback ? fallback_mode : kBlend);
   std::vector<double> hist(1, rr);
   if (cudaMemsetAsync(w.sc, 0, sizeof(Scal), w.s) != cudaSuccess) return TPFA_ECUDA;
+  // the newest direction's share of e (directions are stored, so there is one)
+  auto flush = [&] {
+    const size_t slot = (size_t)((head - 1 + m) % m);
+    flush_kernel<<<w.nb, kT, 0, w.s>>>(w.e, w.P + slot * w.slot_stride(), w.sc, w.n);
+    ++w.launches;
+  };
   while (res->iters < maxit && rr > target * target * rr0) {
     const int jac = mode != kIdentity, with_net = mode == kBlend;
     Dirs qd, pd;
@@ -644,7 +730,7 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
       uc.cplane = uc.cx * (w.dims[1] >> L);
     }
     if (with_net) {
-      int rc = network_term(c, net, coef, lnk, w, !fused);
+      int rc = network_term(c, net, coef, lnk, w, !fused, restricted);
       if (rc) return rc;
       if (fused) {
         if (launch_apply_dots_tma_batch(w.finst, 1, w.fblocks, 0, w.fact, 1, w.own0, qmap, stored,
@@ -665,12 +751,28 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
     }
     float* p = w.P + (size_t)head * w.slot_stride();
     float* q = w.Q + (size_t)head * w.slot_stride();
-    launch_dir(stored, w.nb, w.s, w.r, w.dinv, w.z, uc, pd, w.sc, jac, with_net, p, w.n, w.part);
+    launch_dir(stored, w.nb, w.s, w.r, w.dinv, w.z, uc, pd, w.sc, jac, with_net, p,
+               stored > 0 ? w.e : nullptr, w.n, w.part);
     int rc = tpfa_apply(c, coef, p, q, w.pq, w.s);
     if (rc) return rc;
     finish_alpha_kernel<<<1, kT, 0, w.s>>>(w.part, w.nb, w.pq, w.sc, head);
-    update_kernel<<<w.nb, kT, 0, w.s>>>(w.e, w.r, p, q, w.sc, w.n, w.part);
-    finish_rr_kernel<<<1, kT, 0, w.s>>>(w.part, w.nb, w.hist + pending);
+    // e follows in the next direction pass, which reads p anyway, or in the flush
+    restricted = with_net && (w.levels == 1 || w.levels == 2);
+    int nbu = w.nb;
+    if (restricted) {
+      // one thread per coarse cell while the partial sums have room
+      const int64_t nc = w.n >> (3 * w.levels), cap = (int64_t)kPartPerBlock * w.nb;
+      nbu = (int)std::min((nc + kT - 1) / kT, cap);
+      if (w.levels == 1)
+        update_restrict_kernel<1><<<nbu, kT, 0, w.s>>>(w.r, q, w.sc, w.rl[1], w.dims[0], w.dims[1],
+                                                       w.dims[2], w.part);
+      else
+        update_restrict_kernel<2><<<nbu, kT, 0, w.s>>>(w.r, q, w.sc, w.rl[2], w.dims[0], w.dims[1],
+                                                       w.dims[2], w.part);
+    } else {
+      update_kernel<<<w.nb, kT, 0, w.s>>>(w.r, q, w.sc, w.n, w.part);
+    }
+    finish_rr_kernel<<<1, kT, 0, w.s>>>(w.part, nbu, w.hist + pending);
     w.launches += 7;
     ++pending;
     ++res->iters;
@@ -700,6 +802,7 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
       stalled = recent > 0.99 * before;
     }
     if (bad || stalled) {
+      flush();
       if (mode != kBlend) {
         res->status = TPFA_EBREAKDOWN;
         return TPFA_OK;
@@ -711,6 +814,7 @@ int fcg_inner(tpfa_ctx* c, tpfa_unet* net, const float* coef, const float* lnk, 
       if (cudaMemsetAsync(w.sc, 0, sizeof(Scal), w.s) != cudaSuccess) return TPFA_ECUDA;
     }
   }
+  if (stored > 0) flush();
   return TPFA_OK;
 }
 
