@@ -368,27 +368,28 @@ sweep_kernel(const SweepArgs a) {
 // ---------------------------------------------------------------------------
 // FP64 residual r = b - A x (one thread per cell, grid-stride, fixed grid).
 // Bound by the FP64 units (1/64 of the FP32 rate): 10 operations per cell, 8
-// without the norms, which are formed only when asked for.  I: 32-bit cell
-// arithmetic where the grid allows it.
-template <typename I, bool NORMS>
+// without the norms, which are formed only when asked for (256^3: 305 us with,
+// 264 without).  The 64-bit index arithmetic hides behind them; with 32-bit
+// indices the same kernel took 329 and 267 us.
+template <bool NORMS>
 __global__ void __launch_bounds__(kElemThreads)
 residual64_kernel(Grid g, const double2* __restrict__ coef64, const double* __restrict__ b,
                   const double* __restrict__ x, double* __restrict__ r, double* norms,
                   CgState* st, double* partials, unsigned int* counter) {
   double rr = 0.0, bb = 0.0;
-  const I nx = (I)g.nx, ny = (I)g.ny, nz = (I)g.nz, plane = (I)g.plane, n = (I)g.n;
-  const I stride = (I)gridDim.x * blockDim.x;
-  for (I c = (I)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += stride) {
-    const I row = c / nx, i = c - row * nx, k = c / plane, j = row - k * ny;
-    const double2 c01 = __ldg(coef64 + 2 * (size_t)c), c23 = __ldg(coef64 + 2 * (size_t)c + 1);
+  const int64_t nx = g.nx, ny = g.ny, nz = g.nz, plane = g.plane;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < g.n; c += stride) {
+    const int64_t row = c / nx, i = c - row * nx, k = c / plane, j = row - k * ny;
+    const double2 c01 = __ldg(coef64 + 2 * c), c23 = __ldg(coef64 + 2 * c + 1);
     const double xc = __ldg(x + c);
     double s = c23.y * xc;
     if (i + 1 < nx) s = fma(-c01.x, __ldg(x + c + 1), s);
-    if (i > 0) s = fma(-__ldg(&coef64[2 * (size_t)(c - 1)].x), __ldg(x + c - 1), s);
+    if (i > 0) s = fma(-__ldg(&coef64[2 * (c - 1)].x), __ldg(x + c - 1), s);
     if (j + 1 < ny) s = fma(-c01.y, __ldg(x + c + nx), s);
-    if (j > 0) s = fma(-__ldg(&coef64[2 * (size_t)(c - nx)].y), __ldg(x + c - nx), s);
+    if (j > 0) s = fma(-__ldg(&coef64[2 * (c - nx)].y), __ldg(x + c - nx), s);
     if (k + 1 < nz) s = fma(-c23.x, __ldg(x + c + plane), s);
-    if (k > 0) s = fma(-__ldg(&coef64[2 * (size_t)(c - plane) + 1].x), __ldg(x + c - plane), s);
+    if (k > 0) s = fma(-__ldg(&coef64[2 * (c - plane) + 1].x), __ldg(x + c - plane), s);
     const double bc = __ldg(b + c);
     const double rc = bc - s;
     r[c] = rc;
@@ -729,19 +730,12 @@ cudaError_t launch_residual64(const Grid& g, const double* coef64, const double*
                               const double* x, double* r, double* norms, CgState* st,
                               double* partials, unsigned int* counter, int nblocks,
                               cudaStream_t s) {
-  // below 2^31 cells minus one grid stride, 32-bit indices cannot overflow
-  const bool small = g.n < (int64_t)0x7fffffff - (int64_t)nblocks * kElemThreads;
   const double2* c64 = reinterpret_cast<const double2*>(coef64);
   auto run = [&](auto kernel) {
     kernel<<<nblocks, kElemThreads, 0, s>>>(g, c64, b, x, r, norms, st, partials, counter);
   };
-  if (norms != nullptr || st != nullptr) {
-    if (small) run(residual64_kernel<uint32_t, true>);
-    else run(residual64_kernel<int64_t, true>);
-  } else {
-    if (small) run(residual64_kernel<uint32_t, false>);
-    else run(residual64_kernel<int64_t, false>);
-  }
+  if (norms != nullptr || st != nullptr) run(residual64_kernel<true>);
+  else run(residual64_kernel<false>);
   return cudaGetLastError();
 }
 
