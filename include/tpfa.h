@@ -234,8 +234,9 @@ int tpfa_residual64(tpfa_ctx* ctx, const double* coef64, const double* b, const 
  * that fit on the chip (about one 32 x 16 x 32 brick per SM, 2.5 M cells on
  * GB300) run a whole inner solve as one cooperative launch with the vectors in
  * registers and shared memory, unless TPFA_OPT_SWEEP or TPFA_OPT_TILE_VY asks
- * for a sweep; it needs a few MB of context memory, 12 bytes per cell more
- * above 1.2 M cells, and falls back to the sweeps where that cannot be had.
+ * for a sweep; it needs a few MB of context memory and 12 bytes per cell more
+ * above 1.2 M cells (the sweeps' vectors are not allocated then), and the sweeps
+ * take over where the device refuses a cooperative launch of that size.
  * An explicit TPFA_OPT_TILE_ZC takes the bricks of a batch, so that results
  * are bit-identical to it.
  * Outer loop: FP64 residual with coef64, FP32 correction solve, FP64 update

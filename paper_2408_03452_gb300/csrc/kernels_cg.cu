@@ -370,7 +370,8 @@ sweep_kernel(const SweepArgs a) {
 // Bound by the FP64 units (1/64 of the FP32 rate): 10 operations per cell, 8
 // without the norms, which are formed only when asked for (256^3: 305 us with,
 // 264 without).  The 64-bit index arithmetic hides behind them; with 32-bit
-// indices the same kernel took 329 and 267 us.
+// indices the same kernel took 329 and 267 us, and with signed instead of unsigned
+// offsets into coef64 352.
 template <bool NORMS>
 __global__ void __launch_bounds__(kElemThreads)
 residual64_kernel(Grid g, const double2* __restrict__ coef64, const double* __restrict__ b,
@@ -381,15 +382,15 @@ residual64_kernel(Grid g, const double2* __restrict__ coef64, const double* __re
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < g.n; c += stride) {
     const int64_t row = c / nx, i = c - row * nx, k = c / plane, j = row - k * ny;
-    const double2 c01 = __ldg(coef64 + 2 * c), c23 = __ldg(coef64 + 2 * c + 1);
+    const double2 c01 = __ldg(coef64 + 2 * (size_t)c), c23 = __ldg(coef64 + 2 * (size_t)c + 1);
     const double xc = __ldg(x + c);
     double s = c23.y * xc;
     if (i + 1 < nx) s = fma(-c01.x, __ldg(x + c + 1), s);
-    if (i > 0) s = fma(-__ldg(&coef64[2 * (c - 1)].x), __ldg(x + c - 1), s);
+    if (i > 0) s = fma(-__ldg(&coef64[2 * (size_t)(c - 1)].x), __ldg(x + c - 1), s);
     if (j + 1 < ny) s = fma(-c01.y, __ldg(x + c + nx), s);
-    if (j > 0) s = fma(-__ldg(&coef64[2 * (c - nx)].y), __ldg(x + c - nx), s);
+    if (j > 0) s = fma(-__ldg(&coef64[2 * (size_t)(c - nx)].y), __ldg(x + c - nx), s);
     if (k + 1 < nz) s = fma(-c23.x, __ldg(x + c + plane), s);
-    if (k > 0) s = fma(-__ldg(&coef64[2 * (c - plane) + 1].x), __ldg(x + c - plane), s);
+    if (k > 0) s = fma(-__ldg(&coef64[2 * (size_t)(c - plane) + 1].x), __ldg(x + c - plane), s);
     const double bc = __ldg(b + c);
     const double rc = bc - s;
     r[c] = rc;
