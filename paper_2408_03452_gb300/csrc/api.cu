@@ -205,17 +205,23 @@ int ensure_r64(tpfa_ctx* c) {
   return TPFA_OK;
 }
 
-int ensure_comm(tpfa_ctx* c, size_t words) {
+// Cleared on the solve's own stream: a non-blocking stream is not ordered with the
+// legacy one, and a clear still queued there would wipe words in use.
+int ensure_comm(tpfa_ctx* c, size_t words, cudaStream_t s) {
   if (words <= c->comm_words) return TPFA_OK;
   unsigned long long* m = nullptr;
   if (cudaMalloc(&m, words * 8) != cudaSuccess) {
     cudaGetLastError();
     return TPFA_ENOMEM;
   }
+  if (cudaMemsetAsync(m, 0, words * 8, s) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(m);
+    return TPFA_ECUDA;
+  }
   if (c->comm) cudaFree(c->comm);
   c->comm = m;
   c->comm_words = words;
-  CK(cudaMemset(m, 0, words * 8));
   return TPFA_OK;
 }
 
@@ -742,7 +748,7 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
   ResPlan rp;
   const bool resident = use_resident(c, &rp);
   rc = ensure_r64(c);
-  if (!rc) rc = resident ? ensure_comm(c, rp.words) : ensure_vectors(c);
+  if (!rc && !resident) rc = ensure_vectors(c);
   if (rc) return rc;
   if (resident && rp.packed > 0 && c->packed == nullptr &&
       cudaMalloc(&c->packed, rp.packed) != cudaSuccess) {
@@ -757,10 +763,9 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
       return TPFA_ENOMEM;
     }
   }
-  if (!resident) {
-    rc = ensure_loop(c, coef, b16);
-    if (rc) return rc;
-  }
+  // (after the other allocations: the solve that queued the clear waits for it)
+  rc = resident ? ensure_comm(c, rp.words, s) : ensure_loop(c, coef, b16);
+  if (rc) return rc;
   const CgVecs vecs = resident ? CgVecs{} : loop_vecs(c, b16);
   CK(cudaMemsetAsync(c->counter, 0, 64, s));
   CK(cudaEventRecord(c->ev[0], s));

@@ -62,8 +62,10 @@ bool batch_resident(const tpfa_batch* b) {
   return true;
 }
 
-// Plans and buffers of the resident solves, on first use.
-int setup_batch_resident(tpfa_batch* b) {
+// Plans and buffers of the resident solves, on first use; the exchange words are
+// cleared on the solve's own stream (a non-blocking stream is not ordered with the
+// legacy one).
+int setup_batch_resident(tpfa_batch* b, cudaStream_t s) {
   if (b->sched != nullptr) return TPFA_OK;
   const int N = b->ninst;
   b->rplan.resize(N);
@@ -76,22 +78,26 @@ int setup_batch_resident(tpfa_batch* b) {
     blocks += (size_t)b->rplan[i].nblk;
   }
   b->comm_words = words;
+  int rc = TPFA_OK;
   if (cudaMalloc(&b->comm, words * 8) != cudaSuccess ||
       cudaMalloc(&b->team, blocks * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&b->prob_dev, sizeof(ResProb) * N) != cudaSuccess ||
-      cudaMalloc(&b->sched, resident_batch_words(N, b->num_sms) * 8) != cudaSuccess) {
+      cudaMalloc(&b->sched, resident_batch_words(N, b->num_sms) * 8) != cudaSuccess)
+    rc = TPFA_ENOMEM;
+  else if (cudaMemsetAsync(b->comm, 0, words * 8, s) != cudaSuccess)
+    rc = TPFA_ECUDA;
+  if (rc != TPFA_OK) {
     cudaGetLastError();
     cudaFree(b->comm);
     cudaFree(b->team);
     cudaFree(b->prob_dev);
+    cudaFree(b->sched);
     b->comm = nullptr;
     b->team = nullptr;
     b->prob_dev = nullptr;
     b->sched = nullptr;
-    return TPFA_ENOMEM;
   }
-  BK(cudaMemset(b->comm, 0, words * 8));
-  return TPFA_OK;
+  return rc;
 }
 
 // Automatic z-runs of the TMA-staged batched sweep: one common run length,
@@ -506,10 +512,10 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       !dev_ok(rhs, n * 8, 8, b->device) || !dev_ok(x, n * 8, 8, b->device))
     return TPFA_EINVAL;
   if ((const void*)rhs == (const void*)x) return TPFA_EINVAL;
-  const bool resident = batch_resident(b);
-  rc = resident ? setup_batch_resident(b) : ensure_batch_loop(b, coef);
-  if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
+  const bool resident = batch_resident(b);
+  rc = resident ? setup_batch_resident(b, s) : ensure_batch_loop(b, coef);
+  if (rc) return rc;
   const int N = b->ninst;
   std::vector<ResProb> probs;
   const float4* cf = reinterpret_cast<const float4*>(coef);

@@ -1,0 +1,79 @@
+"""First calls on a side stream while the default stream has work queued: what a
+call clears or copies for itself is ordered with the caller's stream, whatever
+another stream is doing."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2408_03452_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2408_03452_gb300 import build, tpfa
+    build.build()
+    return tpfa
+
+
+def _busy():
+    """About 0.1 s of ordinary work on the default stream."""
+    a = torch.ones(1 << 28, device="cuda")
+    for _ in range(300):
+        a.mul_(1.0)
+    return a
+
+
+def _system(tp, shape, seed):
+    nx, ny, nz = shape
+    K = torch.from_numpy(synth.lognormal_field(nx, ny, nz, 1.0, seed)).cuda()
+    mask, pD = (torch.from_numpy(v).cuda() for v in synth.dirichlet_faces(nx, ny, nz, "x", 1.0, 0.0))
+    with tp.Context(*shape) as ctx:
+        coef, coef64 = ctx.build_trans(K, mask, None, 0.0)
+        b = ctx.build_rhs(K, mask, None, pD)
+    return coef, coef64, b
+
+
+@pytest.mark.parametrize("precond", [0, 1])
+@pytest.mark.parametrize("shape", [(33, 17, 9), (128, 128, 80)])
+def test_first_solve_on_a_side_stream(tp, shape, precond):
+    """Low and tall bricks of the resident solve."""
+    coef, coef64, b = _system(tp, shape, 21)
+    side = torch.cuda.Stream()
+    xs = []
+    for busy in (False, True):
+        with tp.Context(*shape) as ctx:
+            ctx.set_option("precond", precond)
+            x = torch.zeros_like(b)
+            torch.cuda.synchronize()
+            keep = _busy() if busy else None
+            with torch.cuda.stream(side):
+                _, info = ctx.cg_solve(coef, coef64, b, x=x, tol=1e-8, maxit=20000, check=False)
+            torch.cuda.synchronize()
+            del keep
+            assert info["code"] == 0, info
+            xs.append(x.cpu().numpy())
+    assert np.array_equal(*xs)
+
+
+def test_first_batched_solve_on_a_side_stream(tp):
+    grids = [(33, 17, 9), (48, 48, 24), (20, 40, 12)]
+    parts = [_system(tp, g, 31 + i) for i, g in enumerate(grids)]
+    coef, coef64, b = (torch.cat([p[k] for p in parts]) for k in range(3))
+    side = torch.cuda.Stream()
+    xs = []
+    for busy in (False, True):
+        with tp.BatchContext(grids) as bc:
+            x = torch.zeros_like(b)
+            torch.cuda.synchronize()
+            keep = _busy() if busy else None
+            with torch.cuda.stream(side):
+                _, _, tot = bc.cg_solve(coef, coef64, b, x=x, tol=1e-8, maxit=20000, check=False)
+            torch.cuda.synchronize()
+            del keep
+            assert tot["code"] == 0, tot
+            xs.append(x.cpu().numpy())
+    assert np.array_equal(*xs)
