@@ -119,7 +119,7 @@ int batch_tma_zauto(const tpfa_batch* b) {
 // Per-instance tilings and tensor maps of the TMA-staged batched sweep for
 // one coefficient array, the interleaved vector records on first use, and
 // partial-sum room for its blocks.
-int setup_batch_tma(tpfa_batch* b, const float* coef) {
+int setup_batch_tma(tpfa_batch* b, const float* coef, cudaStream_t s) {
   const int N = b->ninst;
   const size_t pad = ((size_t)b->cells + 15) / 16 * 16;
   if (b->vec4 == nullptr) {
@@ -179,8 +179,11 @@ int setup_batch_tma(tpfa_batch* b, const float* coef) {
     b->partials = np;
     b->partials_cap = (size_t)blocks * 4;
   }
-  BK(cudaMemcpy(b->maps_dev, maps.data(), sizeof(CUtensorMap) * 4 * N, cudaMemcpyHostToDevice));
-  BK(cudaMemcpy(b->tinst_dev, b->tinst.data(), sizeof(TmaInst) * N, cudaMemcpyHostToDevice));
+  BK(cudaMemcpyAsync(b->maps_dev, maps.data(), sizeof(CUtensorMap) * 4 * N,
+                     cudaMemcpyHostToDevice, s));
+  BK(cudaMemcpyAsync(b->tinst_dev, b->tinst.data(), sizeof(TmaInst) * N, cudaMemcpyHostToDevice,
+                     s));
+  BK(cudaStreamSynchronize(s));
   b->v.v4[0] = b->vec4;
   b->v.v4[1] = b->vec4 + pad;
   return TPFA_OK;
@@ -202,7 +205,7 @@ bool grid_ok(const tpfa_grid& g) {
 }
 
 // While loop {batched sweep; condition} for one coefficient array.
-int ensure_batch_loop(tpfa_batch* b, const float* coef) {
+int ensure_batch_loop(tpfa_batch* b, const float* coef, cudaStream_t s) {
   if (b->loop_exec && b->loop_key_coef == coef && b->loop_key_precond == b->precond &&
       b->loop_key_sweep == b->sweep_sel && b->loop_key_tile == b->tma_tile)
     return TPFA_OK;
@@ -210,7 +213,7 @@ int ensure_batch_loop(tpfa_batch* b, const float* coef) {
   b->loop_exec = nullptr;
   const bool tma = batch_tma(b);
   if (tma) {
-    const int rc = setup_batch_tma(b, coef);
+    const int rc = setup_batch_tma(b, coef, s);
     if (rc) return rc;
   } else {
     b->v.v4[0] = b->v.v4[1] = nullptr;
@@ -365,6 +368,8 @@ int tpfa_batch_create(const tpfa_grid* grids, int n_inst, const int* zc, tpfa_ba
   for (int i = 0; i < 4; ++i)
     if (cudaEventCreate(&b->ev[i]) != cudaSuccess) goto fail;
   if (sweep_blocks_per_sm(4, 4) < 1) goto fail;
+  // the clears above are on the legacy stream, which solves are not ordered with
+  if (cudaDeviceSynchronize() != cudaSuccess) goto fail;
   *out = b;
   return TPFA_OK;
 fail:
@@ -514,7 +519,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
   if ((const void*)rhs == (const void*)x) return TPFA_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   const bool resident = batch_resident(b);
-  rc = resident ? setup_batch_resident(b, s) : ensure_batch_loop(b, coef);
+  rc = resident ? setup_batch_resident(b, s) : ensure_batch_loop(b, coef, s);
   if (rc) return rc;
   const int N = b->ninst;
   std::vector<ResProb> probs;

@@ -544,7 +544,7 @@ struct Work {
            cudaMalloc(&sc, sizeof(Scal)) == cudaSuccess &&
            cudaMalloc(&hist, sizeof(double) * kCheckEvery) == cudaSuccess &&
            cudaMallocHost(&hhist, sizeof(double) * kCheckEvery) == cudaSuccess &&
-           cudaMemset(sc, 0, sizeof(Scal)) == cudaSuccess;
+           cudaMemsetAsync(sc, 0, sizeof(Scal), s) == cudaSuccess;
   }
   ~Work() {
     if (s) cudaStreamSynchronize(s);

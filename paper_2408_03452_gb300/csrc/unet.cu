@@ -557,6 +557,8 @@ int tpfa_unet_create(int nx, int ny, int nz, int ns, int train, tpfa_unet** out)
                                                                   : 64 * kBiasBlocks;
   ok = ok && alloc_zero((void**)&u->rms, (size_t)ns * 4) && alloc_zero((void**)&u->partials, np * 8) &&
        alloc_zero((void**)&u->counters, (size_t)ns * 4);
+  // the clears are on the legacy stream, which the callers' streams are not ordered with
+  ok = ok && cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     unet_free(u);

@@ -77,3 +77,58 @@ def test_first_batched_solve_on_a_side_stream(tp):
             assert tot["code"] == 0, tot
             xs.append(x.cpu().numpy())
     assert np.array_equal(*xs)
+
+
+def test_new_network_on_a_side_stream(tp):
+    """Created while the default stream is busy: the clears of its buffers do not
+    land in the weights or between the layers."""
+    from paper_2408_03452_gb300 import learned
+    n = 32
+    g = torch.Generator(device="cuda").manual_seed(5)
+    r, lnk = (torch.randn(n ** 3, generator=g, device="cuda") for _ in range(2))
+    P = learned.init_params(3).cuda()
+    side = torch.cuda.Stream()
+    zs = []
+    for busy in (False, True):
+        torch.cuda.synchronize()
+        keep = _busy() if busy else None
+        net = tp.UNet(n, n, n, 1)
+        with torch.cuda.stream(side):
+            net.set_params(P)
+            z = net.forward(r, lnk)
+        torch.cuda.synchronize()
+        del keep
+        zs.append(z.cpu().numpy())
+    assert np.isfinite(zs[0]).all() and np.abs(zs[0]).max() > 0
+    assert np.array_equal(*zs)
+
+
+def test_batched_sweeps_and_flexible_cg_on_a_side_stream(tp):
+    """A batch created, and a flexible-CG solve made, while the default stream is busy."""
+    grids = [(24, 20, 12), (33, 17, 9)]
+    parts = [_system(tp, g, 41 + i) for i, g in enumerate(grids)]
+    coef, coef64, b = (torch.cat([p[k] for p in parts]) for k in range(3))
+    side = torch.cuda.Stream()
+    xs, es = [], []
+    for busy in (False, True):
+        x, e = torch.zeros_like(b), torch.zeros_like(parts[0][2])
+        with tp.Context(*grids[0]) as ctx:
+            ctx.set_option("fcg_m", 2)
+            torch.cuda.synchronize()
+            keep = _busy() if busy else None
+            with torch.cuda.stream(side):
+                _, info = ctx.fcg_solve(*parts[0], x=e, tol=1e-8,
+                                        maxit=5000, check=False)
+            torch.cuda.synchronize()
+            del keep
+        keep = _busy() if busy else None
+        with tp.BatchContext(grids) as bc:
+            bc.set_option("tma_tile", 1)
+            with torch.cuda.stream(side):
+                _, _, tot = bc.cg_solve(coef, coef64, b, x=x, tol=1e-8, maxit=20000, check=False)
+            torch.cuda.synchronize()
+        del keep
+        assert info["code"] == 0 and tot["code"] == 0, (info, tot)
+        xs.append(x.cpu().numpy())
+        es.append(e.cpu().numpy())
+    assert np.array_equal(*xs) and np.array_equal(*es)
