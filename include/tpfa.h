@@ -333,6 +333,14 @@ int cg_solve_batch(tpfa_batch* batch, const float* coef, const double* coef64, c
                    double* x, double tol, int64_t maxit, tpfa_cg_info* infos,
                    tpfa_cg_info* total, void* stream);
 
+/* Test hook for the failure path of resident solves: bounds of the waits inside
+ * them, for the later solves of a context or a batch (one of the two, the other
+ * NULL).  polls: looks of one wait for another block's words (1 to 2^23; 0 = the
+ * default, 2^23); looks: looks of an idle block at its mailbox while no running
+ * instance advances (batches; 1 to 2^25; 0 = the default, 2^25).  A solve whose
+ * wait runs out returns TPFA_EINTERNAL; the next one is sound again. */
+int tpfa_resident_wait_limits(tpfa_ctx* ctx, tpfa_batch* batch, uint32_t polls, uint32_t looks);
+
 /*
  * Tensor-core GEMM tile (tcgen05, BF16 inputs, FP32 accumulation in tensor
  * memory): C[M x N] = A[M x K] * B[K x N], with A row-major (K contiguous),

@@ -53,6 +53,7 @@ struct tpfa_ctx {
   size_t comm_words;
   float2* packed;    // coefficients of the resident CG with tall bricks (on first use)
   int resident_off;  // the device refused a cooperative launch of this size
+  uint32_t poll_limit;  // tpfa_resident_wait_limits
   TmaMaps* maps;     // tensor maps of the TMA-staged sweep (host copy, built with the loop)
   TmaPlan tplan;
   cudaStream_t cap_stream;
@@ -385,6 +386,8 @@ double ctx_option(const tpfa_ctx* c, int option) {
   }
 }
 
+void ctx_poll_limit(tpfa_ctx* c, uint32_t polls) { c->poll_limit = polls; }
+
 // The TMA-staged operator's plan for tpfa_apply's arguments (coef, p 16-byte
 // aligned; dots: the variant fused with the flexible-CG dot products), or
 // false when tpfa_apply would take the cp.async kernel.
@@ -446,6 +449,7 @@ int tpfa_create(const tpfa_grid* grid, tpfa_ctx** out) {
   c->precond = 0;
   c->zc = 0;
   c->chunk = 32;
+  c->poll_limit = kResPollLimit;
   int rc = TPFA_ECUDA;
   if (cudaGetDevice(&c->device) != cudaSuccess) goto fail;
   if (cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
@@ -816,6 +820,7 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
         ResProb prob = make_res_prob(c->g, rp, coef, b16, c->dinv, c->r64, x, c->st, rtol,
                                      (long long)(maxit - total_iters), c->comm);
         prob.packed = c->packed;
+        prob.poll_limit = c->poll_limit;
         const cudaError_t e = launch_resident(prob, c->precond == 1, s);
         if (e == cudaErrorCooperativeLaunchTooLarge && outer == 0) {
           // fewer SMs than the device reports: this context keeps the sweeps

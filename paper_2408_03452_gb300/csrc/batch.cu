@@ -289,6 +289,8 @@ int tpfa_batch_create(const tpfa_grid* grids, int n_inst, const int* zc, tpfa_ba
   b->fcg_fallback = 0;
   b->sweep_sel = 0;
   b->tma_tile = 0;
+  b->poll_limit = kResPollLimit;
+  b->look_limit = kResLookLimit;
   b->zc_req.assign(n_inst, 0);
   if (zc != nullptr)
     for (int i = 0; i < n_inst; ++i) b->zc_req[i] = zc[i];
@@ -466,6 +468,19 @@ int tpfa_batch_set_option(tpfa_batch* b, int option, double value) {
   }
 }
 
+int tpfa_resident_wait_limits(tpfa_ctx* c, tpfa_batch* b, uint32_t polls, uint32_t looks) {
+  if ((c == nullptr) == (b == nullptr) || polls > kResPollLimit || looks > kResLookLimit)
+    return TPFA_EINVAL;
+  const uint32_t p = polls > 0 ? polls : kResPollLimit;
+  if (c != nullptr) {
+    ctx_poll_limit(c, p);
+  } else {
+    b->poll_limit = p;
+    b->look_limit = looks > 0 ? looks : kResLookLimit;
+  }
+  return TPFA_OK;
+}
+
 int tpfa_batch_build_trans(tpfa_batch* b, const double* K, const uint8_t* dirichlet,
                            const double* d, double d_uniform, float* coef, double* coef64,
                            void* stream) {
@@ -597,7 +612,9 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
         probs.push_back(make_res_prob(b->g[i], b->rplan[i], cf + o, false, nullptr, b->r64 + o,
                                       x + o, b->st + i, rtol, (long long)(maxit - iters[i]),
                                       b->comm + b->comm_off[i]));
-        probs.back().abort = reinterpret_cast<uint32_t*>(b->sched + 2);
+        probs.back().abort = resident_batch_abort(b->sched);
+        probs.back().beat = resident_batch_beat(b->sched);
+        probs.back().poll_limit = b->poll_limit;
         probs.back().team = b->team + team0[i];
       }
       BK(cudaMemcpyAsync(b->prob_dev, probs.data(), sizeof(ResProb) * probs.size(),
@@ -612,7 +629,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       for (size_t p0 = 0, p1 = 0; p0 < probs.size() && e == cudaSuccess; p0 = p1) {
         while (p1 < probs.size() && probs[p1].cz == probs[p0].cz) ++p1;
         e = launch_resident_batch(b->prob_dev + p0, (int)(p1 - p0), probs[p0].cz, b->num_sms,
-                                  b->precond == 1, b->sched, s);
+                                  b->precond == 1, b->sched, b->look_limit, s);
         ++launches;
       }
       if (e == cudaErrorCooperativeLaunchTooLarge && step == 0) {

@@ -51,6 +51,7 @@ struct tpfa_batch {
   tpfa::ResProb* prob_dev;
   unsigned long long* sched;
   int resident_off;  // the device refused the cooperative launch
+  uint32_t poll_limit, look_limit;  // tpfa_resident_wait_limits
   cudaGraphExec_t loop_exec;
   const void* loop_key_coef;
   int loop_key_precond;

@@ -44,7 +44,7 @@ namespace {
 
 constexpr int kRW = 16;                 // warps per block = brick rows
 constexpr int kRT = kRW * 32;           // threads
-constexpr uint32_t kPollLimit = 1u << 23;  // polls of one wait before giving up
+constexpr uint32_t kBeat = 64;          // iterations between signs of progress (batches)
 
 // ---- unevaluated sums of two floats ----------------------------------------
 struct Dfl {
@@ -131,7 +131,6 @@ template <int NH, bool EARLY>
 struct ResComm {
   uint2* part;
   const uint2* face;
-  uint32_t* abort;
   int nblk, blk;
   int hoff[NH];  // face words this thread reads (index in one buffer), -1: none
   size_t face_buf;
@@ -165,8 +164,8 @@ struct ResComm {
   // Sends this block's sums and waits for every block's and for the
   // neighbours' face words.  The totals are there in warp 0 only.  Returns
   // false when the wait ran out (or another block gave up).
-  __device__ __forceinline__ bool exchange(const Dfl (&mine)[4], uint32_t epoch, Dfl (&tot)[4],
-                                           float (&qh)[NH], ResShared& sh) {
+  __device__ __forceinline__ bool exchange(const ResProb& a, const Dfl (&mine)[4], uint32_t epoch,
+                                           Dfl (&tot)[4], float (&qh)[NH], ResShared& sh) {
     auto& sA = sh.a;
     auto& sB = sh.b;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -202,8 +201,8 @@ struct ResComm {
     bool ok = true;
     uint32_t polls = 0;
     auto give_up = [&]() -> bool {
-      if ((++polls & 1023u) != 0u) return false;
-      return polls >= kPollLimit || *(volatile uint32_t*)abort != 0u;
+      if (++polls >= a.poll_limit) return true;
+      return (polls & 1023u) == 0u && *(volatile uint32_t*)a.abort != 0u;
     };
     while (need != 0u) {
 #pragma unroll
@@ -223,9 +222,9 @@ struct ResComm {
     // the sums of every block: item = 4 block + value, in order
     Dfl sum = {0.f, 0.f};
     for (int item = tid; ok && item < 4 * nblk;) {
-      const uint2 a = ll_load(pb + (size_t)item * 2), b = ll_load(pb + (size_t)item * 2 + 1);
-      if (a.y == epoch && b.y == epoch) {
-        sum = df_acc(sum, {__uint_as_float(a.x), __uint_as_float(b.x)});
+      const uint2 h = ll_load(pb + (size_t)item * 2), l = ll_load(pb + (size_t)item * 2 + 1);
+      if (h.y == epoch && l.y == epoch) {
+        sum = df_acc(sum, {__uint_as_float(h.x), __uint_as_float(l.x)});
         item += kRT;
       } else if (give_up()) {
         ok = false;
@@ -236,7 +235,7 @@ struct ResComm {
     sum = df_acc(sum, df_xor(sum, 16));
     if (lane < 4) sB[warp][lane] = make_float2(sum.h, sum.l);
     if (__syncthreads_or(!ok)) {
-      if (tid == 0) *(volatile uint32_t*)abort = 1u;
+      if (tid == 0) *(volatile uint32_t*)a.abort = 1u;
       return false;
     }
     if (warp == 0) {
@@ -270,7 +269,8 @@ __device__ __forceinline__ float operator_scale(const ResProb& a, int blk, float
         dmax = fmaxf(dmax, __uint_as_float(v.x));
         break;
       }
-      if ((++polls & 1023u) == 0u && (polls >= kPollLimit || *(volatile uint32_t*)a.abort != 0u)) {
+      if (++polls >= a.poll_limit ||
+          ((polls & 1023u) == 0u && *(volatile uint32_t*)a.abort != 0u)) {
         fault = true;
         break;
       }
@@ -353,8 +353,9 @@ struct ResScalars {
   }
 };
 
-// One inner solve, run by the blocks blk = 0 .. a.nblk - 1 of its brick grid.
-template <int CZ, bool JAC>
+// One inner solve, run by the blocks blk = 0 .. a.nblk - 1 of its brick grid
+// (BATCH: with signs of progress for the scheduler).
+template <int CZ, bool JAC, bool BATCH>
 __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float* sm,
                                                ResShared& sh) {
   using LY = ResLayout<CZ>;
@@ -417,7 +418,6 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
   ResComm<5, (CZ <= 8)> cm;
   cm.part = a.part;
   cm.face = a.face;
-  cm.abort = a.abort;
   cm.nblk = a.nblk;
   cm.blk = blk;
   cm.face_buf = (size_t)a.nblk * LY::kFaces;
@@ -589,10 +589,12 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     Dfl mine[4], tot[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) mine[v] = df_fast(acc[v].s, -acc[v].c);
-    if (!cm.exchange(mine, epoch, tot, qh, sh)) {
+    if (!cm.exchange(a, mine, epoch, tot, qh, sh)) {
       fault = true;
       break;
     }
+    if (BATCH && (epoch & (kBeat - 1u)) == 0u && blk == 0 && tid == 0)
+      atomicAdd(a.beat, 1u);
     // the scalars are formed by warp 0 alone: in all 16 warps the same chain takes
     // twice as long
     if (warp == 0) {
@@ -618,7 +620,7 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
       mine[j < 4 ? j : 0] = {0.f, 0.f};
     }
     mine[0] = df_fast(s0.s, -s0.c);
-    const bool ok = cm.exchange(mine, epoch, tot, qh, sh);
+    const bool ok = cm.exchange(a, mine, epoch, tot, qh, sh);
 #pragma unroll
     for (int j = 0; j < 5; ++j) cm.hoff[j] = keep[j];
     if (!ok) {
@@ -763,7 +765,6 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
   ResComm<NH, false> cm;
   cm.part = a.part;
   cm.face = a.face;
-  cm.abort = a.abort;
   cm.nblk = a.nblk;
   cm.blk = blk;
   cm.face_buf = (size_t)a.nblk * LY::kFaces;
@@ -926,7 +927,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     Dfl mine[4], tot[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) mine[v] = df_fast(acc[v].s, -acc[v].c);
-    if (!cm.exchange(mine, epoch, tot, qh, sh)) {
+    if (!cm.exchange(a, mine, epoch, tot, qh, sh)) {
       fault = true;
       break;
     }
@@ -952,7 +953,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     }
     mine[0] = df_fast(s0.s, -s0.c);
     mine[1] = mine[2] = mine[3] = {0.f, 0.f};
-    const bool ok = cm.exchange(mine, epoch, tot, qh, sh);
+    const bool ok = cm.exchange(a, mine, epoch, tot, qh, sh);
 #pragma unroll
     for (int j = 0; j < NH; ++j) cm.hoff[j] = keep[j];
     if (!ok) {
@@ -999,7 +1000,7 @@ template <int CZ, bool JAC>
 __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant__ ResProb a) {
   extern __shared__ __align__(16) float sm[];
   __shared__ ResShared sh;
-  resident_solve<CZ, JAC>(a, blockIdx.x, sm, sh);
+  resident_solve<CZ, JAC, false>(a, blockIdx.x, sm, sh);
 }
 
 // ---- many instances in one launch --------------------------------------------
@@ -1010,11 +1011,14 @@ __global__ void __launch_bounds__(kRT, 1) resident_kernel(const __grid_constant_
 // then starts the largest waiting instance that fits the free blocks, and so on
 // down the list.  Free blocks wait for a word in their mailbox.  A started team
 // always has all its blocks, so every wait ends.
+//
+// A free block waits for as long as other teams run, which a solve of many
+// iterations stretches at will, so its limit is on looks without progress: every
+// running team counts up a word once in kBeat iterations, and so does every release.
 struct ResSched {
   int lock, nfree, left;   // left: instances not yet started
-  int pad;
+  uint32_t beat;
 };
-constexpr uint32_t kMailLimit = 1u << 28;  // looks at an empty mailbox before giving up
 constexpr uint32_t kExit = 0xffffffffu;
 
 struct ResBatchArgs {
@@ -1026,6 +1030,7 @@ struct ResBatchArgs {
   uint32_t* sent;       // [nblocks] words sent to a block so far
   unsigned long long* mail;  // [nblocks] {message, sequence number}
   uint32_t* abort;      // the instances' abort flag, shared
+  uint32_t look_limit;  // looks of a free block without progress before it gives up
 };
 
 // Returns `n` blocks (members, or all blocks when null) to the free list and starts what
@@ -1035,7 +1040,7 @@ __device__ void sched_release(const ResBatchArgs& a, const int* members, int n) 
   if (lane == 0) {
     uint32_t polls = 0;
     while (atomicCAS(&a.sched->lock, 0, 1) != 0) {
-      if (++polls >= kPollLimit) {
+      if (++polls >= kResPollLimit) {
         *(volatile uint32_t*)a.abort = 1u;
         break;
       }
@@ -1084,6 +1089,7 @@ __device__ void sched_release(const ResBatchArgs& a, const int* members, int n) 
   }
   __syncwarp();
   if (lane == 0) {
+    atomicAdd(&a.sched->beat, 1u);
     *(volatile int*)&a.sched->nfree = nfree;
     *(volatile int*)&a.sched->left = left;
     __threadfence();
@@ -1108,14 +1114,24 @@ __global__ void __launch_bounds__(kRT, 1) resident_batch_kernel(const __grid_con
   }
   for (uint32_t seq = 1;; ++seq) {
     if (threadIdx.x == 0) {
-      uint32_t got = kExit;
-      for (uint32_t polls = 0; polls < kMailLimit; ++polls) {
+      uint32_t got = kExit, beat = 0u;
+      for (uint32_t polls = 0;; ++polls) {
         const uint2 w = ll_load(reinterpret_cast<const uint2*>(a.mail + me));
         if (w.y == seq) {
           got = w.x;
           break;
         }
         if (*(volatile uint32_t*)a.abort != 0u) break;
+        if (polls >= a.look_limit) {
+          const uint32_t now = *(volatile uint32_t*)&a.sched->beat;
+          if (now == beat) {
+            // a team started from now on could not have this block: none may wait for it
+            *(volatile uint32_t*)a.abort = 1u;
+            break;
+          }
+          beat = now;
+          polls = 0;
+        }
         __nanosleep(200);
       }
       msg = got;
@@ -1125,7 +1141,7 @@ __global__ void __launch_bounds__(kRT, 1) resident_batch_kernel(const __grid_con
     const uint32_t m = msg;
     if (m == kExit) return;
     const int rank = (int)(m & 4095u);
-    resident_solve<CZ, JAC>(prob, rank, sm, sh);
+    resident_solve<CZ, JAC, true>(prob, rank, sm, sh);
     __syncthreads();
     // the blocks of a team end in the same iteration: its first block returns
     // them together, so that a large instance waiting for that many blocks is
@@ -1227,6 +1243,8 @@ ResProb make_res_prob(const Grid& g, const ResPlan& p, const void* coef, bool b1
   a.face = a.part + (size_t)2 * p.nblk * 8;
   a.team = nullptr;
   a.packed = nullptr;
+  a.beat = nullptr;
+  a.poll_limit = kResPollLimit;
   return a;
 }
 
@@ -1247,9 +1265,15 @@ cudaError_t launch_resident(const ResProb& prob, bool jac, cudaStream_t s) {
 }
 
 size_t resident_batch_words(int nprob, int num_sms) { return sched_words(nprob, num_sms); }
+uint32_t* resident_batch_abort(unsigned long long* sched) {
+  return reinterpret_cast<uint32_t*>(sched + 2);
+}
+uint32_t* resident_batch_beat(unsigned long long* sched) {
+  return &reinterpret_cast<ResSched*>(sched)->beat;
+}
 
 cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int cz, int num_sms, bool jac,
-                                  unsigned long long* sched, cudaStream_t s) {
+                                  unsigned long long* sched, uint32_t look_limit, cudaStream_t s) {
   const size_t words = sched_words(nprob, num_sms);
   cudaError_t e = cudaMemsetAsync(sched, 0, words * 8, s);
   if (e != cudaSuccess) return e;
@@ -1258,7 +1282,8 @@ cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int cz, in
   a.nprob = nprob;
   a.nblocks = num_sms;
   a.sched = reinterpret_cast<ResSched*>(sched);
-  a.abort = reinterpret_cast<uint32_t*>(sched + 2);
+  a.abort = resident_batch_abort(sched);
+  a.look_limit = look_limit;
   a.mail = sched + 4;
   a.started = reinterpret_cast<int*>(sched + 4 + num_sms);
   a.freel = a.started + nprob;

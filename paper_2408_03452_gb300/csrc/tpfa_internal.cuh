@@ -247,7 +247,11 @@ struct ResProb {
   uint32_t* abort;        // set by a block whose wait ran out
   int* team;              // batched: [nblk] blocks that run it
   float2* packed;         // bricks above 16 planes: p.packed bytes of workspace
+  uint32_t* beat;         // batched: counted up while the solve advances
+  uint32_t poll_limit;    // polls of one wait before it gives up
 };
+constexpr uint32_t kResPollLimit = 1u << 23;  // seconds; an exchange takes microseconds
+constexpr uint32_t kResLookLimit = 1u << 25;  // likewise, 64 iterations between beats
 // Bricks for one grid; false when it does not fit at one brick per SM.
 // dense = false: the lowest bricks that fit (shortest iterations of a solve that
 // has the chip to itself).  dense = true: the bricks with the least block time
@@ -262,11 +266,14 @@ ResProb make_res_prob(const Grid& g, const ResPlan& p, const void* coef, bool b1
 cudaError_t launch_resident(const ResProb& prob, bool jac, cudaStream_t s);
 // Several FP32-record instances with dense plans of one brick height cz (device
 // table sorted by nblk, largest first; at most kResMaxProb) in one launch; each has
-// its own comm, team, and prob.abort == the word at sched + 2.
+// its own comm and team; abort and beat are those of the scheduler's buffer.
 constexpr int kResMaxProb = 1 << 19;
 size_t resident_batch_words(int nprob, int num_sms);
+uint32_t* resident_batch_abort(unsigned long long* sched);
+uint32_t* resident_batch_beat(unsigned long long* sched);
 cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int cz, int num_sms,
-                                  bool jac, unsigned long long* sched, cudaStream_t s);
+                                  bool jac, unsigned long long* sched, uint32_t look_limit,
+                                  cudaStream_t s);
 // Resident launches of one device are made one at a time (held from the launch
 // until the host has waited for it), so that the blocks of two of them never
 // compete for the same SMs.
@@ -278,6 +285,7 @@ std::mutex& resident_mutex(int device);
 int64_t ctx_cells(const tpfa_ctx* c);
 void ctx_dims(const tpfa_ctx* c, int64_t* d3);
 double ctx_option(const tpfa_ctx* c, int option);
+void ctx_poll_limit(tpfa_ctx* c, uint32_t polls);
 bool ctx_apply_tma_plan(const tpfa_ctx* c, TmaPlan* p, Grid* g, int dots = 0);
 bool dev_ok(const void* p, size_t bytes, size_t align, int device);
 bool opt_dev_ok(const void* p, size_t bytes, size_t align, int device);

@@ -97,6 +97,7 @@ SIGNATURES = {
     "tpfa_batch_set_option": (C.c_int, [_P, C.c_int, C.c_double]),
     "tpfa_batch_build_trans": (C.c_int, [_P, _P, _P, _P, C.c_double, _P, _P, _P]),
     "tpfa_batch_build_rhs": (C.c_int, [_P, _P, _P, _P, _P, _P, _P]),
+    "tpfa_resident_wait_limits": (C.c_int, [_P, _P, C.c_uint32, C.c_uint32]),
     "cg_solve_batch": (C.c_int, [_P, _P, _P, _P, _P, C.c_double, C.c_int64, _P,
                                  C.POINTER(_Info), _P]),
     "fcg_solve_batch": (C.c_int, [_P, _P, C.c_int, _P, _P, _P, _P, _P, _P, C.c_double,
