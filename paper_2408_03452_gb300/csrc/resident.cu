@@ -23,10 +23,13 @@
 //
 // Scalars.  FP64 runs at 1/64 of the FP32 rate on this chip, so beyond the
 // thread sums (compensated FP32, as in the sweeps) the dot products are added
-// as unevaluated pairs of floats (48 bits; Dekker 1971, Knuth TAOCP 4.2.2:
-// TwoSum, and products by FMA), in a fixed order, and every block forms the
-// same alpha and beta from them.  The operator is scaled by a power of two at
-// load time (largest D in [1, 2)), which changes no mantissa and keeps the
+// as unevaluated pairs of floats (48 bits, fp32_pair.cuh) in a fixed order, and every
+// block forms the same alpha and beta from them: pair quotients rounded once, which
+// is what the sweeps' FP64 quotients round to.  Against the exact sums the totals are
+// off by 1e-10 to 3e-10 (the thread sums' share), the same to four digits as with FP64
+// trees, whose own share is 2e-16 against 9e-15; with the scalars in FP64 an iteration
+// takes 1.0 us longer (32^3 3.06 against 2.04).  The operator is scaled by a power of
+// two at load time (largest D in [1, 2)), which changes no mantissa and keeps the
 // pairs inside the FP32 range; the solution is scaled back at the end.
 //
 // us per iteration (GB300, plain CG), the sweeps in their graph loop and here:
@@ -37,6 +40,7 @@
 // stencil, 0.2 us per plane.
 #include <math.h>
 
+#include "fp32_pair.cuh"
 #include "sweep_common.cuh"
 
 namespace tpfa {
@@ -46,42 +50,6 @@ constexpr int kRW = 16;                 // warps per block = brick rows
 constexpr int kRT = kRW * 32;           // threads
 constexpr uint32_t kBeat = 64;          // iterations between signs of progress (batches)
 
-// ---- unevaluated sums of two floats ----------------------------------------
-struct Dfl {
-  float h, l;
-};
-__device__ __forceinline__ Dfl df_fast(float a, float b) {  // |a| >= |b|
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ Dfl df_add(Dfl a, Dfl b) {
-  const float s = __fadd_rn(a.h, b.h);
-  const float v = __fsub_rn(s, a.h);
-  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
-  return df_fast(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ bool df_le(Dfl a, Dfl b) {
-  return a.h < b.h || (a.h == b.h && a.l <= b.l);
-}
-// the same without the final normalisation: for trees of a few levels, where
-// the correction stays small; only one addition is on the critical path
-__device__ __forceinline__ Dfl df_acc(Dfl a, Dfl b) {
-  const float s = __fadd_rn(a.h, b.h);
-  const float v = __fsub_rn(s, a.h);
-  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
-  return {s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
-}
-__device__ __forceinline__ Dfl df_mulf(Dfl a, float b) {
-  const float p = __fmul_rn(a.h, b);
-  return df_fast(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
-}
-// a / b to an ulp: a quotient from the approximate reciprocal and one residual
-// correction
-__device__ __forceinline__ float quot(float a, float b) {
-  const float y = __fdividef(1.f, b);
-  const float q = __fmul_rn(a, y);
-  return __fmaf_rn(__fmaf_rn(-q, b, a), y, q);
-}
 __device__ __forceinline__ Dfl df_xor(Dfl a, int m) {
   return {__shfl_xor_sync(kFull, a.h, m), __shfl_xor_sync(kFull, a.l, m)};
 }
@@ -311,13 +279,13 @@ struct ResScalars {
     }
     // alpha is the FP32 step the vectors take, so that rho - 2 alpha r'q +
     // alpha^2 q'q is the norm of the residual it leaves
-    const float al = quot(rho.h, tot[1].h);
+    const float al = df_quot(rho, tot[1]);
     const Dfl u = df_mulf(tot[3], al);
     const Dfl v = df_mulf(df_add({2.f * tot[2].h, 2.f * tot[2].l}, {-u.h, -u.l}), al);
     Dfl rn = df_add(rho, {-v.h, -v.l});
     if (rn.h < 0.f) rn = {0.f, 0.f};
     alpha = al;
-    beta = quot(rn.h, rho.h);
+    beta = df_quot(rn, rho);
     // 0 unless one of the sums is infinite or NaN
     const float bad = fmaf(tot[0].h, 0.f, fmaf(tot[1].h, 0.f, fmaf(tot[2].h, 0.f, tot[3].h * 0.f)));
     const bool stay = bad == 0.f && tot[1].h > 0.f && !df_le(rho, thresh);
@@ -337,7 +305,7 @@ struct ResScalars {
     const Dfl prev = rho;
     rho = tot[0];
     if (done == kConvEst && !df_le(rho, thresh) && iter < maxit && isfinite(rho.h) && prev.h > 0.f) {
-      beta = quot(rho.h, prev.h);
+      beta = df_quot(rho, prev);
       done = kRunning;
     }
     alpha = 0.f;
