@@ -86,22 +86,102 @@ struct ResNext {
   int done;
 };
 
+// Scalars of an iteration, formed by warp 0 (tall bricks: kept in shared memory, a
+// dozen registers of every thread otherwise): alpha, beta and the stop test (as
+// cg_finish).
+struct ResScalars {
+  Dfl rho, rho0, thresh;
+  long long iter, sweeps;
+  float alpha, beta;
+  int done;
+
+  __device__ __forceinline__ void init() {
+    rho = rho0 = thresh = {0.f, 0.f};
+    iter = sweeps = 0;
+    alpha = beta = 0.f;
+    done = kRunning;
+  }
+  __device__ __forceinline__ void update(const Dfl (&tot)[4], double rtol2, long long maxit) {
+    rho = tot[0];
+    if (iter == 0) {
+      const float h = (float)rtol2, l = (float)(rtol2 - (double)h);
+      rho0 = rho;
+      thresh = df_add(df_mulf(rho0, h), df_mulf(rho0, l));
+    }
+    // alpha is the FP32 step the vectors take, so that rho - 2 alpha r'q +
+    // alpha^2 q'q is the norm of the residual it leaves
+    const float al = df_quot(rho, tot[1]);
+    const Dfl u = df_mulf(tot[3], al);
+    const Dfl v = df_mulf(df_add({2.f * tot[2].h, 2.f * tot[2].l}, {-u.h, -u.l}), al);
+    Dfl rn = df_add(rho, {-v.h, -v.l});
+    if (rn.h < 0.f) rn = {0.f, 0.f};
+    alpha = al;
+    beta = df_quot(rn, rho);
+    // 0 unless one of the sums is infinite or NaN
+    const float bad = fmaf(tot[0].h, 0.f, fmaf(tot[1].h, 0.f, fmaf(tot[2].h, 0.f, tot[3].h * 0.f)));
+    const bool stay = bad == 0.f && tot[1].h > 0.f && !df_le(rho, thresh);
+    ++iter;
+    if (!stay || df_le(rn, thresh) || iter >= maxit || ++sweeps > 2 * maxit + 64) {
+      done = stay ? (df_le(rn, thresh) ? kConvEst : iter >= maxit ? kMaxit : kGuard)
+                  : (bad != 0.f ? kNonFinite : df_le(rho, thresh) ? kConvTrue : kBreakdown);
+      if (!stay) {
+        alpha = 0.f;
+        --iter;
+      }
+    }
+  }
+  // after the last step: the true r'r of the residual it leaves; if the estimate
+  // that stopped the loop was too optimistic, go on with the exact continuation
+  __device__ __forceinline__ void finish(const Dfl (&tot)[4], long long maxit) {
+    const Dfl prev = rho;
+    rho = tot[0];
+    if (done == kConvEst && !df_le(rho, thresh) && iter < maxit && isfinite(rho.h) && prev.h > 0.f) {
+      beta = df_quot(rho, prev);
+      done = kRunning;
+    }
+    alpha = 0.f;
+  }
+  __device__ __forceinline__ void report(CgState* st, double scale, bool fault) const {
+    st->rho = (double)rho.h + (double)rho.l;
+    st->rho0 = (double)rho0.h + (double)rho0.l;
+    st->scale = scale;
+    st->iter = iter;
+    st->launches = 1;
+    st->done = fault ? (int)kGuard : done;
+    st->fault = fault ? 1 : 0;
+  }
+};
+
 struct ResShared {
   float2 a[kRW][4], b[kRW][4];  // sums per warp: of the block, of all blocks
   float mx[kRW];
+  ResScalars sc;
   ResNext next;
+};
+
+// the face words a thread waits for, where their offsets are not held: has(j), off(j)
+template <class Has, class Off>
+struct FaceWords {
+  Has has;
+  Off off;
 };
 
 // the block's sums of four values, sent to every block and added up in a fixed
 // order; the neighbours' face words arrive in the same wait
-// (NH: words a thread waits for; EARLY: first look before the sums are sent)
-template <int NH, bool EARLY>
+// (NH: words a thread waits for; EARLY: first look before the sums are sent; BW: words
+// of one look.  With 8 words their offsets and both halves take 24 registers, which the
+// tall bricks do not have: there they are looked at four at a time and the offsets
+// formed on the way, 128^3 10.6 against 12.6 us per iteration.)
+template <int NH, bool EARLY, int BW = NH>
 struct ResComm {
   uint2* part;
   const uint2* face;
   int nblk, blk;
-  int hoff[NH];  // face words this thread reads (index in one buffer), -1: none
+  int hoff[BW == NH ? NH : 1];  // face words this thread reads (index in one buffer), -1: none
   size_t face_buf;
+
+  __device__ __forceinline__ bool has(int j) const { return hoff[j] >= 0; }
+  __device__ __forceinline__ int off(int j) const { return hoff[j]; }
 
   // warp-wide transposing sum of four pairs: lane l ends with value (l >> 3)
   __device__ __forceinline__ static Dfl warp4(const Dfl (&v)[4]) {
@@ -130,10 +210,12 @@ struct ResComm {
   }
 
   // Sends this block's sums and waits for every block's and for the
-  // neighbours' face words.  The totals are there in warp 0 only.  Returns
-  // false when the wait ran out (or another block gave up).
+  // neighbours' face words (FACES; wd.has(j): there is one, wd.off(j): its index in one
+  // buffer).  The totals are there in warp 0 only.  Returns false when the wait ran out (or another block gave up).
+  template <bool FACES, class Words>
   __device__ __forceinline__ bool exchange(const ResProb& a, const Dfl (&mine)[4], uint32_t epoch,
-                                           Dfl (&tot)[4], float (&qh)[NH], ResShared& sh) {
+                                           const Words& wd, Dfl (&tot)[4], float (&qh)[NH],
+                                           ResShared& sh) {
     auto& sA = sh.a;
     auto& sB = sh.b;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -148,16 +230,17 @@ struct ResComm {
     // while warp 0 sends the sums (64^3: 2.89 -> 2.66 us per iteration); with
     // tall ones the loads would only hold up those (128x128x64: 5.3 against 5.9)
     unsigned need = 0u;
-    uint2 f[NH];
-    auto look = [&]() {
+    uint2 f[BW];
+    auto look = [&](int j0) {
+      if (!FACES) return;
 #pragma unroll
-      for (int j = 0; j < NH; ++j)
-        if (hoff[j] >= 0) {
+      for (int j = 0; j < BW; ++j)
+        if (j0 + j < NH && wd.has(j0 + j)) {
           need |= 1u << j;
-          f[j] = ll_load(fb + hoff[j]);
+          f[j] = ll_load(fb + wd.off(j0 + j));
         }
     };
-    if (EARLY) look();
+    if (EARLY) look(0);
     if (warp == 0) {
       const Dfl t = warps16(sA);
       if (lane < 4) {
@@ -165,27 +248,36 @@ struct ResComm {
         ll_store(pb + ((size_t)blk * 4 + lane) * 2 + 1, t.l, epoch);
       }
     }
-    if (!EARLY) look();
+    if (!EARLY) look(0);
     bool ok = true;
     uint32_t polls = 0;
     auto give_up = [&]() -> bool {
       if (++polls >= a.poll_limit) return true;
       return (polls & 1023u) == 0u && *(volatile uint32_t*)a.abort != 0u;
     };
-    while (need != 0u) {
+    auto await = [&](int j0) {
+      while (need != 0u) {
 #pragma unroll
-      for (int j = 0; j < NH; ++j)
-        if (((need >> j) & 1u) && f[j].y == epoch) {
-          qh[j] = __uint_as_float(f[j].x);
-          need &= ~(1u << j);
+        for (int j = 0; j < BW; ++j)
+          if (j0 + j < NH && ((need >> j) & 1u) && f[j].y == epoch) {
+            qh[j0 + j] = __uint_as_float(f[j].x);
+            need &= ~(1u << j);
+          }
+        if (need != 0u && give_up()) {
+          ok = false;
+          break;
         }
-      if (need != 0u && give_up()) {
-        ok = false;
-        break;
-      }
 #pragma unroll
-      for (int j = 0; j < NH; ++j)
-        if ((need >> j) & 1u) f[j] = ll_load(fb + hoff[j]);
+        for (int j = 0; j < BW; ++j)
+          if (j0 + j < NH && ((need >> j) & 1u)) f[j] = ll_load(fb + wd.off(j0 + j));
+      }
+    };
+    await(0);
+#pragma unroll
+    for (int j0 = BW; j0 < NH; j0 += BW) {
+      if (!ok) break;
+      look(j0);
+      await(j0);
     }
     // the sums of every block: item = 4 block + value, in order
     Dfl sum = {0.f, 0.f};
@@ -255,71 +347,6 @@ __device__ __forceinline__ float operator_scale(const ResProb& a, int blk, float
   e = e > 120 ? 120 : (e < -120 ? -120 : e);
   return exp2f((float)-e);
 }
-
-// Scalars of an iteration, kept by warp 0: alpha, beta and the stop test (as
-// cg_finish).
-struct ResScalars {
-  Dfl rho, rho0, thresh;
-  long long iter, sweeps;
-  float alpha, beta;
-  int done;
-
-  __device__ __forceinline__ void init() {
-    rho = rho0 = thresh = {0.f, 0.f};
-    iter = sweeps = 0;
-    alpha = beta = 0.f;
-    done = kRunning;
-  }
-  __device__ __forceinline__ void update(const Dfl (&tot)[4], double rtol2, long long maxit) {
-    rho = tot[0];
-    if (iter == 0) {
-      const float h = (float)rtol2, l = (float)(rtol2 - (double)h);
-      rho0 = rho;
-      thresh = df_add(df_mulf(rho0, h), df_mulf(rho0, l));
-    }
-    // alpha is the FP32 step the vectors take, so that rho - 2 alpha r'q +
-    // alpha^2 q'q is the norm of the residual it leaves
-    const float al = df_quot(rho, tot[1]);
-    const Dfl u = df_mulf(tot[3], al);
-    const Dfl v = df_mulf(df_add({2.f * tot[2].h, 2.f * tot[2].l}, {-u.h, -u.l}), al);
-    Dfl rn = df_add(rho, {-v.h, -v.l});
-    if (rn.h < 0.f) rn = {0.f, 0.f};
-    alpha = al;
-    beta = df_quot(rn, rho);
-    // 0 unless one of the sums is infinite or NaN
-    const float bad = fmaf(tot[0].h, 0.f, fmaf(tot[1].h, 0.f, fmaf(tot[2].h, 0.f, tot[3].h * 0.f)));
-    const bool stay = bad == 0.f && tot[1].h > 0.f && !df_le(rho, thresh);
-    ++iter;
-    if (!stay || df_le(rn, thresh) || iter >= maxit || ++sweeps > 2 * maxit + 64) {
-      done = stay ? (df_le(rn, thresh) ? kConvEst : iter >= maxit ? kMaxit : kGuard)
-                  : (bad != 0.f ? kNonFinite : df_le(rho, thresh) ? kConvTrue : kBreakdown);
-      if (!stay) {
-        alpha = 0.f;
-        --iter;
-      }
-    }
-  }
-  // after the last step: the true r'r of the residual it leaves; if the estimate
-  // that stopped the loop was too optimistic, go on with the exact continuation
-  __device__ __forceinline__ void finish(const Dfl (&tot)[4], long long maxit) {
-    const Dfl prev = rho;
-    rho = tot[0];
-    if (done == kConvEst && !df_le(rho, thresh) && iter < maxit && isfinite(rho.h) && prev.h > 0.f) {
-      beta = df_quot(rho, prev);
-      done = kRunning;
-    }
-    alpha = 0.f;
-  }
-  __device__ __forceinline__ void report(CgState* st, double scale, bool fault) const {
-    st->rho = (double)rho.h + (double)rho.l;
-    st->rho0 = (double)rho0.h + (double)rho0.l;
-    st->scale = scale;
-    st->iter = iter;
-    st->launches = 1;
-    st->done = fault ? (int)kGuard : done;
-    st->fault = fault ? 1 : 0;
-  }
-};
 
 // One inner solve, run by the blocks blk = 0 .. a.nblk - 1 of its brick grid
 // (BATCH: with signs of progress for the scheduler).
@@ -394,15 +421,22 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
   float rh[5], mh[5], pz[2] = {0.f, 0.f}, qh[5];
   const int xs = tid / LY::kFx, xi = tid % LY::kFx;  // x-halo: side, index w CZ + k
   int pslot[3];                                      // sP index of halo cells 2, 3, 4
+  const unsigned halo =
+      (bz > 0 ? 1u : 0u) | (bz + 1 < a.nbz ? 2u : 0u) | (warp < CZ && by > 0 ? 4u : 0u) |
+      (warp < CZ && by + 1 < a.nby ? 8u : 0u) |
+      ((xs == 0 && bx > 0) || (xs == 1 && bx + 1 < a.nbx) ? 16u : 0u);
+  auto hindex = [&](int j) {
+    constexpr int fy = 2 * LY::kFx, fz = 2 * (LY::kFx + LY::kFy);
+    return j == 0   ? (blk - a.nbx * a.nby) * LY::kFaces + fz + LY::kFz + tid
+           : j == 1 ? (blk + a.nbx * a.nby) * LY::kFaces + fz + tid
+           : j == 2 ? (blk - a.nbx) * LY::kFaces + fy + LY::kFy + tid
+           : j == 3 ? (blk + a.nbx) * LY::kFaces + fy + tid
+           : xs == 0 ? (blk - 1) * LY::kFaces + LY::kFx + xi
+                     : (blk + 1) * LY::kFaces + xi;
+  };
+#pragma unroll
+  for (int j = 0; j < 5; ++j) cm.hoff[j] = ((halo >> j) & 1u) ? hindex(j) : -1;
   {
-    const int nb[5] = {bz > 0 ? blk - a.nbx * a.nby : -1, bz + 1 < a.nbz ? blk + a.nbx * a.nby : -1,
-                       (warp < CZ && by > 0) ? blk - a.nbx : -1,
-                       (warp < CZ && by + 1 < a.nby) ? blk + a.nbx : -1,
-                       xs == 0 ? (bx > 0 ? blk - 1 : -1)
-                               : (xs == 1 && bx + 1 < a.nbx ? blk + 1 : -1)};
-    const int w[5] = {2 * (LY::kFx + LY::kFy) + LY::kFz + tid, 2 * (LY::kFx + LY::kFy) + tid,
-                      2 * LY::kFx + LY::kFy + tid, 2 * LY::kFx + tid,
-                      xs == 0 ? LY::kFx + xi : xi};
     const int xk = xi % CZ, xw = xi / CZ;
     pslot[0] = warp * (kRW + 2) * 34 + lane + 1;
     pslot[1] = (warp * (kRW + 2) + kRW + 1) * 34 + lane + 1;
@@ -413,11 +447,10 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     const int64_t hz[5] = {Z0 - 1, Z0 + CZ, Z0 + warp, Z0 + warp, Z0 + xk};
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-      cm.hoff[j] = nb[j] < 0 ? -1 : nb[j] * LY::kFaces + w[j];
       rh[j] = 0.f;
       mh[j] = 0.f;
       qh[j] = 0.f;
-      if (nb[j] >= 0 && hx[j] < g.nx && hy[j] < g.ny && hz[j] < g.nz) {
+      if (((halo >> j) & 1u) && hx[j] < g.nx && hy[j] < g.ny && hz[j] < g.nz) {
         const int64_t c = hx[j] + g.nx * hy[j] + g.plane * hz[j];
         rh[j] = (float)(scale * a.r64[c]);
         if (JAC) mh[j] = a.b16 ? a.dinv[c] : jac_inv(__ldg(c32 + c).w);
@@ -557,7 +590,7 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     Dfl mine[4], tot[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) mine[v] = df_fast(acc[v].s, -acc[v].c);
-    if (!cm.exchange(a, mine, epoch, tot, qh, sh)) {
+    if (!cm.template exchange<true>(a, mine, epoch, cm, tot, qh, sh)) {
       fault = true;
       break;
     }
@@ -580,17 +613,9 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     step(false, s0);
     ++epoch;
     // the face words of this exchange are not sent: nothing reads them
-    int keep[5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      keep[j] = cm.hoff[j];
-      cm.hoff[j] = -1;
-      mine[j < 4 ? j : 0] = {0.f, 0.f};
-    }
     mine[0] = df_fast(s0.s, -s0.c);
-    const bool ok = cm.exchange(a, mine, epoch, tot, qh, sh);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) cm.hoff[j] = keep[j];
+    mine[1] = mine[2] = mine[3] = {0.f, 0.f};
+    const bool ok = cm.template exchange<false>(a, mine, epoch, cm, tot, qh, sh);
     if (!ok) {
       fault = true;
       break;
@@ -625,12 +650,20 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
 
 // ---- bricks of up to 32 planes -------------------------------------------------
 // The same iteration for grids of up to twice that size (2.5 M cells on GB300).
-// r and q are in registers, p, x and Ty in shared memory, and the other
-// coefficients (Tx, Tz, D: 12 bytes per cell) are read every iteration from a
-// packed copy, which each thread writes for itself at the start and which stays
-// in L2; loads run four planes ahead of the stencil.  The Jacobi variant is plain
-// CG on S A S with S = M^-1/2 (the same iterates: r'M^-1 r is the norm of S r), so
-// that neither M^-1 nor a second vector is needed.
+// r and q are in registers, p, x and Ty in shared memory, with bricks of 24 planes D as
+// well; the other coefficients (Tx, Tz and D, or with Jacobi M^-1: 12 bytes per cell) are
+// read every iteration from a packed copy, which each thread writes for itself at the
+// start and which stays in L2; loads run four planes ahead of the stencil.
+//
+// The Jacobi variant keeps z = M^-1 r and w = M^-1 q in place of r and q: the step then
+// needs no M^-1, the words of the faces carry w, and r'z is the sum of D z^2, formed in
+// the stencil, where D is at hand.  The operator is that of the records, as in the
+// sweeps.  (CG on S A S with S = M^-1/2, every coefficient rounded again, took 15 to 23 %
+// more iterations than the sweep over 24 fields with FP32 records, 50 % more on the worst;
+// so it is within 0.6 % of the sweep, 3 % on the worst.)  us per iteration, plain /
+// Jacobi, before and now: 100^3 (24 planes) 9.2 / 7.9 and 7.5 / 8.0, 128^3 (32 planes)
+// 10.8 / 10.9 and 10.7 / 11.6.  M^-1 is loaded beside D in shared memory (8.0 us against
+// 9.5 by reciprocals), and formed where D is loaded (11.7 against 12.3 by a second load).
 template <int CZ>
 struct BigLayout {
   static constexpr int kP = 0;                                  // [CZ][W + 2][34]
@@ -640,8 +673,10 @@ struct BigLayout {
   static constexpr int kFx = CZ * kRW, kFy = CZ * 32, kFz = kRW * 32;
   static constexpr int kFaces = 2 * (kFx + kFy + kFz);
   static constexpr int kNY = CZ / 8, kNX = 2, kNH = 2 + kNY + kNX;  // halo cells per thread
-  static constexpr int kRh = kTx + CZ * kRW;                    // r of the y and x halo cells
-  static constexpr int kFloats = kRh + (kNY + kNX) * kRT;
+  static constexpr int kRh = kTx + CZ * kRW;                    // r (z) of the y and x halo cells
+  static constexpr int kD = kRh + (kNY + kNX) * kRT;            // D [CZ][W][32], where it fits
+  static constexpr bool kHasD = CZ <= 24;
+  static constexpr int kFloats = kD + (kHasD ? CZ * kRT : 0);
   static_assert(CZ % 8 == 0 && CZ <= 32, "halo rows per warp");
 };
 
@@ -678,13 +713,6 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     const uint2 u = __ldg(c16 + c);
     return make_float4(bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y));
   };
-  // S of a cell (Jacobi): the root of M^-1; 1 without preconditioner, 0 outside
-  auto root = [&](int64_t x, int64_t y, int64_t z) -> float {
-    if (!inside(x, y, z)) return 0.f;
-    if (!JAC) return 1.f;
-    const int64_t c = x + g.nx * y + g.plane * z;
-    return __fsqrt_rn(a.b16 ? __ldg(a.dinv + c) : jac_inv(__ldg(c32 + c).w));
-  };
   // D of an own cell (BF16 records: formed from the faces as the sweeps do)
   auto diag = [&](int64_t z, const float4& cf) -> float {
     if (!a.b16) return cf.w;
@@ -697,40 +725,45 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
   bool fault = false;
   float tscale = 1.f;
   {
-    float dmax = JAC ? 1.f : 0.f;  // S A S has a unit diagonal
-    if (!JAC && inxy)
+    float dmax = 0.f;
+    if (inxy)
       for (int k = 0; k < CZ && Z0 + k < g.nz; ++k)
         dmax = fmaxf(dmax, diag(Z0 + k, rec(gx, gy, Z0 + k)));
     tscale = operator_scale(a, blk, dmax, ++epoch, sh, fault);
   }
-  // every face value is (T s_low) s_high in both its cells
   float2* pk = a.packed + ((size_t)blk * CZ * kRW + warp) * 32 + lane;           // (Tx, Tz)
-  float* pd = reinterpret_cast<float*>(a.packed + (size_t)a.nblk * CZ * kRT) +
-              ((size_t)blk * CZ * kRW + warp) * 32 + lane;                         // D
-  const float tzlo = inxy ? rec(gx, gy, Z0 - 1).z * tscale * root(gx, gy, Z0 - 1) *
-                                root(gx, gy, Z0) : 0.f;
+  // D, or M^-1 (Jacobi) where D is in shared memory
+  float* pe = reinterpret_cast<float*>(a.packed + (size_t)a.nblk * CZ * kRT) +
+              ((size_t)blk * CZ * kRW + warp) * 32 + lane;
+  constexpr bool kLoadE = JAC || !LY::kHasD;
+  float* sD = sm + LY::kD + tid;
+  const float mscale = 1.f / tscale;  // exact: a power of two
+  // M^-1 of a cell, 0 outside
+  auto minv = [&](int64_t x, int64_t y, int64_t z) -> float {
+    if (!inside(x, y, z)) return 0.f;
+    const int64_t c = x + g.nx * y + g.plane * z;
+    return mscale * (a.b16 ? __ldg(a.dinv + c) : jac_inv(__ldg(c32 + c).w));
+  };
+  const float tzlo = inxy ? rec(gx, gy, Z0 - 1).z * tscale : 0.f;
 #pragma unroll 1
   for (int k = 0; k < CZ; ++k) {
     const int64_t z = Z0 + k;
     const float4 cf = rec(gx, gy, z);
-    const float sc = root(gx, gy, z);
     const bool in = inxy && z < g.nz;
-    const float D = in ? diag(z, cf) : 0.f;
-    pk[(size_t)k * kRT] = make_float2(cf.x * tscale * sc * root(gx + 1, gy, z),
-                                      cf.z * tscale * sc * root(gx, gy, z + 1));
-    pd[(size_t)k * kRT] = D * tscale * sc * sc;
-    sTy[(k * (kRW + 1) + warp + 1) * 32 + lane] = cf.y * tscale * sc * root(gx, gy + 1, z);
-    if (warp == 0)
-      sTy[k * (kRW + 1) * 32 + lane] = rec(gx, gy - 1, z).y * tscale * root(gx, gy - 1, z) * sc;
-    if (lane == 0)
-      sTx[k * kRW + warp] = rec(gx - 1, gy, z).x * tscale * root(gx - 1, gy, z) * sc;
+    pk[(size_t)k * kRT] = make_float2(cf.x * tscale, cf.z * tscale);
+    const float D = in ? diag(z, cf) * tscale : 0.f;
+    if (LY::kHasD) sD[k * kRT] = D;
+    if (kLoadE) pe[(size_t)k * kRT] = LY::kHasD ? minv(gx, gy, z) : D;
+    sTy[(k * (kRW + 1) + warp + 1) * 32 + lane] = cf.y * tscale;
+    if (warp == 0) sTy[k * (kRW + 1) * 32 + lane] = rec(gx, gy - 1, z).y * tscale;
+    if (lane == 0) sTx[k * kRW + warp] = rec(gx - 1, gy, z).x * tscale;
     sX[(k * kRW + warp) * 32 + lane] = 0.f;
   }
   for (int i = tid; i < CZ * (kRW + 2) * 34; i += kRT) sP[i] = 0.f;
   __syncthreads();
 
   // ---- halo cells: 0, 1 below and above; kNY y rows; kNX x cells -------------------
-  ResComm<NH, false> cm;
+  ResComm<NH, false, 4> cm;
   cm.part = a.part;
   cm.face = a.face;
   cm.nblk = a.nblk;
@@ -738,40 +771,55 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
   cm.face_buf = (size_t)a.nblk * LY::kFaces;
   float rz[2] = {0.f, 0.f}, pz[2] = {0.f, 0.f}, qh[NH];
   // y rows: row id warp + 16 j counts (side, k); x cells: tid + 512 j counts (side, w, k)
-  auto yk = [&](int j) { return (warp + kRW * j) % CZ; };
-  auto yhi = [&](int j) { return warp + kRW * j >= CZ; };
-  auto xk = [&](int j) { return (tid + kRT * j) % LY::kFx % CZ; };
-  auto xw = [&](int j) { return (tid + kRT * j) % LY::kFx / CZ; };
-  auto xhi = [&](int j) { return tid + kRT * j >= LY::kFx; };
+  // (indices from `ht`, which is made opaque in every iteration: as invariants they
+  // would be held in registers)
+  int ht = tid;
+  auto yk = [&](int j) { return ((ht >> 5) + kRW * j) % CZ; };
+  auto yhi = [&](int j) { return (ht >> 5) + kRW * j >= CZ; };
+  auto xk = [&](int j) { return (ht + kRT * j) % LY::kFx % CZ; };
+  auto xw = [&](int j) { return (ht + kRT * j) % LY::kFx / CZ; };
+  auto xhi = [&](int j) { return ht + kRT * j >= LY::kFx; };
+  unsigned halo = (bz > 0 ? 1u : 0u) | (bz + 1 < a.nbz ? 2u : 0u);
+#pragma unroll
+  for (int j = 0; j < LY::kNY; ++j)
+    if (yhi(j) ? by + 1 < a.nby : by > 0) halo |= 4u << j;
+#pragma unroll
+  for (int j = 0; j < LY::kNX; ++j)
+    if (tid + kRT * j < 2 * LY::kFx && (xhi(j) ? bx + 1 < a.nbx : bx > 0)) halo |= 4u << (LY::kNY + j);
+  auto hoff = [&](int j) {
+    constexpr int fy = 2 * LY::kFx, fz = 2 * (LY::kFx + LY::kFy);
+    if (j == 0) return (blk - a.nbx * a.nby) * LY::kFaces + fz + LY::kFz + ht;
+    if (j == 1) return (blk + a.nbx * a.nby) * LY::kFaces + fz + ht;
+    if (j < 2 + LY::kNY) {
+      const int w = yk(j - 2) * 32 + (ht & 31);
+      return yhi(j - 2) ? (blk + a.nbx) * LY::kFaces + fy + w
+                        : (blk - a.nbx) * LY::kFaces + fy + LY::kFy + w;
+    }
+    const int i = j - 2 - LY::kNY, w = (ht + kRT * i) % LY::kFx;
+    return xhi(i) ? (blk + 1) * LY::kFaces + w : (blk - 1) * LY::kFaces + LY::kFx + w;
+  };
+  auto has = [&](int j) { return ((halo >> j) & 1u) != 0u; };
+  const FaceWords<decltype(has), decltype(hoff)> wd{has, hoff};
+  // the vector of a cell: r, or z = M^-1 r
   auto halo_r = [&](int64_t x, int64_t y, int64_t z) -> float {
     if (!inside(x, y, z)) return 0.f;
-    return (float)(scale * a.r64[x + g.nx * y + g.plane * z]) * root(x, y, z);
+    const float v = (float)(scale * a.r64[x + g.nx * y + g.plane * z]);
+    return JAC ? v * minv(x, y, z) : v;
   };
   {
-    const int fz = 2 * (LY::kFx + LY::kFy), fy = 2 * LY::kFx;
-    cm.hoff[0] = bz > 0 ? (blk - a.nbx * a.nby) * LY::kFaces + fz + LY::kFz + tid : -1;
-    cm.hoff[1] = bz + 1 < a.nbz ? (blk + a.nbx * a.nby) * LY::kFaces + fz + tid : -1;
     rz[0] = halo_r(gx, gy, Z0 - 1);
     rz[1] = halo_r(gx, gy, Z0 + CZ);
 #pragma unroll
     for (int j = 0; j < LY::kNY; ++j) {
-      const int w = yk(j) * 32 + lane;
-      cm.hoff[2 + j] = yhi(j) ? (by + 1 < a.nby ? (blk + a.nbx) * LY::kFaces + fy + w : -1)
-                              : (by > 0 ? (blk - a.nbx) * LY::kFaces + fy + LY::kFy + w : -1);
-      sRh[j * kRT + tid] =
-          halo_r(gx, kRW * (int64_t)by + (yhi(j) ? kRW : -1), Z0 + yk(j));
+      const int64_t y = kRW * (int64_t)by + (yhi(j) ? kRW : -1), z = Z0 + yk(j);
+      sRh[j * kRT + tid] = halo_r(gx, y, z);
     }
 #pragma unroll
     for (int j = 0; j < LY::kNX; ++j) {
       const bool use = tid + kRT * j < 2 * LY::kFx;
-      const int w = xw(j) * CZ + xk(j);
-      cm.hoff[2 + LY::kNY + j] =
-          !use ? -1
-               : xhi(j) ? (bx + 1 < a.nbx ? (blk + 1) * LY::kFaces + w : -1)
-                        : (bx > 0 ? (blk - 1) * LY::kFaces + LY::kFx + w : -1);
-      sRh[(LY::kNY + j) * kRT + tid] =
-          use ? halo_r(32 * (int64_t)bx + (xhi(j) ? 32 : -1), kRW * (int64_t)by + xw(j), Z0 + xk(j))
-              : 0.f;
+      const int64_t x = 32 * (int64_t)bx + (xhi(j) ? 32 : -1), y = kRW * (int64_t)by + xw(j),
+                    z = Z0 + xk(j);
+      sRh[(LY::kNY + j) * kRT + tid] = use ? halo_r(x, y, z) : 0.f;
     }
 #pragma unroll
     for (int j = 0; j < NH; ++j) qh[j] = 0.f;
@@ -786,25 +834,24 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
 
   float alpha = 0.f, beta = 0.f;
   int done = kRunning;
-  ResScalars sc;  // (warp 0)
-  sc.init();
+  if (tid == 0) sh.sc.init();
   uint2* fmine = a.face + (size_t)blk * LY::kFaces;
 
   auto step = [&](bool dir, Acc& s0) {
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      if (cm.hoff[j] < 0) continue;
+      if (!((halo >> j) & 1u)) continue;
       rz[j] = fmaf(-alpha, qh[j], rz[j]);
       if (dir) pz[j] = fmaf(beta, pz[j], rz[j]);
     }
 #pragma unroll
     for (int j = 0; j < LY::kNY + LY::kNX; ++j) {
-      if (cm.hoff[2 + j] < 0) continue;
-      const float rn = fmaf(-alpha, qh[2 + j], sRh[j * kRT + tid]);
-      sRh[j * kRT + tid] = rn;
+      if (!((halo >> (2 + j)) & 1u)) continue;
+      const float rn = fmaf(-alpha, qh[2 + j], sRh[j * kRT + ht]);
+      sRh[j * kRT + ht] = rn;
       if (!dir) continue;
       const int i = j - LY::kNY;
-      float* ps = j < LY::kNY ? sP + (yk(j) * (kRW + 2) + (yhi(j) ? kRW + 1 : 0)) * 34 + lane + 1
+      float* ps = j < LY::kNY ? sP + (yk(j) * (kRW + 2) + (yhi(j) ? kRW + 1 : 0)) * 34 + (ht & 31) + 1
                               : sP + (xk(i) * (kRW + 2) + xw(i) + 1) * 34 + (xhi(i) ? 33 : 0);
       *ps = fmaf(beta, *ps, rn);
     }
@@ -817,7 +864,9 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
       *xs = fmaf(alpha, p0, *xs);
       r[k] = fmaf(-alpha, q[k], r[k]);
       if (dir) *ps = fmaf(beta, p0, r[k]);
-      s = fmaf(r[k], r[k], s);
+      if (JAC && dir) continue;  // r'z is formed with D, in the stencil
+      const float D = !JAC ? 1.f : LY::kHasD ? sD[k * kRT] : __ldcg(pe + (size_t)k * kRT);
+      s = fmaf(JAC ? r[k] * D : r[k], r[k], s);
       if ((k & 3) == 3) {
         kadd(s0, s);
         s = 0.f;
@@ -826,21 +875,22 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
   };
 
   while (!fault) {
+    asm volatile("" : "+r"(ht));
     Acc acc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
     // the first planes' coefficients, in flight during the step
     constexpr int kPre = 4;
     float2 tc[kPre];
-    float dc[kPre];
+    float ec[kPre];
 #pragma unroll
     for (int k = 0; k < kPre; ++k) {
       tc[k] = __ldcg(pk + (size_t)k * kRT);
-      dc[k] = __ldcg(pd + (size_t)k * kRT);
+      if (kLoadE) ec[k] = __ldcg(pe + (size_t)k * kRT);
     }
     step(true, acc[0]);
     __syncthreads();
     ++epoch;
     uint2* fo = fmine + (epoch & 1u) * cm.face_buf;
-    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
     float tz0 = tzlo, pm = pz[0];
     float pc = sP[(warp + 1) * 34 + lane + 1];
 #pragma unroll
@@ -849,24 +899,27 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
       const float pp = k + 1 < CZ ? ps[(kRW + 2) * 34] : pz[1];
       const float* ty = sTy + (k * (kRW + 1) + warp) * 32 + lane;
       const float2 t = tc[k % kPre];
-      const float D = dc[k % kPre];
+      const float D = LY::kHasD ? sD[k * kRT] : ec[k % kPre];
+      const float m = !JAC ? 1.f : LY::kHasD ? ec[k % kPre] : jac_inv(D);
       if (k + kPre < CZ) {
         tc[k % kPre] = __ldcg(pk + (size_t)(k + kPre) * kRT);
-        dc[k % kPre] = __ldcg(pd + (size_t)(k + kPre) * kRT);
+        if (kLoadE) ec[k % kPre] = __ldcg(pe + (size_t)(k + kPre) * kRT);
       }
       float txm = __shfl_up_sync(kFull, t.x, 1);
       if (lane == 0) txm = sTx[k * kRW + warp];
       const float4 cf = make_float4(t.x, ty[32], t.y, D);
       const float v = stencil7(cf, txm, ty[0], tz0, pc, ps[1], ps[-1], ps[34], ps[-34], pp, pm);
-      q[k] = v;
+      q[k] = JAC ? v * m : v;
+      if (JAC) s0 = fmaf(r[k] * D, r[k], s0);
       s1 = fmaf(pc, v, s1);
       s2 = fmaf(r[k], v, s2);
-      s3 = fmaf(v, v, s3);
+      s3 = fmaf(v, q[k], s3);
       if ((k & 3) == 3) {
+        if (JAC) kadd(acc[0], s0);
         kadd(acc[1], s1);
         kadd(acc[2], s2);
         kadd(acc[3], s3);
-        s1 = s2 = s3 = 0.f;
+        s0 = s1 = s2 = s3 = 0.f;
       }
       tz0 = t.y;
       pm = pc;
@@ -895,13 +948,17 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     Dfl mine[4], tot[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) mine[v] = df_fast(acc[v].s, -acc[v].c);
-    if (!cm.exchange(a, mine, epoch, tot, qh, sh)) {
+    if (!cm.template exchange<true>(a, mine, epoch, wd, tot, qh, sh)) {
       fault = true;
       break;
     }
     if (warp == 0) {
+      ResScalars sc = sh.sc;
       sc.update(tot, a.rtol2, a.maxit);
-      if (lane == 0) sh.next = {sc.alpha, sc.beta, sc.done};
+      if (lane == 0) {
+        sh.sc = sc;
+        sh.next = {sc.alpha, sc.beta, sc.done};
+      }
     }
     __syncthreads();
     alpha = sh.next.alpha;
@@ -910,27 +967,23 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     if (done == kRunning) continue;
     if (done != kConvEst && done != kMaxit) break;
     // the last step, and the true r'r of the residual it leaves (no face words)
-    Acc s0 = {0.f, 0.f};
-    step(false, s0);
+    Acc rr = {0.f, 0.f};
+    step(false, rr);
     ++epoch;
-    int keep[NH];
-#pragma unroll
-    for (int j = 0; j < NH; ++j) {
-      keep[j] = cm.hoff[j];
-      cm.hoff[j] = -1;
-    }
-    mine[0] = df_fast(s0.s, -s0.c);
+    mine[0] = df_fast(rr.s, -rr.c);
     mine[1] = mine[2] = mine[3] = {0.f, 0.f};
-    const bool ok = cm.exchange(a, mine, epoch, tot, qh, sh);
-#pragma unroll
-    for (int j = 0; j < NH; ++j) cm.hoff[j] = keep[j];
+    const bool ok = cm.template exchange<false>(a, mine, epoch, wd, tot, qh, sh);
     if (!ok) {
       fault = true;
       break;
     }
     if (warp == 0) {
+      ResScalars sc = sh.sc;
       sc.finish(tot, a.maxit);
-      if (lane == 0) sh.next = {sc.alpha, sc.beta, sc.done};
+      if (lane == 0) {
+        sh.sc = sc;
+        sh.next = {sc.alpha, sc.beta, sc.done};
+      }
     }
     __syncthreads();
     alpha = sh.next.alpha;
@@ -944,12 +997,11 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     const double inv = (double)tscale / scale;
     for (int k = 0; k < CZ && Z0 + k < g.nz; ++k) {
       const int64_t c = c0 + g.plane * (Z0 + k);
-      const double e = (double)sX[(k * kRW + warp) * 32 + lane] * (double)root(gx, gy, Z0 + k);
-      a.x64[c] = fma(e, inv, a.x64[c]);
+      a.x64[c] = fma((double)sX[(k * kRW + warp) * 32 + lane], inv, a.x64[c]);
     }
   }
   if (blk == 0 && tid == 0) {
-    sc.report(st, scale, fault);
+    sh.sc.report(st, scale, fault);
     *(volatile uint32_t*)a.ctl = epoch;
   }
 }

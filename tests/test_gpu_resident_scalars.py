@@ -1,4 +1,5 @@
-"""Scalars of the resident CG over the whole FP32 range."""
+"""Precision of the resident CG: scalars over the whole FP32 range, iterations of the
+sweep on high-contrast fields."""
 import pytest
 import torch
 
@@ -42,3 +43,27 @@ def test_inner_tolerance_of_1e20(tp, shape, precond):
     assert a["rel_res_inner"] <= 1.01e-20
     assert abs(a["iters"] - s["iters"]) <= 0.1 * s["iters"], (a, s)
     assert a["rel_res_fp64"] <= 2 * s["rel_res_fp64"], (a, s)
+
+
+@pytest.mark.parametrize("b16", [False, True], ids=["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(100, 100, 100), (128, 128, 80), (128, 128, 120)])
+def test_jacobi_iterations_of_tall_bricks(tp, shape, b16):
+    """High-contrast fields (channels 1e4 times more permeable) over bricks of 24 and 32
+    planes: the operator of the inner solve is that of the records, so the resident
+    Jacobi solve takes the iterations of the sweep, to 3 % over four fields."""
+    nx, ny, nz = shape
+    total = [0, 0]
+    for seed in range(4):
+        K = torch.from_numpy(synth.channelized_field(nx, ny, nz, 2.0, 60 + seed)).cuda()
+        mask, pD = (torch.from_numpy(v).cuda() for v in synth.dirichlet_faces(nx, ny, nz, "x", 1.0, 0.0))
+        for sweep in (0, 1):
+            with tp.Context(*shape) as ctx:
+                ctx.set_option("precond", 1)
+                ctx.set_option("sweep", sweep)
+                coef, coef64 = ctx.build_trans(K, mask, None, 0.0)
+                inner = ctx.build_trans_bf16(K, mask, None, 0.0) if b16 else coef
+                b = ctx.build_rhs(K, mask, None, pD)
+                _, info = ctx.cg_solve(inner, coef64, b, tol=1e-12, maxit=100000, check=False)
+                assert info["code"] == 0, info
+                total[sweep] += info["iters"]
+    assert abs(total[0] - total[1]) <= 0.03 * total[1], total
