@@ -298,10 +298,11 @@ int cg_solve_bf16(tpfa_ctx* ctx, const uint16_t* coef16, const double* coef64, c
  * innermost inside the instance.  The CG iterations of all instances run as
  * one sweep launch per iteration inside one CUDA-graph while loop; each
  * instance has its own scalars and convergence flag, and the blocks of a
- * converged instance return immediately.  A batch whose instances each fit on
- * the chip (1.2 M cells on GB300) runs its inner solves in one cooperative
- * launch instead, whose SMs take the instances one after another (see cg_solve
- * for when; explicit z-runs are the sweeps' and do not matter there).
+ * converged instance return immediately.  Instances that fit on the chip (1.2 M
+ * cells on GB300) run their inner solves in cooperative launches instead, whose
+ * SMs take the instances one after another (see cg_solve for when; explicit
+ * z-runs are the sweeps' and do not matter there); what else is in the batch makes
+ * no difference to an instance's result once its z-run is given.
  */
 typedef struct tpfa_batch tpfa_batch;
 

@@ -4,10 +4,11 @@
 // the instance).  The CG iterations of all instances run as one sweep launch
 // per iteration inside one CUDA-graph while loop; each instance keeps its
 // own scalars, completion counter and convergence flag, and the blocks of a
-// converged instance return at once.  Batches whose instances fit on the chip run
-// their inner solves in one cooperative launch instead (resident.cu).  Coefficients, right-hand sides, FP64
-// residuals and the refinement steps are launched per instance (a handful of
-// launches per refinement step).
+// converged instance return at once.  Instances that fit on the chip run their inner
+// solves in cooperative launches instead (resident.cu), whatever else is in the batch,
+// so that an instance's result does not depend on its company.  Coefficients,
+// right-hand sides, FP64 residuals and the refinement steps are launched per instance
+// (a handful of launches per refinement step).
 #include <math.h>
 #include <string.h>
 
@@ -51,15 +52,11 @@ bool batch_tma(const tpfa_batch* b) {
   return true;
 }
 
-// The inner solves run in the resident kernel when every instance fits on the
-// chip, unless a sweep or a tile is asked for (z-runs are those of the sweeps).
-bool batch_resident(const tpfa_batch* b) {
-  if (b->sweep_sel != 0 || b->tma_tile != 0 || b->resident_off || b->ninst > kResMaxProb)
-    return false;
-  ResPlan p;
-  for (int i = 0; i < b->ninst; ++i)
-    if (!plan_resident(b->g[i], b->num_sms, true, &p)) return false;
-  return true;
+// The inner solves of an instance that fits on the chip run in the resident kernel,
+// unless a sweep or a tile is asked for (z-runs are those of the sweeps).
+bool batch_resident(const tpfa_batch* b, int i, ResPlan* p) {
+  return b->sweep_sel == 0 && b->tma_tile == 0 && !b->resident_off && b->ninst <= kResMaxProb &&
+         plan_resident(b->g[i], b->num_sms, true, p);
 }
 
 // Plans and buffers of the resident solves, on first use; the exchange words are
@@ -72,8 +69,11 @@ int setup_batch_resident(tpfa_batch* b, cudaStream_t s) {
   b->comm_off.resize(N);
   size_t words = 0, blocks = 0;
   for (int i = 0; i < N; ++i) {
-    if (!plan_resident(b->g[i], b->num_sms, true, &b->rplan[i])) return TPFA_EINVAL;
     b->comm_off[i] = words;
+    if (!plan_resident(b->g[i], b->num_sms, true, &b->rplan[i])) {
+      b->rplan[i].nblk = 0;
+      continue;
+    }
     words += (b->rplan[i].words + 31) / 32 * 32;
     blocks += (size_t)b->rplan[i].nblk;
   }
@@ -533,10 +533,22 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
     return TPFA_EINVAL;
   if ((const void*)rhs == (const void*)x) return TPFA_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
-  const bool resident = batch_resident(b);
-  rc = resident ? setup_batch_resident(b, s) : ensure_batch_loop(b, coef, s);
-  if (rc) return rc;
   const int N = b->ninst;
+  std::vector<char> res(N);  // instances solved in the resident kernel
+  int nres = 0;
+  for (int i = 0; i < N; ++i) {
+    ResPlan p;
+    res[i] = batch_resident(b, i, &p);
+    nres += res[i];
+  }
+  if (nres < N) {
+    rc = ensure_batch_loop(b, coef, s);
+    if (rc) return rc;
+  }
+  if (nres > 0) {
+    rc = setup_batch_resident(b, s);
+    if (rc) return rc;
+  }
   std::vector<ResProb> probs;
   const float4* cf = reinterpret_cast<const float4*>(coef);
   unsigned int* ecounter = b->counters + N;  // shared by the per-instance helper kernels
@@ -590,11 +602,18 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       }
     }
     if (nact == 0) break;
-    if (resident) {
+    // the resident instances' solves, then the others' sweeps, in which those and the
+    // inactive instances are marked done, so that their blocks return at once
+    std::vector<int> order;
+    for (int i = 0; i < N; ++i) {
+      if (active[i] && res[i]) order.push_back(i);
+      hs[i].done = active[i] && res[i] ? kGuard  // what a team that never ran would leave
+                                       : kConvTrue;
+    }
+    const bool sweeps = nact > (int)order.size();
+    BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
+    if (!order.empty()) {
       probs.clear();
-      std::vector<int> order;
-      for (int i = 0; i < N; ++i)
-        if (active[i]) order.push_back(i);
       // one launch per brick height; largest teams first, among equals the
       // longest solve of the last step
       std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
@@ -622,8 +641,6 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       BK(cudaStreamSynchronize(s));
       // the stream is idle: nothing the launch waits for can need the lock
       std::lock_guard<std::mutex> lock(resident_mutex(b->device));
-      for (int i : order) hs[i].done = kGuard;  // what a team that never ran would leave
-      BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
       BK(cudaEventRecord(b->ev[2], s));
       cudaError_t e = cudaSuccess;
       for (size_t p0 = 0, p1 = 0; p0 < probs.size() && e == cudaSuccess; p0 = p1) {
@@ -649,16 +666,10 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
         if (gave_up) BK(cudaMemsetAsync(b->comm, 0, b->comm_words * 8, s));
       }
     }
-    if (resident && b->resident_off)
+    if (!order.empty() && b->resident_off)
       return cg_solve_batch(b, coef, coef64, rhs, x, tol, maxit, infos, total, stream);
-    // inactive instances: mark done so their sweep blocks return at once
-    if (!resident) {
-      for (int i = 0; i < N; ++i)
-        if (!active[i]) hs[i].done = kConvTrue;
-      BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
-    }
-    for (int i = 0; i < N && !resident; ++i) {
-      if (!active[i]) continue;
+    for (int i = 0; i < N; ++i) {
+      if (!active[i] || res[i]) continue;
       double rtol = 0.5 * tol / rel[i];
       if (rtol < b->inner_rtol) rtol = b->inner_rtol;
       if (rtol > 0.5) rtol = 0.5;
@@ -667,7 +678,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       ++launches;
     }
     // while any instance runs: batched sweep + condition (guarded)
-    for (int relaunch = 0; !resident; ++relaunch) {
+    for (int relaunch = 0; sweeps; ++relaunch) {
       // the captured condition kernel stops the loop once the sweep counter
       // passes 0: start it at minus the guard limit
       const long long start = -(2 * mx + 64);
@@ -676,7 +687,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       BK(cudaGraphLaunch(b->loop_exec, s));
       BK(cudaEventRecord(b->ev[3], s));
       for (int i = 0; i < N; ++i) {
-        if (!active[i]) continue;
+        if (!active[i] || res[i]) continue;
         BK(launch_finalize(b->g[i], vecs_at(b->v, b->off[i]), b->st + i, b->partials, ecounter,
                            elem_blocks(b->g[i], b->num_sms),
                            b->precond ? cf + b->off[i] : nullptr, nullptr, s));
@@ -692,13 +703,13 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
         if (active[i] && hs[i].done == kRunning) ++again;
       if (again == 0 || relaunch > 64) break;
     }
-    if (!resident) {
+    if (sweeps) {
       // every batched sweep launch (and the condition kernel after it) is
       // counted once in each instance's state: the most any instance saw
-      long long sweeps = 0;
+      long long most = 0;
       for (int i = 0; i < N; ++i)
-        if (active[i] && hs[i].launches > sweeps) sweeps = hs[i].launches;
-      launches += 2 * sweeps;
+        if (active[i] && !res[i] && hs[i].launches > most) most = hs[i].launches;
+      launches += 2 * most;
     }
     for (int i = 0; i < N; ++i) {
       if (!active[i]) continue;
@@ -712,7 +723,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
     for (int i = 0; i < N; ++i) {
       if (!active[i]) continue;
       const int64_t o = b->off[i];
-      if (!resident) {  // the resident kernel has added its correction
+      if (!res[i]) {  // the resident kernel has added its correction
         BK(launch_correct(b->g[i], vecs_at(b->v, o), x + o, b->st + i, s));
         ++launches;
       }

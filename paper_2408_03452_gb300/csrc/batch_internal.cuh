@@ -41,7 +41,7 @@ struct tpfa_batch {
   CUtensorMap* maps_dev;
   int64_t tma_blocks;
   size_t partials_cap;  // doubles
-  // resident inner solves (instances that all fit on the chip): plans, exchange
+  // resident inner solves (instances that fit on the chip; others: nblk = 0): plans, exchange
   // buffers of every instance (comm_off: first word), teams, table, scheduler
   std::vector<tpfa::ResPlan> rplan;
   std::vector<size_t> comm_off;
