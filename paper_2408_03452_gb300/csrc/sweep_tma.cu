@@ -117,6 +117,15 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
+// The warp is done with a stage.  The fence keeps the copy that refills it behind every
+// lane's reads: an arrival does not wait for loads whose values nothing has used yet
+// (p and Tz below the first plane of a run), and with another stream's traffic in the
+// load pipe they came a microsecond later, from the refilled stage.
+__device__ __forceinline__ void release_stage(uint64_t* empty) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
+}
 __device__ __forceinline__ void tma_3d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, int y,
                                        int z) {
   asm volatile(
@@ -294,10 +303,7 @@ cg_sweep_tma_kernel(const __grid_constant__ TmaArgs a) {
     auto wait_full = [&](int j) -> bool {
       return mbar_wait(&full[j % S], (j / S) & 1, kWaitLimit);
     };
-    auto release = [&](int j) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[j % S]);
-    };
+    auto release = [&](int j) { release_stage(&empty[j % S]); };
 
     float Pm[VY], P0[VY + 2], R0[VY], Z0[VY], H0[VY], E0[VY], Tzm[VY];
     float s0 = 0.f;
@@ -629,10 +635,7 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
     auto wait_full = [&](int j) -> bool {
       return mbar_wait(&full[j % S], (j / S) & 1, kWaitLimit);
     };
-    auto release = [&](int j) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[j % S]);
-    };
+    auto release = [&](int j) { release_stage(&empty[j % S]); };
 
     float Pm[VY], P0[VY + 2], H0[VY], Tzm[VY];
     int64_t zdone = z0;  // first plane of the run not yet written

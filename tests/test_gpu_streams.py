@@ -132,3 +132,65 @@ def test_batched_sweeps_and_flexible_cg_on_a_side_stream(tp):
         xs.append(x.cpu().numpy())
         es.append(e.cpu().numpy())
     assert np.array_equal(*xs) and np.array_equal(*es)
+
+
+@pytest.mark.parametrize("bf16", [False, True], ids=["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(24, 20, 12), (64, 33, 40)])
+def test_operator_beside_another_stream(tp, shape, bf16):
+    """The operator on a vector rewritten before each call, quiet and beside traffic
+    that fills the load pipes: bit for bit the same (a stage of the ring is refilled
+    only when every lane has read it)."""
+    nx, ny, nz = shape
+    n = nx * ny * nz
+    K = torch.from_numpy(synth.lognormal_field(nx, ny, nz, 1.0, 51)).cuda()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    ps = [torch.randn(n, generator=g, device="cuda") for _ in range(150)]
+    work = torch.empty(n, device="cuda")
+    side = torch.cuda.Stream()
+    with tp.Context(*shape) as ctx:
+        coef = ctx.build_trans_bf16(K, None, None, 1e-3) if bf16 else ctx.build_trans(K, None, None, 1e-3)[0]
+        op = ctx.apply_bf16 if bf16 else ctx.apply
+        out = [[torch.empty(n, device="cuda") for _ in ps] for _ in range(2)]
+        torch.cuda.synchronize()
+        for p, y in zip(ps, out[0]):
+            work.copy_(p)
+            op(coef, work, y)
+        for _ in range(6):
+            torch.cuda.synchronize()
+            keep = _busy()
+            with torch.cuda.stream(side):
+                for p, y in zip(ps, out[1]):
+                    work.copy_(p)
+                    op(coef, work, y)
+            torch.cuda.synchronize()
+            del keep
+            assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("levels", [0, 1, 2])
+def test_learned_solve_beside_another_stream(tp, levels):
+    """Flexible CG with a network, whose operator also forms the dot products (levels 1
+    and 2: of the network's coarser output), quiet and beside another stream."""
+    from paper_2408_03452_gb300 import learned
+    n = 32
+    coef, coef64, b = _system(tp, (n, n, n), 52)
+    lnk = tp.log_perm(torch.from_numpy(synth.lognormal_field(n, n, n, 1.0, 52)).cuda())
+    net = tp.UNet(*(3 * [n >> levels]))
+    net.set_params(learned.init_params(4).cuda())
+    side = torch.cuda.Stream()
+    xs = []
+    with tp.Context(n, n, n) as ctx:
+        ctx.set_option("fcg_m", 2)
+        for busy in (False, True, True, True):
+            x = torch.zeros_like(b)
+            torch.cuda.synchronize()
+            keep = _busy() if busy else None
+            with torch.cuda.stream(side):
+                _, info = ctx.fcg_solve(coef, coef64, b, net=net, lnk=lnk, x=x, tol=1e-8, maxit=3000,
+                                        check=False)
+            torch.cuda.synchronize()
+            del keep
+            xs.append((x.cpu().numpy(), info["iters"], info["code"]))
+    assert xs[0][2] == 0
+    for x, it, _ in xs[1:]:
+        assert it == xs[0][1] and np.array_equal(x, xs[0][0])
