@@ -4,6 +4,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <condition_variable>
+#include <mutex>
 #include <new>
 
 #include "tpfa_internal.cuh"
@@ -365,9 +367,35 @@ int read_state(tpfa_ctx* c, cudaStream_t s) {
 }  // namespace
 
 namespace tpfa {
-std::mutex& resident_mutex(int device) {
-  static std::mutex m[64];
-  return m[(unsigned)device % 64u];
+namespace {
+struct SmPool {
+  std::mutex m;
+  std::condition_variable cv;
+  int used = 0;
+  uint64_t next = 0, serving = 0;  // tickets
+};
+SmPool& sm_pool(int device) {
+  static SmPool pool[64];
+  return pool[(unsigned)device % 64u];
+}
+}  // namespace
+
+ResidentSms::ResidentSms(int device, int num_sms, int need) : device_(device), need_(need) {
+  SmPool& p = sm_pool(device);
+  std::unique_lock<std::mutex> lock(p.m);
+  const uint64_t ticket = p.next++;
+  p.cv.wait(lock, [&] {
+    return p.serving == ticket && (p.used == 0 || p.used + need <= num_sms);
+  });
+  p.used += need;
+  ++p.serving;
+  p.cv.notify_all();
+}
+ResidentSms::~ResidentSms() {
+  SmPool& p = sm_pool(device_);
+  std::lock_guard<std::mutex> lock(p.m);
+  p.used -= need_;
+  p.cv.notify_all();
 }
 
 int64_t ctx_cells(const tpfa_ctx* c) { return c ? c->g.n : 0; }
@@ -813,9 +841,9 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
       if (rtol > 0.5) rtol = 0.5;
       int inner_status = kRunning;
       if (resident) {
-        // the stream is idle here (the state was just read), so nothing the
-        // launch waits for can need the lock
-        std::lock_guard<std::mutex> lock(resident_mutex(c->device));
+        // the stream is idle here (the state was just read), so nothing the launch
+        // waits for can need the SMs it takes
+        ResidentSms sms(c->device, c->num_sms, rp.nblk);
         CK(cudaEventRecord(c->ev[2], s));
         ResProb prob = make_res_prob(c->g, rp, coef, b16, c->dinv, c->r64, x, c->st, rtol,
                                      (long long)(maxit - total_iters), c->comm);

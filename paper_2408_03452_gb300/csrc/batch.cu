@@ -639,8 +639,8 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       BK(cudaMemcpyAsync(b->prob_dev, probs.data(), sizeof(ResProb) * probs.size(),
                          cudaMemcpyHostToDevice, s));
       BK(cudaStreamSynchronize(s));
-      // the stream is idle: nothing the launch waits for can need the lock
-      std::lock_guard<std::mutex> lock(resident_mutex(b->device));
+      // the stream is idle: nothing the launch waits for can need the SMs it takes
+      ResidentSms sms(b->device, b->num_sms, b->num_sms);
       BK(cudaEventRecord(b->ev[2], s));
       cudaError_t e = cudaSuccess;
       for (size_t p0 = 0, p1 = 0; p0 < probs.size() && e == cudaSuccess; p0 = p1) {
@@ -649,6 +649,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
                                   b->precond == 1, b->sched, b->look_limit, s);
         ++launches;
       }
+      if (e != cudaSuccess) cudaStreamSynchronize(s);  // launches made before it hold SMs
       if (e == cudaErrorCooperativeLaunchTooLarge && step == 0) {
         // fewer SMs than the device reports: this batch keeps the sweeps
         cudaGetLastError();

@@ -5,8 +5,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <mutex>
-
 #include "sweep_plan.h"
 #include "tpfa.h"
 
@@ -274,10 +272,21 @@ uint32_t* resident_batch_beat(unsigned long long* sched);
 cudaError_t launch_resident_batch(const ResProb* prob_dev, int nprob, int cz, int num_sms,
                                   bool jac, unsigned long long* sched, uint32_t look_limit,
                                   cudaStream_t s);
-// Resident launches of one device are made one at a time (held from the launch
-// until the host has waited for it), so that the blocks of two of them never
-// compete for the same SMs.
-std::mutex& resident_mutex(int device);
+// SMs of a device that resident launches hold, from the launch until the host has
+// waited for it: every block of such a launch has to be running before any of them
+// ends, so launches that together need more SMs than there are could wait for each
+// other for ever.  Each block is counted as one SM (some share one); launches that fit
+// run side by side, the others wait their turn in the order they came.
+class ResidentSms {
+ public:
+  ResidentSms(int device, int num_sms, int need);
+  ~ResidentSms();
+  ResidentSms(const ResidentSms&) = delete;
+  ResidentSms& operator=(const ResidentSms&) = delete;
+
+ private:
+  int device_, need_;
+};
 
 // Argument checks shared by the entry points: a device (or managed)
 // allocation on `device` that holds [p, p + bytes) and is `align`-aligned.
