@@ -867,8 +867,11 @@ static int solve_impl(tpfa_ctx* c, const void* coef, bool b16, const double* coe
           float ms = 0.f;
           CK(cudaEventElapsedTime(&ms, c->ev[2], c->ev[3]));
           inner_ms += ms;
-          inner_status = hs->done;
-          if (inner_status == kGuard) CK(cudaMemsetAsync(c->comm, 0, c->comm_words * 8, s));
+          inner_status = hs->fault ? (int)kGuard : hs->done;
+          if (inner_status == kGuard) {
+            CK(cudaMemsetAsync(c->comm, 0, c->comm_words * 8, s));
+            CK(cudaMemsetAsync(&c->st->fault, 0, sizeof(int), s));
+          }
         }
       } else {
         CK(launch_prepare(c->g, c->r64, vecs, c->st, rtol, (long long)(maxit - total_iters), s));

@@ -609,6 +609,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       if (active[i] && res[i]) order.push_back(i);
       hs[i].done = active[i] && res[i] ? kGuard  // what a team that never ran would leave
                                        : kConvTrue;
+      hs[i].fault = 0;
     }
     const bool sweeps = nact > (int)order.size();
     BK(cudaMemcpyAsync(b->st, hs, sizeof(CgState) * N, cudaMemcpyHostToDevice, s));
@@ -663,7 +664,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
         BK(cudaEventElapsedTime(&ms, b->ev[2], b->ev[3]));
         inner_ms += ms;
         bool gave_up = false;
-        for (int i : order) gave_up = gave_up || hs[i].done == kGuard;
+        for (int i : order) gave_up = gave_up || hs[i].fault || hs[i].done == kGuard;
         if (gave_up) BK(cudaMemsetAsync(b->comm, 0, b->comm_words * 8, s));
       }
     }
@@ -716,7 +717,7 @@ int cg_solve_batch(tpfa_batch* b, const float* coef, const double* coef64, const
       if (!active[i]) continue;
       iters[i] += hs[i].iter;
       rel_inner[i] = hs[i].rho0 > 0 ? sqrt(hs[i].rho / hs[i].rho0) : 0.0;
-      const int d = hs[i].done;
+      const int d = hs[i].fault ? (int)kGuard : hs[i].done;
       if (d == kGuard || d == kRunning) { status[i] = TPFA_EINTERNAL; active[i] = 0; }
       else if (d == kNonFinite) { status[i] = TPFA_ENONFINITE; active[i] = 0; }
       else if (d == kBreakdown && hs[i].iter == 0) { status[i] = TPFA_EBREAKDOWN; active[i] = 0; }

@@ -148,7 +148,6 @@ struct ResScalars {
     st->iter = iter;
     st->launches = 1;
     st->done = fault ? (int)kGuard : done;
-    st->fault = fault ? 1 : 0;
   }
 };
 
@@ -631,6 +630,9 @@ __device__ __forceinline__ void resident_solve(const ResProb& a, int blk, float*
     if (done != kRunning) break;
   }
 
+  // a wait that ran out in any block, be it the last one's, whose brick then lacks its
+  // correction, is a failure of the solve (the host clears the flag)
+  if (fault && tid == 0) *(volatile int*)&st->fault = 1;
   if (fault) done = kGuard;
   // x64 += correction (the scaled operator's solution times the scale)
   if (done != kNonFinite && done != kGuard && inxy) {
@@ -992,6 +994,9 @@ __global__ void __launch_bounds__(kRT, 1) resident_big_kernel(const __grid_const
     if (done != kRunning) break;
   }
 
+  // a wait that ran out in any block, be it the last one's, whose brick then lacks its
+  // correction, is a failure of the solve (the host clears the flag)
+  if (fault && tid == 0) *(volatile int*)&st->fault = 1;
   if (fault) done = kGuard;
   if (done != kNonFinite && done != kGuard && inxy) {
     const double inv = (double)tscale / scale;
