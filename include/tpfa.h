@@ -315,6 +315,9 @@ int tpfa_batch_destroy(tpfa_batch* batch);
 int tpfa_batch_offsets(const tpfa_batch* batch, int64_t* offsets);
 /* zc: host, n_inst entries: the z-run length each instance uses. */
 int tpfa_batch_zc(const tpfa_batch* batch, int* zc);
+/* resident: host, n_inst entries: 1 where cg_solve_batch runs the instance's inner
+ * solves in the resident kernel under the options set, 0 where in the sweeps. */
+int tpfa_batch_resident(const tpfa_batch* batch, int* resident);
 /* TPFA_OPT_INNER_RTOL, TPFA_OPT_MAX_OUTER, TPFA_OPT_PRECOND; for fcg_solve_batch
  * also TPFA_OPT_FCG_M and TPFA_OPT_FCG_FALLBACK. */
 int tpfa_batch_set_option(tpfa_batch* batch, int option, double value);

@@ -16,9 +16,11 @@ so it is measured on the real solve:
      fixed.
 Each candidate is timed with CUDA events over a complete batched solve to the
 target tolerance.  Results can be cached in a JSON file keyed by the device
-name, the preconditioner, the tolerance and the size mix.  A batch whose
-instances fit on the chip is solved without sweeps unless TPFA_OPT_SWEEP asks for
-them (the cp.async candidate does), so its tilings time alike.
+name, the preconditioner, the tolerance, the size mix and a version that
+changes with the solver's choice of kernels.  Instances that fit on the chip
+are solved without sweeps, several times faster: a batch of such instances
+has nothing to tune and keeps the defaults, and in a mixed batch only the
+classes that run in the sweeps are searched.
 """
 from __future__ import annotations
 
@@ -31,6 +33,7 @@ from . import tpfa
 
 CANDIDATES = (4, 8, 16, 32, 64, 128)
 TMA_TILES = (0, 1, 2, 3)
+VERSION = "resident"  # entries from before the resident solves chose sweeps for every grid
 
 
 def _time_batch(grids, zc, coef, coef64, b, tol, maxit, precond, sweep=0, tile=0):
@@ -50,7 +53,16 @@ def _key(grids, precond, tol, what):
     counts = {s: sum(1 for g in grids if tuple(g[:3]) == s) for s in sizes}
     name = torch.cuda.get_device_name()
     return json.dumps([name, precond, tol, [[list(s), counts[s]] for s in sizes]] +
-                      ([what] if what else []))
+                      ([what] if what else []) + [VERSION])
+
+
+def _resident(grids, coef):
+    """Per instance: solved in the resident kernel by default (coef: the records to
+    be solved with, on the device that solves)."""
+    if coef is None:
+        return [False] * len(grids)
+    with torch.cuda.device(coef.device), tpfa.BatchContext(grids) as bc:
+        return bc.resident
 
 
 def _load(cache, key):
@@ -93,7 +105,9 @@ def tune_batch(grids, coef, coef64, b, tol=1e-8, maxit=100000, precond=0, cache=
                     "ms_per_solve": hit.get("ms_per_solve")}
         except (KeyError, TypeError, ValueError):
             pass
-    classes = sorted({tuple(g[:3]) for g in grids})
+    fits = _resident(grids, coef)
+    classes = sorted({tuple(g[:3]) for g, r in zip(grids, fits) if not r})
+    every = sorted({tuple(g[:3]) for g in grids})
 
     def run(assign, sweep, tile):
         zc = [assign[tuple(g[:3])] for g in grids]
@@ -103,12 +117,12 @@ def tune_batch(grids, coef, coef64, b, tol=1e-8, maxit=100000, precond=0, cache=
         return t
 
     best_t, best, bs, bt = None, None, 0, 0
-    for z in CANDIDATES:
-        assign = {c: z for c in classes}
+    for z in CANDIDATES if classes else CANDIDATES[:1]:
+        assign = {c: z for c in every}
         t = run(assign, 0, 0)
         if best_t is None or t < best_t:
             best_t, best = t, dict(assign)
-    if kernels:
+    if kernels and classes:
         shapes = [(0, tl) for tl in (TMA_TILES[1:] if not precond else ())] + [(1, 0)]
         for sw, tl in shapes:
             t = run(best, sw, tl)

@@ -431,6 +431,14 @@ int tpfa_batch_zc(const tpfa_batch* b, int* zc) {
   return TPFA_OK;
 }
 
+int tpfa_batch_resident(const tpfa_batch* b, int* resident) {
+  if (b == nullptr || resident == nullptr) return TPFA_EINVAL;
+  for (int i = 0; i < b->ninst; ++i) {
+    ResPlan p;
+    resident[i] = batch_resident(b, i, &p) ? 1 : 0;
+  }
+  return TPFA_OK;
+}
 
 int tpfa_batch_set_option(tpfa_batch* b, int option, double value) {
   if (b == nullptr || !isfinite(value)) return TPFA_EINVAL;

@@ -94,6 +94,7 @@ SIGNATURES = {
     "tpfa_batch_destroy": (C.c_int, [_P]),
     "tpfa_batch_offsets": (C.c_int, [_P, _P]),
     "tpfa_batch_zc": (C.c_int, [_P, _P]),
+    "tpfa_batch_resident": (C.c_int, [_P, _P]),
     "tpfa_batch_set_option": (C.c_int, [_P, C.c_int, C.c_double]),
     "tpfa_batch_build_trans": (C.c_int, [_P, _P, _P, _P, C.c_double, _P, _P, _P]),
     "tpfa_batch_build_rhs": (C.c_int, [_P, _P, _P, _P, _P, _P, _P]),
@@ -648,6 +649,13 @@ class BatchContext:
         z = (C.c_int * self.ninst)()
         _check(lib().tpfa_batch_zc(self._h, C.cast(z, C.c_void_p)), "tpfa_batch_zc")
         return [int(v) for v in z]
+
+    @property
+    def resident(self):
+        """Per instance: whether cg_solve runs its inner solves in the resident kernel."""
+        r = (C.c_int * self.ninst)()
+        _check(lib().tpfa_batch_resident(self._h, C.cast(r, C.c_void_p)), "tpfa_batch_resident")
+        return [bool(v) for v in r]
 
     def close(self):
         if self._h:
