@@ -1,9 +1,12 @@
 // 3x3x3 convolutions of BF16 channels-last volumes on the tcgen05 tensor
 // cores (implicit GEMM, FP32 accumulation in tensor memory).
 //
-// Forward (and input gradient).  An output tile is 128 consecutive voxel
-// indices of the haloed layout (halo voxels inside the range are computed
-// and discarded).  For one z-offset dz the three rows dy = -1, 0, 1 of 130
+// Forward (and input gradient).  The default is conv_fwd_ws_kernel: tiles of 8 x 16
+// voxels followed through the planes, whole voxel rows copied in the copy engine's
+// swizzle.  Kernels 0 to 2, taken by selection, stage blocks of 8 channels; kernel 0:
+//
+// An output tile is 128 consecutive voxel indices of the haloed layout (halo
+// voxels inside the range are computed and discarded).  For one z-offset dz the three rows dy = -1, 0, 1 of 130
 // voxels (the tile plus one voxel either side) are copied to shared memory
 // as "row groups" in the K-major core-matrix layout [CIN/8][130][8 channels],
 // i.e. 16 bytes per voxel and channel block.  With M-direction stride 128
@@ -1256,10 +1259,11 @@ cudaError_t zf_launch(const uint16_t* x, const uint16_t* w, const float* bias,
 }
 
 // Planes per unit: the split of the planes into runs with the fewest plane steps
-// on the busiest CTA (a run of zc outputs takes zc + 2 steps).  Measured, us: 64^3
-// 16 -> 16 with runs of 4 / 8 / 16 planes 17.5 / 16.3 / 18.5 (8 taken), 160^3
-// 148 / 132 / 124 (16 taken), 64^3 32 -> 64 33.8 / 33.7 / 33.6 (16 taken; linear
-// runs).
+// on the busiest CTA (a run of zc outputs takes zc + 2 steps).  Measured, us a call,
+// with runs of 4 / 8 / 16 / 24 planes and with the rule's: 16 -> 16 at 64^3 17.1 / 16.5 /
+// 18.6 / 24.8, rule 16.6; at 160^3 127 / 115 / 109 / 111, rule 107; 32 -> 64 at 64^3 32.9 /
+// 33.0 / 33.0 / 45.3, rule 33.0; 64 -> 32 at 64^3 39.1 / 35.0 / 37.1 / 53.4, rule 37.1; 32 ->
+// 16 at 96^3 44.2 / 39.6 / 43.2 / 37.9, rule 38.3.
 int ws_run(int nb, int nz, int ns, int ctas) {
   long long best = 0;
   int zc = nz;

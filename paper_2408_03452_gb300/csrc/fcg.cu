@@ -515,7 +515,7 @@ struct Work {
   float* lnkc = nullptr;
   int64_t launches = 0;
   // the TMA-staged operator fused with the blend's dot products (a batch of
-  // one): maps {coefficients, z, P slots, r, M^-1, Q slots}
+  // one): maps {coefficients, z, P slots, r, Q slots}
   bool fused = false;
   CUtensorMap* fmaps = nullptr;
   tpfa::TmaInst* finst = nullptr;
@@ -641,18 +641,17 @@ int setup_fused(const tpfa_ctx* c, const float* coef, Work& w) {
   if (!ctx_apply_tma_plan(c, &p, &g, w.levels > 0 ? 2 : 1) || reinterpret_cast<uintptr_t>(coef) % 16 != 0 ||
       w.m > kMaxDirs)
     return TPFA_OK;
-  const int per = 4 + 2 * w.m;
+  const int per = 3 + 2 * w.m;
   std::vector<CUtensorMap> maps(per);
-  std::vector<const float*> in(1 + w.m), own(2 + w.m);
+  std::vector<const float*> in(1 + w.m), own(1 + w.m);
   in[0] = w.z;
   own[0] = w.r;
-  own[1] = w.dinv;
   for (int k = 0; k < w.m; ++k) {
     in[1 + k] = w.P + (size_t)k * w.slot_stride();
-    own[2 + k] = w.Q + (size_t)k * w.slot_stride();
+    own[1 + k] = w.Q + (size_t)k * w.slot_stride();
   }
   if (!make_apply_maps(g, p, coef, in.data(), 1 + w.m, maps.data()) ||
-      !make_own_maps(g, p, own.data(), 2 + w.m, maps.data() + 2 + w.m))
+      !make_own_maps(g, p, own.data(), 1 + w.m, maps.data() + 2 + w.m))
     return TPFA_OK;  // the unfused passes
   TmaInst I{};
   I.g = g;

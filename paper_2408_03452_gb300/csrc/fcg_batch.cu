@@ -580,10 +580,10 @@ int setup_apply_tma(const tpfa_batch* batch, const float* coef, BWork& w) {
     return TPFA_OK;
   for (const Grid& g : batch->g)
     if (!tma_apply_ok(g, false)) return TPFA_OK;
-  // maps per instance: coefficients, z, P slots (with halo); r, M^-1, Q slots
+  // maps per instance: coefficients, z, P slots (with halo); r, Q slots
   // (own cells, for the fused dot products)
-  const int N = w.ninst, per = 4 + 2 * w.m;
-  std::vector<const float*> own(2 + w.m);
+  const int N = w.ninst, per = 3 + 2 * w.m;
+  std::vector<const float*> own(1 + w.m);
   const std::vector<int> zr = batch_tma_zc_request(batch);
   std::vector<CUtensorMap> maps((size_t)per * N);
   std::vector<TmaInst> inst(N);
@@ -595,11 +595,10 @@ int setup_apply_tma(const tpfa_batch* batch, const float* coef, BWork& w) {
     in[0] = w.z + o;
     for (int k = 0; k < w.m; ++k) in[1 + k] = w.P + (size_t)k * w.stride + o;
     own[0] = w.r + o;
-    own[1] = w.dinv + o;
-    for (int k = 0; k < w.m; ++k) own[2 + k] = w.Q + (size_t)k * w.stride + o;
+    for (int k = 0; k < w.m; ++k) own[1 + k] = w.Q + (size_t)k * w.stride + o;
     if (!make_apply_maps(batch->g[i], p, reinterpret_cast<const float4*>(coef) + o, in.data(),
                          1 + w.m, &maps[(size_t)per * i]) ||
-        !make_own_maps(batch->g[i], p, own.data(), 2 + w.m, &maps[(size_t)per * i + 2 + w.m]))
+        !make_own_maps(batch->g[i], p, own.data(), 1 + w.m, &maps[(size_t)per * i + 2 + w.m]))
       return TPFA_ECUDA;
     TmaInst& I = inst[i];
     I.g = batch->g[i];

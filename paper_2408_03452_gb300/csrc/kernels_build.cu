@@ -28,7 +28,7 @@ __device__ __forceinline__ double face_trans(double kK, double kL, const Num& a,
 
 __device__ __forceinline__ bool is_dir(const uint8_t* m, int64_t c) { return m != nullptr && m[c] != 0; }
 
-// Records of one run of z-planes of a 32 x 16 column, FP32 + FP64 (B16 = false)
+// Records of one run of z-planes of a 32 x 8 column, FP32 + FP64 (B16 = false)
 // or BF16.
 //
 // The FP64 pipe (1/64 of the FP32 rate on GB300) bounds this kernel, so it is left
@@ -61,9 +61,9 @@ build_trans_kernel(Grid g, Geo geo, const double* __restrict__ K, const uint8_t*
                    double2* __restrict__ coef64, ushort4* __restrict__ coef16, int64_t nbx,
                    int64_t nby, int zc) {
   __shared__ double sX[kBY][34];             // h/(2k) along x, columns -1 .. 32
-  __shared__ double sY[kBY + 2][32];         // h/(2k) along y, rows -1 .. 16
+  __shared__ double sY[kBY + 2][32];         // h/(2k) along y, rows -1 .. 8
   __shared__ double fX[kBY][33];             // T of the faces x-1|x, x = 0 .. 32
-  __shared__ double fY[kBY + 1][32];         // T of the faces y-1|y, y = 0 .. 16
+  __shared__ double fY[kBY + 1][32];         // T of the faces y-1|y, y = 0 .. 8
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t bx = blockIdx.x % nbx, t_ = blockIdx.x / nbx;
   const int64_t X0 = 32 * bx, Y0 = kBY * (t_ % nby), z0 = (t_ / nby) * zc;
@@ -183,7 +183,7 @@ build_trans_kernel(Grid g, Geo geo, const double* __restrict__ K, const uint8_t*
 }
 
 // The same records, one thread per cell, every face formed by both its cells: for
-// thin grids, which leave most threads of the 32 x 16 tiles idle.
+// thin grids, which leave most threads of the 32 x 8 tiles idle.
 template <bool B16>
 __global__ void __launch_bounds__(kElemThreads)
 build_trans_cell_kernel(Grid g, Geo geo, const double* __restrict__ K,

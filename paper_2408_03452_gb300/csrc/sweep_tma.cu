@@ -447,7 +447,7 @@ struct ApplyArgs {
   // instance u'q, u'r, q'w, w'q_j and u'q_j (j < DM) into
   // dots[id * kApplyDotsStride + ...], u'q also into pAp[id].  r and the q_j
   // are staged like p, own cells only, from the instance's maps own0 (r) and
-  // own0 + 2 + qmap[j]; M^-1 = 1 / D comes from the cell's record.
+  // own0 + 1 + qmap[j]; M^-1 = 1 / D comes from the cell's record.
   int own0;
   int qmap[kApplyMaxDirs];
   double* dots;
@@ -549,7 +549,7 @@ apply_tma_kernel(const __grid_constant__ ApplyArgs a) {
           tma_3d(sb + LY::kE, mown, &full[s], X0, Y0, z);                        // r
 #pragma unroll
           for (int q = 0; q < (DM > 0 ? DM : 0); ++q)
-            tma_3d(sb + LY::kE + (1 + q) * LY::kOwnBytes, mown + 2 + a.qmap[q], &full[s], X0, Y0,
+            tma_3d(sb + LY::kE + (1 + q) * LY::kOwnBytes, mown + 1 + a.qmap[q], &full[s], X0, Y0,
                    z);
         }
         issued = j + 1;

@@ -135,8 +135,8 @@ bool make_apply_maps(const Grid& g, const TmaPlan& p, const void* coef, const fl
 // (act[id] & need) == need, with u its input `which`, q = A u and w = M^-1 r:
 // u'q into uq[id] and, at dots + id * kApplyDotsStride, u'q, u'r, q'w, then
 // w'q_j and u'q_j (j < ndirs <= kApplyMaxDirs).  The instance's maps from
-// index own0 on are own-cell maps (make_own_maps) of r, M^-1 (not read: it is
-// 1 / D of the records) and the direction slots; q_j is slot qmap[j].
+// index own0 on are own-cell maps (make_own_maps) of r and the direction slots; q_j
+// is slot qmap[j].  M^-1 is 1 / D of the records.
 // partials: 3 + 2 ndirs doubles per block.  With uc (one instance only) u is
 // the value of each cell's ancestor on the 2^lev coarser grid, lev >= 1, and
 // input `which` is not read.
