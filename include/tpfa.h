@@ -91,7 +91,8 @@ enum tpfa_option {
   TPFA_OPT_TILE_VY = 4,      /* rows per warp in the stencil sweeps: 4 or 8 (default 4; 8 sets 3 stages) */
   TPFA_OPT_TILE_ZC = 5,      /* planes per warp in the stencil sweeps, 0 = automatic              */
   TPFA_OPT_CHUNK = 6,        /* CG iterations per graph launch when TPFA_OPT_LOOP = 1 (default 32) */
-  TPFA_OPT_STAGES = 7,       /* shared-memory plane stages per warp: 3 or 4 (default 4; 4 needs VY = 4) */
+  TPFA_OPT_STAGES = 7,       /* shared-memory plane stages per warp of the sweeps: 3 or 4 (default 4;
+                                4 needs VY = 4)                                                   */
   /* 8, 9, 10: retired (a CG sweep that recomputed q = A p at 40 B/cell was
      measured slower than the stored-q sweep); tpfa_set_option refuses them */
   TPFA_OPT_INNER_RTOL_BF16 = 11, /* lower bound on the inner relative tolerance of cg_solve_bf16 (1e-3) */

@@ -34,7 +34,7 @@
 //
 // us per iteration (GB300, plain CG), the sweeps in their graph loop and here:
 //   32^3 20.1 / 2.1    64^3 20.0 / 2.6    96x96x48 20.3 / 3.2
-//   128x128x64 23.3 / 5.1    128^3 28.4 / 11.0 (the kernel for taller bricks below)
+//   128x128x64 23.3 / 5.0    128^3 28.4 / 10.6 (the kernel for taller bricks below)
 // The sweeps pay a graph-node launch and a march of a few planes on a few blocks;
 // here an iteration costs one trip of words through L2 (1.5 us) and the brick's
 // stencil, 0.2 us per plane.
@@ -1212,7 +1212,7 @@ size_t sched_words(int nprob, int nblocks) {  // 8-byte words after the sums and
 // L2) and hardly with the number of blocks.  dense: batches, where an SM not taken
 // by one instance works on another, so the cost is blocks times their time; one
 // kernel per height, hence few of them.  Every grid that fits takes this path: it
-// is 2.8 times as fast as the sweeps even at the largest (160x160x96: 11.3 us per
+// is 2.9 times as fast as the sweeps even at the largest (160x160x96: 10.9 us per
 // iteration against 31.8).
 bool plan_resident(const Grid& g, int num_sms, bool dense, ResPlan* p) {
   const int64_t bx = (g.nx + 31) / 32, by = (g.ny + kRW - 1) / kRW;
